@@ -181,6 +181,13 @@ __device__ __forceinline__ void load_m_block(const WaveArgs &a, int q, float *sM
   __syncthreads();
 }
 
+// A cluster's stored info (vertex offset, triangle offset, vertex count | triangle count << 16,
+// the longest edge's squared length) as (vertex offset, triangle offset, vertices, triangles).
+__device__ __forceinline__ int4 cluster_info(int4 v, float &edge2) {
+  edge2 = __int_as_float(v.w);
+  return make_int4(v.x, v.y, v.z & 0xffff, v.z >> 16);
+}
+
 // Clusters chunk*256 + threadIdx.x of pose q: test, and append the visible ones.
 __device__ __forceinline__ void cull_block(const WaveArgs &a, int q, int chunk, float *sM) {
   load_m_block(a, q, sM);
@@ -309,6 +316,48 @@ __device__ __forceinline__ void emit_ray_warp(bool valid, const RayRec &rr, int4
   }
 }
 
+// Contract side normals of a ray-table triangle: cross products of each edge's vertices in
+// increasing global index (bit k of `order`: vertex k before its successor), the sign sigma_k of
+// the inner side, and the sign bits. False for a degenerate triangle.
+__device__ __forceinline__ bool ray_sides(const float3 v[3], int order, float3 side[3], float sg[3], int &sig) {
+  const float3 c12 = cross_c(v[1], v[2]);
+  const float det = dot_c(v[0].x, v[0].y, v[0].z, c12.x, c12.y, c12.z);
+  if (det == 0.0f || det != det) return false;
+  sig = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int m = k == 2 ? 0 : k + 1;
+    const bool lo_is_k = (order >> k) & 1;
+    side[k] = lo_is_k ? cross_c(v[k], v[m]) : cross_c(v[m], v[k]);
+    sg[k] = (det > 0.0f ? 1.0f : -1.0f) * (lo_is_k ? 1.0f : -1.0f);
+    if (sg[k] > 0.0f) sig |= 1 << k;
+  }
+  return true;
+}
+
+// The record of a triangle: side normals, signs and the inverse-depth normal.
+__device__ __forceinline__ void ray_fill(const float3 v[3], const float3 side[3], int sig, unsigned id, RayRec &rr) {
+  rr.c0x = side[0].x; rr.c0y = side[0].y; rr.c0z = side[0].z;
+  rr.c1x = side[1].x; rr.c1y = side[1].y; rr.c1z = side[1].z;
+  rr.c2x = side[2].x; rr.c2y = side[2].y; rr.c2z = side[2].z;
+  const PlaneN pl = plane_n(v[0], v[1], v[2]);
+  rr.nix = __fdiv_rn(pl.nx, pl.d);
+  rr.niy = __fdiv_rn(pl.ny, pl.d);
+  rr.niz = __fdiv_rn(pl.nz, pl.d);
+  rr.id = id;
+  rr.sig = sig;
+  rr.rect0 = rr.rect1 = 0;
+}
+
+__device__ __forceinline__ bool ray_record(const float3 v[3], int order, unsigned id, RayRec &rr) {
+  float3 side[3];
+  float sg[3];
+  int sig;
+  if (!ray_sides(v, order, side, sg, sig)) return false;
+  ray_fill(v, side, sig, id, rr);
+  return true;
+}
+
 // Ray-table triangle: contract side normals and inverse-depth normal, then a conservative
 // pixel rectangle from the layout (azimuth from the vertices' smallest enclosing arc, full
 // when a pole is inside; elevation from the vertices widened by the great-circle bulge
@@ -317,22 +366,18 @@ __device__ __forceinline__ void emit_ray_warp(bool valid, const RayRec &rr, int4
 // at the seam into at most two rectangles (i0, i1, j0, j1), which are returned with their
 // count. A triangle between pixel rays gets no rectangle; most far triangles of a panorama
 // are such, so the record's plane is computed only once a rectangle exists.
-__device__ __forceinline__ int setup_ray(const float3 v[3], const float4 u[3], const int gid[3],
-                                         unsigned id, const DevCam &cam, RayRec &rr,
-                                         int4 rect[2]) {
-  const float3 c12 = cross_c(v[1], v[2]);
-  const float det = dot_c(v[0].x, v[0].y, v[0].z, c12.x, c12.y, c12.z);
-  if (det == 0.0f || det != det) return 0;
-  float3 side[3];
+__device__ __forceinline__ int setup_ray(const float3 v[3], int order, unsigned id,
+                                         const DevCam &cam, RayRec &rr, int4 rect[2]) {
   float sg[3];
-  int sig = 0;
+  float3 side[3];
+  int sig;
+  if (!ray_sides(v, order, side, sg, sig)) return 0;
+  float4 u[3];  // unit direction (approximate: it only bounds the rectangle) and azimuth
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const int m = k == 2 ? 0 : k + 1;
-    const bool lo_is_k = gid[k] < gid[m];
-    side[k] = lo_is_k ? cross_c(v[k], v[m]) : cross_c(v[m], v[k]);
-    sg[k] = (det > 0.0f ? 1.0f : -1.0f) * (lo_is_k ? 1.0f : -1.0f);
-    if (sg[k] > 0.0f) sig |= 1 << k;
+    const float n2 = v[k].x * v[k].x + v[k].y * v[k].y + v[k].z * v[k].z;
+    const float inv = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
+    u[k] = make_float4(v[k].x * inv, v[k].y * inv, v[k].z * inv, atan2f(v[k].x, v[k].z));
   }
   // ---- conservative pixel rectangle (any rounding; margins absorb it)
   // An edge plane keeps the up (down) direction out when sg side.y exceeds 1e-4 |side| (below
@@ -405,16 +450,7 @@ __device__ __forceinline__ int setup_ray(const float3 v[3], const float4 u[3], c
       }
     }
   }
-  rr.c0x = side[0].x; rr.c0y = side[0].y; rr.c0z = side[0].z;
-  rr.c1x = side[1].x; rr.c1y = side[1].y; rr.c1z = side[1].z;
-  rr.c2x = side[2].x; rr.c2y = side[2].y; rr.c2z = side[2].z;
-  const PlaneN pl = plane_n(v[0], v[1], v[2]);
-  rr.nix = __fdiv_rn(pl.nx, pl.d);
-  rr.niy = __fdiv_rn(pl.ny, pl.d);
-  rr.niz = __fdiv_rn(pl.nz, pl.d);
-  rr.id = id;
-  rr.sig = sig;
-  rr.rect0 = rr.rect1 = 0;
+  ray_fill(v, side, sig, id, rr);
   return nrect;
 }
 
@@ -453,7 +489,8 @@ __device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker
   const float near_m = a.cam.near_m;
   constexpr bool raytable = MODEL != 0;  // one instantiation per camera model
   for (int ci = worker * 8 + warp; ci < nvis; ci += nworkers * 8) {
-    const int4 info = __ldcg(&vis[ci]);  // vert offset, tri offset, nv, nt
+    float edge2;
+    const int4 info = cluster_info(__ldcg(&vis[ci]), edge2);
     for (int k = lane; k < info.z; k += 32) {
       const float4 v = a.cl_pos[info.x + k];
       const int gv = __float_as_int(v.w);
@@ -485,16 +522,15 @@ __device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker
           const unsigned id = (unsigned)a.cl_ids[info.y + k];
           const int loc[3] = {t.x, t.y, t.z};
           float3 v[3];
-          float4 u[3];
           int gid[3];
 #pragma unroll
           for (int m = 0; m < 3; ++m) {
             const float4 p = s_vc[warp][loc[m]];
             v[m] = make_float3(p.x, p.y, p.z);
-            u[m] = s_dir[warp][loc[m]];
             gid[m] = s_gid[warp][loc[m]];
           }
-          nrect = setup_ray(v, u, gid, id, a.cam, rr, rect);
+          const int order = (gid[0] < gid[1] ? 1 : 0) | (gid[1] < gid[2] ? 2 : 0) | (gid[2] < gid[0] ? 4 : 0);
+          nrect = setup_ray(v, order, id, a.cam, rr, rect);
         }
         emit_ray_warp(nrect > 0, rr, rect[0], a, counts, bins);
         if (__any_sync(0xffffffffu, nrect > 1)) emit_ray_warp(nrect > 1, rr, rect[1], a, counts, bins);
@@ -568,6 +604,371 @@ __device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker
       if (__any_sync(0xffffffffu, vb))
         emit_piece_warp(vb, sx[0], sy[0], sx[2], sy[2], sx[3], sy[3], A, B, C, id, a, counts, bins);
     }
+    __syncwarp();
+  }
+}
+
+// ------------------------------------------------------------------ ray-table setup
+//
+// A panoramic view of a large map reaches setup with about a million triangles, nine tenths of
+// which hold no ray: they lie between two rows or columns of the table. One warp takes a cluster
+// at a time, gets the fractional (column, row) of each vertex, drops the whole cluster when no
+// row or column centre lies in its rectangle, then tests each triangle's rectangle and pushes the
+// survivors into the warp's ring in shared memory. Whenever 32 are waiting, one warp-wide step
+// computes their edge normals and planes (so that step's lanes are full, whatever share of a
+// cluster survives) and, for the ones whose rectangle holds at most kDirectRay rays, tests the
+// rays, spread evenly over the lanes, and updates the pose's z-buffer in L2 with 64-bit minima.
+// Larger ones are binned. Bound by instruction issue (0.67 of its peak): about 95 warp
+// instructions per 32 vertices and 60 per 32 triangles. 64 poses of a 1024x64 table on a
+// 2M-triangle terrain: setup 4.0 -> 1.5 ms and raster 3.7 -> 0.11 ms (every triangle used to be
+// set up, binned and read back); the call 6.1 -> 1.93 ms. Rectangles of up to 12 and up to 32 rays
+// as the line between direct and binned measured the same, and 32 leaves few records to bin.
+// Seven CTAs per SM (72 registers): eight spill (1.86 ms), six hide less latency (1.75 ms).
+
+constexpr int kRaySetupThreads = 128;
+constexpr int kRayRing = 64;    // 31 waiting + 32 pushed at most
+constexpr int kRayEntry = 5;    // 16-byte words per ring entry: 8 lanes' entries in distinct banks
+#ifndef RM_DIRECT_RAY
+#define RM_DIRECT_RAY 32
+#endif
+constexpr int kDirectRay = RM_DIRECT_RAY;  // at most 255: the fragment index decode
+constexpr float kFarColumn = 1e30f;  // column of a vertex the quick rectangle cannot hold
+constexpr float kAngleErr = 6e-6f;   // error bound of the vertices' approximate angles, radians
+constexpr float kRoundMagic = 12582912.0f;  // 1.5 2^23: x + this holds rint(x) in its low bits
+
+struct RaySetupSmem {
+  float M[12];
+  int nvis;
+  float dev[2];  // the table's largest column and row deviation from its layout, pixels
+  float4 ring[kRaySetupThreads / 32][kRayRing * kRayEntry];
+  float4 vc[kRaySetupThreads / 32][kClusterMax];  // camera-frame vertex, global index bits in w
+  float2 uv[kRaySetupThreads / 32][kClusterMax];  // packed bounds, or fractional column and row
+};
+
+// arctan t for |t| <= 1, error at most 1.8e-6: the odd polynomial of degree 11 fitted to arctan at
+// Chebyshev nodes (least squares, reweighted towards the largest error).
+__device__ __forceinline__ float atan_unit(float t) {
+  const float s = t * t;
+  float p = fmaf(s, -0.0117191346f, 0.0526473485f);
+  p = fmaf(s, p, -0.1164264827f);
+  p = fmaf(s, p, 0.1935403794f);
+  p = fmaf(s, p, -0.3326228261f);
+  return t * fmaf(s, p, 0.9999772310f);
+}
+
+// Approximate reciprocal and reciprocal square root without the subnormal handling.
+__device__ __forceinline__ float fast_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float fast_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ float warp_min_f(float x) {
+  float m;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
+__device__ __forceinline__ float warp_max_f(float x) {
+  float m;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
+
+// Largest deviation of the table's rays from their layout, in columns and rows: maxima of
+// non-negative floats as integers into dev[2] (zero before). Triangles of a far surface are smaller
+// than a pixel, so a rectangle margin of the allowed quarter pixel on each side makes most of
+// them test a ray that they cannot hold; a calibrated table is usually on its layout to
+// rounding. Not a number counts as "anywhere".
+__global__ void __launch_bounds__(256) k_ray_dev(DevCam cam, int *dev) {
+  float du = 0.0f, dv = 0.0f;
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < cam.W * cam.H; p += gridDim.x * blockDim.x) {
+    const int i = p % cam.W, j = p / cam.W;
+    const float x = cam.rays[3 * (long long)p], y = cam.rays[3 * (long long)p + 1], z = cam.rays[3 * (long long)p + 2];
+    float da = fabsf(atan2f(x, z) - (cam.az0 + cam.az_step * (i + 0.5f)));
+    da = fabsf(da - 6.28318530717958647692f * rintf(da * 0.15915494309189533577f));
+    const float de = fabsf(atan2f(-y, sqrtf(x * x + z * z)) - (cam.el0 - cam.el_step * j));
+    const float u = da / cam.az_step, v = de / cam.el_step;
+    du = u <= du ? du : (u == u ? u : INFINITY);
+    dv = v <= dv ? dv : (v == v ? v : INFINITY);
+  }
+  const int mu = __reduce_max_sync(0xffffffffu, __float_as_int(du)), mv = __reduce_max_sync(0xffffffffu, __float_as_int(dv));
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(dev, mu);
+    atomicMax(dev + 1, mv);
+  }
+}
+
+cudaError_t launch_ray_dev(const DevCam &cam, int *dev, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(dev, 0, 2 * sizeof(int), s);
+  if (e != cudaSuccess) return e;
+  const int n = cam.W * cam.H;
+  k_ray_dev<<<min((n + 255) / 256, 608), 256, 0, s>>>(cam, dev);
+  return cudaGetLastError();
+}
+
+// Rows and columns of every ray that triangles near the fractional columns [ulo, uhi] and rows
+// [vlo, vhi] can hold are those in [ulo - mu, uhi + mu] x [vlo - mv, vhi + mv]: the table's rays are
+// within dev (at most kRayMarginPx) of the layout, the angles good to kAngleErr, and a great-circle
+// edge of angular length L leaves its end points' elevation band by about |tan el| L^2 / 8 (the
+// points have |el| <= 45 degrees, and up to L^2 = 0.1 that is below 0.15 L^2). rint(x - 1/2) and
+// rint(x + 1/2) stand for floor and ceil: they differ only at integers, which another 2e-3 keeps
+// inside. `ok` fails where the bounds are too wide (near the sensor, across the seam): the caller
+// then takes the general way.
+struct QuickRect {
+  float a0, a1;      // column margin - 1/2; row margin - 1/2 without the edges' share
+  float edge, half_turn;  // 0.15 / el_step; columns of half a turn
+  unsigned last;     // last column | last row << 16
+  __device__ __forceinline__ void set(const DevCam &cam, const float *dev) {
+    a0 = dev[0] + 2e-3f + kAngleErr / cam.az_step - 0.5f;
+    a1 = dev[1] + 2e-3f + kAngleErr / cam.el_step - 0.5f;
+    edge = 0.15f / cam.el_step;
+    half_turn = 3.1f / cam.az_step;
+    last = (unsigned)(cam.W - 1) | (unsigned)(cam.H - 1) << 16;
+    // never for a margin that can cross the seam, nor for a table that neither covers one turn
+    // nor stays within (-pi, pi], where the general way places columns past the seam differently
+    const float span = cam.W * cam.az_step;
+    const bool turn = fabsf(span - 6.28318531f) < 0.05f * cam.az_step;
+    if (!(a0 < -0.05f && (turn || (cam.az0 >= -3.14160f && cam.az0 + span <= 3.14160f)))) half_turn = -1.0f;
+  }
+  // b1: the row margin - 1/2 for edges of squared angular length up to L2.
+  __device__ __forceinline__ bool ok(float L2, float ulo, float uhi, float vlo, float vhi, float &b1) const {
+    b1 = fmaf(edge, L2, a1);
+    return L2 <= 0.1f && uhi - ulo < half_turn && uhi < 3e4f && vlo > -1.4e4f && vhi < 1.6e4f && b1 < 1e2f;
+  }
+  // Last and first (column | row << 16) of a point with its margins, the last clipped to the
+  // table and the first to zero. Rounding and clipping are monotone, so a triangle's rectangle is
+  // the maximum and minimum over its vertices. The low half of x + kRoundMagic is rint(x); ok's
+  // limits keep the halves, and the differences last - first, within 16 bits.
+  __device__ __forceinline__ unsigned hi(float u, float v, float b1) const {
+    return __vmins2(__byte_perm(__float_as_uint((u + a0) + kRoundMagic), __float_as_uint((v + b1) + kRoundMagic), 0x5410),
+                    last);
+  }
+  __device__ __forceinline__ unsigned lo(float u, float v, float b1) const {
+    return __vmaxs2(__byte_perm(__float_as_uint((u - a0) + kRoundMagic), __float_as_uint((v - b1) + kRoundMagic), 0x5410),
+                    0u);
+  }
+};
+
+// Tests the rays of the warp's n small records (this lane's: cnt rays, 0 for none; its record
+// already compacted to ring slot head + rank) and updates the z-buffer. Fragment f of the
+// concatenated rectangles belongs to the last record that starts at or before f; the starts
+// inside a window of 32 fragments are collected as a bit mask, so a lane finds its record with
+// two bit counts.
+__device__ __forceinline__ void direct_rays(const DevCam &cam, const float4 *ring, int head, int cnt,
+                                            unsigned long long *zb) {
+  const int lane = threadIdx.x & 31;
+  int incl = cnt;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
+  }
+  const int start = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
+  int r0 = 0, prev = 0;  // records that start before the window; the last one's start
+  for (int base = 0; base < total; base += 32) {
+    const unsigned bit = cnt > 0 && start >= base && start < base + 32 ? 1u << (start - base) : 0u;
+    const unsigned starts = __reduce_or_sync(0xffffffffu, bit);
+    const unsigned le = starts & (0xffffffffu >> (31 - lane));
+    const int f = base + lane;
+    if (f < total) {
+      const int l = le ? lane - (31 - __clz(le)) : f - prev;
+      const float4 *e = ring + ((head + r0 + __popc(le) - 1) & (kRayRing - 1)) * kRayEntry;
+      const float4 w3 = e[3];
+      const unsigned ri = __float_as_uint(w3.z), rj = __float_as_uint(w3.w);
+      const int bw = (ri >> 16) & 0xff, dj = (int)((unsigned)l * (rj >> 15) >> 16);
+      const int p = (int)((rj & 0x7fff) + dj) * cam.W + (int)(ri & 0xffff) + l - dj * bw;
+      const float *ray = cam.rays + 3 * (long long)p;
+      const float x = __ldg(ray), y = __ldg(ray + 1), z = __ldg(ray + 2);
+      const float4 w0 = e[0], w1 = e[1], w2 = e[2];
+      const float s0 = dot_c(x, y, z, w0.x, w0.y, w0.z);
+      const float s1 = dot_c(x, y, z, w0.w, w1.x, w1.y);
+      const float s2 = dot_c(x, y, z, w1.z, w1.w, w2.x);
+      const unsigned sig = ri >> 24;
+      const bool in = ((sig & 1) ? s0 >= 0.0f : s0 < 0.0f) && ((sig & 2) ? s1 >= 0.0f : s1 < 0.0f) &&
+                      ((sig & 4) ? s2 >= 0.0f : s2 < 0.0f);
+      if (in) {
+        const float w = dot_c(w2.y, w2.z, w2.w, x, y, z);
+        if (keep_w(cam, w)) atomicMin(zb + p, make_key(w, __float_as_uint(w3.x)));
+      }
+    }
+    if (starts) {
+      prev = base + 31 - __clz(starts);
+      r0 += __popc(starts);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
+  __shared__ RaySetupSmem sm;
+  if (skipped(a)) return;
+  const int q = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float4 *vc = sm.vc[warp];
+  float2 *uv = sm.uv[warp];
+  float4 *ring = sm.ring[warp];
+  if (threadIdx.x == 0) sm.nvis = ld_cg(&a.vis_count[q]);
+  if (threadIdx.x < 2)
+    sm.dev[threadIdx.x] = a.ray_dev ? fminf(kRayMarginPx, __int_as_float(__ldg(a.ray_dev + threadIdx.x))) : kRayMarginPx;
+  load_m_block(a, q, sm.M);
+  const DevCam &cam = a.cam;
+  const int nvis = sm.nvis, stride = gridDim.x * (kRaySetupThreads / 32);
+  const int4 *vis = a.vis + (long long)q * a.n_clusters;
+  int *counts = a.counts + (long long)q * a.tg.ntiles;
+  unsigned char *bins = a.bins + (long long)q * a.tg.ntiles * a.tg.cap * a.tg.rec_bytes;
+  unsigned long long *zb = a.zbuf ? a.zbuf + (long long)q * cam.W * cam.H : nullptr;
+  const float ias = 1.0f / cam.az_step, ies = 1.0f / cam.el_step;
+  const float period = 6.28318530717958647692f * ias, iperiod = cam.az_step * 0.15915494309189533577f;
+  const float c0 = -cam.az0 * ias - 0.5f, r0 = cam.el0 * ies;
+  QuickRect quick;
+  quick.set(cam, sm.dev);
+  int head = 0, waiting = 0;
+  for (int ci = blockIdx.x * (kRaySetupThreads / 32) + warp;; ci += stride) {
+    const bool last = ci >= nvis;
+    int4 info = make_int4(0, 0, 0, 0);
+    bool packed = false;
+    float b1 = 0.0f, edge2 = 0.0f;
+    if (!last) {
+      info = cluster_info(__ldcg(&vis[ci]), edge2);
+      float M[12];
+#pragma unroll
+      for (int k = 0; k < 12; ++k) M[k] = sm.M[k];
+      float u[2], row[2], near2 = kFarColumn;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h;
+        u[h] = kFarColumn;
+        row[h] = 0.0f;
+        if (k < info.z) {
+          const float4 v = a.cl_pos[info.x + k];
+          const float3 c = xform(M, v.x, v.y, v.z);
+          vc[k] = make_float4(c.x, c.y, c.z, v.w);
+          // fractional column and row from approximate angles (they only bound rectangles)
+          const float h2 = c.x * c.x + c.z * c.z;
+          const float t = -c.y * fast_rsqrt(h2);  // tan el
+          near2 = fminf(near2, h2);
+          const float ax = fabsf(c.x), az = fabsf(c.z);
+          float b = atan_unit(fminf(ax, az) * fast_rcp(fmaxf(ax, az)));
+          b = ax > az ? 1.57079632679f - b : b;
+          b = c.z < 0.0f ? 3.14159265359f - b : b;
+          float w = fmaf(c.x < 0.0f ? -b : b, ias, c0);
+          // into [-0.5, period - 0.5), rint standing for floor as in QuickRect
+          w = fmaf(-period, (fmaf(w + 0.5f, iperiod, -0.5f) + kRoundMagic) - kRoundMagic, w);
+          if (fabsf(t) <= 1.0f && fabsf(w) < 3e4f) {  // neither steep nor on the axis
+            u[h] = w;
+            row[h] = fmaf(atan_unit(t), -ies, r0);
+          }
+        }
+      }
+      const bool two = lane + 32 < info.z;  // a lane without a second vertex repeats its first
+      if (!two) {
+        u[1] = u[0];
+        row[1] = row[0];
+      }
+      const bool one = lane < info.z;
+      const float ulo = warp_min_f(fminf(u[0], u[1])), vlo = warp_min_f(one ? fminf(row[0], row[1]) : kFarColumn);
+      const float uhi = warp_max_f(one ? fmaxf(u[0], u[1]) : -kFarColumn);
+      const float vhi = warp_max_f(one ? fmaxf(row[0], row[1]) : -kFarColumn);
+      // an edge of length e between points at least d away spans at most 2 asin(e / 2d); its
+      // square is below 1.02 (e / d)^2 while that is at most 0.1
+      packed = quick.ok(1.02f * edge2 * fast_rcp(warp_min_f(near2)), ulo, uhi, vlo, vhi, b1);
+      if (packed) {
+        if (__vsub2(quick.hi(uhi, vhi, b1), quick.lo(ulo, vlo, b1)) & 0x80008000u) info.w = 0;  // holds no ray
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const float2 q2 = make_float2(__uint_as_float(quick.hi(u[h], row[h], b1)), __uint_as_float(quick.lo(u[h], row[h], b1)));
+          if (lane + 32 * h < info.z) uv[lane + 32 * h] = q2;
+        }
+      } else {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (lane + 32 * h < info.z) uv[lane + 32 * h] = make_float2(u[h], row[h]);
+      }
+      __syncwarp();
+    }
+    for (int k0 = 0; k0 < info.w || last; k0 += 32) {
+      const int k = k0 + lane;
+      bool live = k < info.w, slow = false;
+      uchar4 t = make_uchar4(0, 0, 0, 0);
+      unsigned hi = 0, lo = 0;  // the triangle's rectangle, as QuickRect::bounds
+      if (live) {
+        t = a.cl_tris[info.y + k];
+        const float2 p0 = uv[t.x], p1 = uv[t.y], p2 = uv[t.z];
+        if (packed) {
+          hi = __vimax3_s16x2(__float_as_uint(p0.x), __float_as_uint(p1.x), __float_as_uint(p2.x));
+          lo = __vimin3_s16x2(__float_as_uint(p0.y), __float_as_uint(p1.y), __float_as_uint(p2.y));
+        } else {
+          const float ulo = fminf(p0.x, fminf(p1.x, p2.x)), uhi = fmaxf(p0.x, fmaxf(p1.x, p2.x));
+          const float vlo = fminf(p0.y, fminf(p1.y, p2.y)), vhi = fmaxf(p0.y, fmaxf(p1.y, p2.y));
+          const float da = (uhi - ulo) * cam.az_step, de = (vhi - vlo) * cam.el_step;
+          slow = !quick.ok(fmaf(da, da, de * de), ulo, uhi, vlo, vhi, b1);
+          if (!slow) {
+            hi = quick.hi(uhi, vhi, b1);
+            lo = quick.lo(ulo, vlo, b1);
+          }
+        }
+        live = slow || !(__vsub2(hi, lo) & 0x80008000u);
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, live);
+      if (live) {
+        const float4 p0 = vc[t.x], p1 = vc[t.y], p2 = vc[t.z];
+        const int g0 = __float_as_int(p0.w), g1 = __float_as_int(p1.w), g2 = __float_as_int(p2.w);
+        const int i0 = lo & 0xffff, j0 = lo >> 16, bw = (int)(hi & 0xffff) - i0 + 1, bh = (int)(hi >> 16) - j0 + 1;
+        slow = slow || !zb || bw * bh > kDirectRay;
+        const int flags = (g0 < g1 ? 1 : 0) | (g1 < g2 ? 2 : 0) | (g2 < g0 ? 4 : 0) | (slow ? 8 : 0);
+        float4 *e = ring + ((head + waiting + __popc(m & ((1u << lane) - 1u))) & (kRayRing - 1)) * kRayEntry;
+        e[0] = make_float4(p0.x, p0.y, p0.z, p1.x);
+        e[1] = make_float4(p1.y, p1.z, p2.x, p2.y);
+        e[2] = make_float4(p2.z, __int_as_float(a.cl_ids[info.y + k]), __int_as_float(flags), 0.0f);
+        e[3] = make_float4(__int_as_float(i0), __int_as_float(bw), __int_as_float(j0), __int_as_float(bh));
+      }
+      waiting += __popc(m);
+      __syncwarp();
+      while (waiting >= 32 || (last && waiting > 0)) {
+        const int n = min(waiting, 32);
+        RayRec rr;
+        int4 rect[2];
+        int nrect = 0, cnt = 0;
+        if (lane < n) {
+          const float4 *e = ring + ((head + lane) & (kRayRing - 1)) * kRayEntry;
+          const float4 e0 = e[0], e1 = e[1], e2 = e[2], e3 = e[3];
+          const float3 v[3] = {make_float3(e0.x, e0.y, e0.z), make_float3(e0.w, e1.x, e1.y),
+                               make_float3(e1.z, e1.w, e2.x)};
+          const unsigned id = __float_as_uint(e2.y);
+          const int flags = __float_as_int(e2.z);
+          if (flags & 8) {
+            nrect = setup_ray(v, flags, id, cam, rr, rect);
+          } else if (ray_record(v, flags, id, rr)) {
+            const int i0 = __float_as_int(e3.x), bw = __float_as_int(e3.y);
+            const int j0 = __float_as_int(e3.z), bh = __float_as_int(e3.w);
+            cnt = bw * bh;
+            rr.rect0 = i0 | (bw << 16) | (rr.sig << 24);
+            rr.rect1 = j0 | (((65535 + bw) / bw) << 15);  // with the multiplier of l / bw
+          }
+        }
+        __syncwarp();
+        const unsigned direct = __ballot_sync(0xffffffffu, cnt > 0);
+        if (cnt > 0) {
+          float4 *e = ring + ((head + __popc(direct & ((1u << lane) - 1u))) & (kRayRing - 1)) * kRayEntry;
+          e[0] = make_float4(rr.c0x, rr.c0y, rr.c0z, rr.c1x);
+          e[1] = make_float4(rr.c1y, rr.c1z, rr.c2x, rr.c2y);
+          e[2] = make_float4(rr.c2z, rr.nix, rr.niy, rr.niz);
+          e[3] = make_float4(__uint_as_float(rr.id), 0.0f, __int_as_float(rr.rect0), __int_as_float(rr.rect1));
+        }
+        __syncwarp();
+        if (direct) direct_rays(cam, ring, head, cnt, zb);
+        if (__any_sync(0xffffffffu, nrect > 0)) emit_ray_warp(nrect > 0, rr, rect[0], a, counts, bins);
+        if (__any_sync(0xffffffffu, nrect > 1)) emit_ray_warp(nrect > 1, rr, rect[1], a, counts, bins);
+        head = (head + n) & (kRayRing - 1);
+        waiting -= n;
+        __syncwarp();
+      }
+      if (last) break;
+    }
+    if (last) break;
     __syncwarp();
   }
 }
@@ -978,7 +1379,11 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
   const int W = a.cam.W, H = a.cam.H;
   const int xe = min(ox + TW, W) - 1, ye = min(oy + TH, H) - 1;
 
-  for (int p = tid; p < NP; p += kThreads) zk[p] = kKeyEmpty;
+  const unsigned long long *zb = a.zbuf ? a.zbuf + (long long)q * W * H : nullptr;
+  for (int p = tid; p < NP; p += kThreads) {
+    const int i = ox + p % TW, j = oy + p / TW;
+    zk[p] = zb && i <= xe && j <= ye ? __ldcg(zb + (long long)j * W + i) : kKeyEmpty;
+  }
   const long long bin = (long long)q * a.tg.ntiles + tile;
   if (tid < 12) sm.M[tid] = __ldcg(a.Ms + 12 * (long long)g + tid);
   if (tid == 0) sm.n = min(ld_cg(&a.counts[bin]), a.tg.cap);
@@ -1338,6 +1743,10 @@ static cudaError_t launch_raster(const WaveArgs &a, int mode, cudaStream_t s) {
 cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t *ev,
                         bool zero_counters) {
   cudaError_t e;
+  if (a.zbuf) {  // every byte of kKeyEmpty is 0xff
+    e = cudaMemsetAsync(a.zbuf, 0xff, sizeof(unsigned long long) * (size_t)a.cam.W * a.cam.H * a.n_poses, s);
+    if (e != cudaSuccess) return e;
+  }
   if (zero_counters) {
     e = cudaMemsetAsync(a.counts, 0, sizeof(int) * (size_t)a.tg.ntiles * a.n_poses, s);
     if (e != cudaSuccess) return e;
@@ -1360,7 +1769,7 @@ cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t
     const int blocks = min(max(a.n_clusters / 64, 1), per_pose);
     dim3 gs(blocks, a.n_poses);
     if (a.cam.model == 0) k_setup<0><<<gs, 256, 0, s>>>(a);
-    else k_setup<1><<<gs, 256, 0, s>>>(a);
+    else k_setup_ray<<<dim3(2 * blocks, a.n_poses), kRaySetupThreads, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;

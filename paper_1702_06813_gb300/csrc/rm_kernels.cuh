@@ -28,7 +28,8 @@ struct WaveArgs {
   const float *Ms;    // 12 floats per global pose (world -> camera, FP32)
   // clusters of <= 64 triangles over <= 64 vertices, built at map creation
   int n_clusters;
-  const int4 *cl_info;     // vertex offset, triangle offset, vertex count, triangle count
+  const int4 *cl_info;     // vertex offset, triangle offset, vertices | triangles << 16, and the
+                           // longest edge's squared length (FP32 bits, rounded up)
   const float4 *cl_sphere; // bounding sphere (re-centred frame)
   const float4 *cl_pos;    // per cluster vertex: position (re-centred), global index bits in w
   const uchar4 *cl_tris;   // local vertex indices per cluster triangle
@@ -37,6 +38,10 @@ struct WaveArgs {
   int *vis_count;     // wave: one counter per pose
   int *counts;        // wave: ntiles per pose
   unsigned char *bins;  // wave: ntiles * cap records of tg.rec_bytes per pose
+  // wave: one z-buffer key per pixel and pose (kKeyEmpty before setup), or null. With it, setup
+  // rasterises small triangles itself and only larger ones go through the bins.
+  unsigned long long *zbuf;
+  const int *ray_dev; // ray table: launch_ray_dev's two floats, or null (kRayMarginPx)
   double *partial;    // wave: ntiles * kNumVals per pose
   unsigned *status;   // device status word
   const int *skip;    // optional: non-zero means "skip this evaluation" (LM control)
@@ -69,6 +74,8 @@ __host__ __device__ constexpr bool is_icp(int mode) { return mode == kIcp || mod
 
 cudaError_t launch_pose_to_m(const double *poses, int n, double cx, double cy, double cz,
                              float *Ms, cudaStream_t s);
+// Largest deviation of cam's rays from their layout (two floats as ints, device memory).
+cudaError_t launch_ray_dev(const DevCam &cam, int *dev, cudaStream_t s);
 // ev (optional, 5 events): recorded before the cull kernel, then after the cull, setup,
 // raster and reduce kernels, on stream s.
 // zero_counters: clear the wave's bin counts and visible-cluster count first (callers that
