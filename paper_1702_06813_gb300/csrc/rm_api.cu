@@ -90,6 +90,9 @@ struct rm_map {
   int *d_cl_ids = nullptr;
   char *arena = nullptr;
   size_t arena_bytes = 0;
+  unsigned long long *zbuf = nullptr;  // z-buffer keys of a call's waves, see ensure_zbuf
+  size_t zbuf_keys = 0;
+  bool zbuf_empty = false;
   unsigned *d_status = nullptr;
   unsigned *h_status = nullptr;
   rm_tuning tuning{};
@@ -322,6 +325,24 @@ rm_status ensure_arena(rm_map *m, size_t bytes, cudaStream_t s) {
   return RM_OK;
 }
 
+// The z-buffers of a call's waves (`keys` of them, every one kKeyEmpty): kept between calls, because
+// the raster leaves every key it reads empty, so a call pays only for the tiles it touches.
+rm_status ensure_zbuf(rm_map *m, size_t keys, cudaStream_t s) {
+  if (keys > m->zbuf_keys) {
+    RM_CK(cudaStreamSynchronize(s));
+    if (m->zbuf) RM_CK(cudaFree(m->zbuf));
+    m->zbuf = nullptr;
+    m->zbuf_keys = 0;
+    RM_CK(cudaMalloc(&m->zbuf, sizeof(unsigned long long) * keys));
+    m->zbuf_keys = keys;
+    m->zbuf_empty = false;
+  }
+  if (!m->zbuf_empty)  // every byte of kKeyEmpty is 0xff
+    RM_CK(cudaMemsetAsync(m->zbuf, 0xff, sizeof(unsigned long long) * m->zbuf_keys, s));
+  m->zbuf_empty = true;
+  return RM_OK;
+}
+
 rm_status check_intr(const rm_intrinsics *in) {
   if (!in) return fail(RM_EINVAL, "intrinsics is NULL");
   if (in->width < 1 || in->height < 1 || in->width > 16384 || in->height > 16384)
@@ -379,12 +400,15 @@ DevCam make_cam(const rm_intrinsics *in, const float *d_rays) {
   return c;
 }
 
-int wave_size(const rm_map *m, int n, const TileGeom &tg) {
+int wave_size(const rm_map *m, int n, const TileGeom &tg, long long P) {
   if (m->tuning.wave_poses > 0) return std::min(n, m->tuning.wave_poses);
-  // up to 128 poses per wave, keeping the per-wave scratch within the map's wave budget
-  size_t per = (size_t)m->n_clusters * sizeof(int4) + (size_t)tg.ntiles * ((size_t)tg.cap * tg.rec_bytes + 8 * 40);
-  size_t w = std::max<size_t>(1, m->wave_budget / std::max<size_t>(per, 1));
-  return (int)std::min<size_t>(std::min<size_t>(w, 128), (size_t)n);
+  // up to 128 poses per wave, keeping the per-wave scratch within the map's wave budget; from 64
+  // poses on at least two waves, whose setup and raster then overlap on the two streams (64 poses
+  // at 640x480: 691 us in one wave, 621 in two; 256: 2.14 ms in two, 2.24 in four, 2.41 in 16)
+  size_t per = (size_t)m->n_clusters * sizeof(int4) + (size_t)tg.ntiles * ((size_t)tg.cap * tg.rec_bytes + 8 * 40) + 8 * (size_t)P;
+  size_t w = std::min<size_t>(128, std::max<size_t>(1, m->wave_budget / std::max<size_t>(per, 1)));
+  if (n >= 64) w = std::min<size_t>(w, ((size_t)n + 1) / 2);
+  return (int)std::min<size_t>(w, (size_t)n);
 }
 
 // Budget of the map's bounded device waits in cycles (dflt unless the tuning sets wait_log2).
@@ -522,7 +546,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
 
   for (int attempt = 0;; ++attempt) {
     TileGeom tg = make_tiles(m, in);
-    const int nw = wave_size(m, r.n, tg);
+    const int nw = wave_size(m, r.n, tg, P);
     // ---- plan the arena
     Carver plan{nullptr};
     if (host_poses) plan.take<double>(16 * (size_t)r.n);
@@ -546,13 +570,12 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
     // include the other stream's kernels)
     const int nbuf = r.n > nw && !m->prof ? 2 : 1;
     plan.take<int4>((size_t)m->n_clusters * nw * nbuf);
-    plan.take<int>((size_t)(tg.ntiles + 1) * r.n);
+    plan.take<int>((size_t)(2 * tg.ntiles + 1) * r.n);
     plan.take<unsigned char>((size_t)tg.ntiles * tg.cap * nw * tg.rec_bytes * nbuf);
     plan.take<double>((size_t)tg.ntiles * rmk::kNumVals * nw * nbuf);
-    const size_t zpx = in->model == RM_RAYTABLE ? (size_t)P * nw : 0;
-    plan.take<unsigned long long>(zpx * nbuf);
     plan.take<int>(2);
     RM_TRY(ensure_arena(m, plan.off, s));
+    RM_TRY(ensure_zbuf(m, (size_t)P * nw * nbuf, s));
     m->batch_inputs_valid = false;
     // ---- carve it
     Carver cv{m->arena};
@@ -582,11 +605,11 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
     }
     int4 *d_vis = cv.take<int4>((size_t)m->n_clusters * nw * nbuf);
     // every pose's bin counts and visible-cluster count, zeroed together once per call
-    int *d_bcount = cv.take<int>((size_t)(tg.ntiles + 1) * r.n);
-    int *d_vcount = d_bcount + (size_t)tg.ntiles * r.n;
+    int *d_bcount = cv.take<int>((size_t)(2 * tg.ntiles + 1) * r.n);
+    int *d_touched = d_bcount + (size_t)tg.ntiles * r.n;
+    int *d_vcount = d_touched + (size_t)tg.ntiles * r.n;
     unsigned char *d_bins = cv.take<unsigned char>((size_t)tg.ntiles * tg.cap * nw * tg.rec_bytes * nbuf);
     double *d_partial = cv.take<double>((size_t)tg.ntiles * rmk::kNumVals * nw * nbuf);
-    unsigned long long *d_zbuf = cv.take<unsigned long long>(zpx * nbuf);
     int *d_dev = cv.take<int>(2);
     // ---- inputs
     if (host_poses)
@@ -594,8 +617,8 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
     if (host_rays) RM_CK(cudaMemcpyAsync((void *)d_rays, in->rays, sizeof(float) * 3 * P, cudaMemcpyHostToDevice, s));
     if (host_scan) RM_CK(cudaMemcpyAsync((void *)d_sd, r.scan->depth, sizeof(float) * P, cudaMemcpyHostToDevice, s));
     if (host_cls) RM_CK(cudaMemcpyAsync((void *)d_sc, r.scan->cls, P, cudaMemcpyHostToDevice, s));
-    RM_CK(rmk::launch_pose_to_m(d_poses, r.n, m->centre[0], m->centre[1], m->centre[2], d_M, s));
-    RM_CK(cudaMemsetAsync(d_bcount, 0, sizeof(int) * (size_t)(tg.ntiles + 1) * r.n, s));
+    RM_CK(rmk::launch_begin(d_poses, r.n, m->centre[0], m->centre[1], m->centre[2], d_M, d_bcount,
+                            (long long)(2 * tg.ntiles + 1) * r.n, s));
     m->launches += 1;
     // ---- waves
     WaveArgs a{};
@@ -647,6 +670,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       RM_CK(cudaEventRecord(m->ev_fork, s));
       RM_CK(cudaStreamWaitEvent(m->aux_stream, m->ev_fork, 0));
     }
+    m->zbuf_empty = false;  // until every wave's raster is on its way
     for (int w0 = 0, k = 0; w0 < r.n; w0 += nw, ++k) {
       const int b = k % nbuf;  // buffer set and stream of this wave
       a.wave_base = w0;
@@ -656,9 +680,11 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       a.vis = d_vis + (size_t)m->n_clusters * nw * b;
       a.bins = d_bins + (size_t)tg.ntiles * tg.cap * nw * tg.rec_bytes * b;
       a.partial = d_partial + (size_t)tg.ntiles * rmk::kNumVals * nw * b;
-      a.zbuf = zpx ? d_zbuf + zpx * b : nullptr;
+      a.zbuf = m->zbuf + (size_t)P * nw * b;
+      a.touched = d_touched + (size_t)w0 * tg.ntiles;
       RM_TRY(wave(m, a, r.mode, b == 0 ? s : m->aux_stream, false));
     }
+    m->zbuf_empty = true;
     if (nbuf == 2) {
       RM_CK(cudaEventRecord(m->ev_join, m->aux_stream));
       RM_CK(cudaStreamWaitEvent(s, m->ev_join, 0));
@@ -1340,6 +1366,7 @@ void rm_map_destroy(rm_map *m) {
   cudaFree(m->d_cl_tris);
   cudaFree(m->d_cl_ids);
   cudaFree(m->arena);
+  cudaFree(m->zbuf);
   if (m->aux_stream) cudaStreamDestroy(m->aux_stream);
   if (m->ev_fork) cudaEventDestroy(m->ev_fork);
   if (m->ev_join) cudaEventDestroy(m->ev_join);

@@ -124,6 +124,21 @@ __global__ void k_pose_to_m(const double *poses, int n, double cx, double cy, do
   if (k < n) pose_to_m(poses + 16 * (long long)k, cx, cy, cz, Ms + 12 * (long long)k);
 }
 
+// Start of a call: the poses' matrices, and the counters of the bins and lists to zero.
+__global__ void __launch_bounds__(256) k_begin(const double *poses, int n, double cx, double cy, double cz,
+                                               float *Ms, int *counters, long long n_counters) {
+  const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+  for (long long k = first; k < n; k += step) pose_to_m(poses + 16 * k, cx, cy, cz, Ms + 12 * k);
+  for (long long k = first; k < n_counters; k += step) counters[k] = 0;
+}
+
+cudaError_t launch_begin(const double *poses, int n, double cx, double cy, double cz, float *Ms, int *counters,
+                         long long n_counters, cudaStream_t s) {
+  const long long work = max((long long)n, n_counters);
+  k_begin<<<(unsigned)min((work + 255) / 256, 1216ll), 256, 0, s>>>(poses, n, cx, cy, cz, Ms, counters, n_counters);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_pose_to_m(const double *poses, int n, double cx, double cy, double cz,
                              float *Ms, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
@@ -454,6 +469,45 @@ __device__ __forceinline__ int setup_ray(const float3 v[3], int order, unsigned 
   return nrect;
 }
 
+// The snapped pieces (a triangle, or a fan of two: `second`) and the inverse-depth plane of a
+// triangle (local vertices t of vc, global index bits in w) with a vertex behind the near plane or
+// beyond the guard band. False when nothing of it is drawn: all vertices behind, or in front with
+// one beyond the guard band.
+__device__ __forceinline__ bool cut_piece(const DevCam &cam, const float4 *vc, uchar4 t, int sx[4], int sy[4],
+                                          float &A, float &B, float &C, bool &second) {
+  const int loc[3] = {t.x, t.y, t.z};
+  int idx[3];
+  float3 v[3];
+  bool in[3];
+  int nin = 0;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const float4 p = vc[loc[m]];
+    v[m] = make_float3(p.x, p.y, p.z);
+    idx[m] = __float_as_int(p.w);
+    in[m] = v[m].z >= cam.near_m;
+    nin += in[m];
+  }
+  if (nin == 0 || nin == 3) return false;
+  const PlaneN pl = plane_n(v[0], v[1], v[2]);
+  fold_pinhole(cam, pl, A, B, C);
+  float3 poly[4];
+  int n = 0;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const int nx = (m + 1) % 3;
+    if (in[m]) poly[n++] = v[m];
+    if (in[m] != in[nx])
+      poly[n++] = idx[m] < idx[nx] ? near_cut(v[m], v[nx], cam.near_m) : near_cut(v[nx], v[m], cam.near_m);
+  }
+  bool ok = true;
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+    if (m < n) ok = ok && snap(cam, poly[m].x, poly[m].y, poly[m].z, sx[m], sy[m]);
+  second = ok && n == 4;
+  return ok;
+}
+
 constexpr int kClusterMax = 64;  // vertices and triangles per cluster
 
 // One warp per visible cluster: its vertices are transformed and snapped once into shared
@@ -505,7 +559,7 @@ __device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker
         int xi, yi;
         sv = snap(a.cam, c.x, c.y, c.z, xi, yi) ? make_int2(xi, yi) : make_int2(kSentinel, 2);
       }
-      s_vc[warp][k] = make_float4(c.x, c.y, c.z, 0.0f);
+      s_vc[warp][k] = make_float4(c.x, c.y, c.z, v.w);
       s_vs[warp][k] = sv;
       s_gid[warp][k] = gv;
     }
@@ -565,45 +619,301 @@ __device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker
           }
         } else {
           // slow path: near-plane cut and/or guard band
-          const int loc[3] = {t.x, t.y, t.z};
-          int idx[3];
-          float3 v[3];
-          bool in[3];
-          int nin = 0;
-#pragma unroll
-          for (int m = 0; m < 3; ++m) {
-            const float4 p = s_vc[warp][loc[m]];
-            v[m] = make_float3(p.x, p.y, p.z);
-            idx[m] = s_gid[warp][loc[m]];
-            in[m] = v[m].z >= near_m;
-            nin += in[m];
-          }
-          // all behind, or all in front with a vertex beyond the guard band: nothing drawn
-          if (nin != 0 && nin != 3) {
-            const PlaneN pl = plane_n(v[0], v[1], v[2]);
-            fold_pinhole(a.cam, pl, A, B, C);
-            float3 poly[4];
-            int n = 0;
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-              const int nx = (m + 1) % 3;
-              if (in[m]) poly[n++] = v[m];
-              if (in[m] != in[nx])
-                poly[n++] = idx[m] < idx[nx] ? near_cut(v[m], v[nx], near_m) : near_cut(v[nx], v[m], near_m);
-            }
-            bool ok = true;
-#pragma unroll
-            for (int m = 0; m < 4; ++m)
-              if (m < n) ok = ok && snap(a.cam, poly[m].x, poly[m].y, poly[m].z, sx[m], sy[m]);
-            va = ok;
-            vb = ok && n == 4;
-          }
+          va = cut_piece(a.cam, s_vc[warp], t, sx, sy, A, B, C, vb);
         }
       }
       emit_piece_warp(va, sx[0], sy[0], sx[1], sy[1], sx[2], sy[2], A, B, C, id, a, counts, bins);
       if (__any_sync(0xffffffffu, vb))
         emit_piece_warp(vb, sx[0], sy[0], sx[2], sy[2], sx[3], sy[3], A, B, C, id, a, counts, bins);
     }
+    __syncwarp();
+  }
+}
+
+// (float)i + 0.5f for 0 <= i < 2^23 without the conversion pipe: 2^23 + i is exact in the
+// mantissa, and subtracting 2^23 - 0.5 (representable) leaves i + 0.5 exactly.
+__device__ __forceinline__ float px_centre(int i) {
+  return __fsub_rn(__int_as_float(0x4B000000 | i), 8388607.5f);
+}
+
+// ------------------------------------------------------------------ direct rasterisation
+//
+// Setup kernels gather the triangles worth setting up in a ring per warp, so that the expensive
+// part of setup runs with full warps, and rasterise the small ones themselves: the pixels of 32
+// triangles' rectangles are laid out one after the other and spread evenly over the lanes.
+
+constexpr int kRing = 64;        // entries: 31 waiting + 32 pushed at most
+constexpr int kRingEntry = 5;    // 16-byte words per entry: 8 lanes' entries in distinct banks
+constexpr int kFragmentMax = 64; // largest rectangle, pixels: the index decode below
+
+// Calls f(record, index within its rectangle) for the concatenated rectangles of the warp, cnt
+// pixels in this lane's (0: none); records are numbered in lane order among the lanes with cnt > 0.
+// A fragment belongs to the last record that starts at or before it; the starts inside a window
+// of 32 fragments are collected as a bit mask, so a lane finds its record with two bit counts.
+template <class F>
+__device__ __forceinline__ void spread_fragments(int cnt, F f) {
+  const int lane = threadIdx.x & 31;
+  int incl = cnt;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
+  }
+  const int start = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
+  int r0 = 0, prev = 0;  // records that start before the window; the last one's start
+  for (int base = 0; base < total; base += 32) {
+    const unsigned bit = cnt > 0 && start >= base && start < base + 32 ? 1u << (start - base) : 0u;
+    const unsigned starts = __reduce_or_sync(0xffffffffu, bit);
+    const unsigned le = starts & (0xffffffffu >> (31 - lane));
+    const int g = base + lane;
+    if (g < total) f(r0 + __popc(le) - 1, le ? lane - (31 - __clz(le)) : g - prev);
+    if (starts) {
+      prev = base + 31 - __clz(starts);
+      r0 += __popc(starts);
+    }
+  }
+}
+
+// Marks the screen tiles that a small rectangle overlaps: the raster reads the z-buffer of marked tiles only.
+__device__ __forceinline__ void mark_tiles(const TileGeom &tg, int *touched, int i0, int i1, int j0, int j1) {
+  const int sx = 31 - __clz(tg.tw), sy = 31 - __clz(tg.th);  // tile sides are powers of two
+  const int tx0 = i0 >> sx, tx1 = i1 >> sx, ty0 = j0 >> sy, ty1 = j1 >> sy;
+  touched[ty0 * tg.ntx + tx0] = 1;
+  if (tx0 != tx1 || ty0 != ty1)
+    for (int ty = ty0; ty <= ty1; ++ty)
+      for (int tx = tx0; tx <= tx1; ++tx) touched[ty * tg.ntx + tx] = 1;
+}
+
+// m with l / n = l m >> 16 for 0 <= l < 2^8, 1 <= n <= 64: m n - 2^16 lies in (0, 2 n], and
+// l (m n - 2^16) stays below 2^16.
+__device__ __forceinline__ int index_multiplier(int n) {
+  return __float2int_rz(__fdividef(65536.0f, __int2float_rn(n)) + 1.0625f);
+}
+
+// Rectangle origin and width of a record with the multiplier of the division by the width, and
+// the pixel of index l.
+__device__ __forceinline__ int2 fragment_rect(int i0, int j0, int bw) {
+  return make_int2(i0 | (bw << 16), j0 | (index_multiplier(bw) << 15));
+}
+__device__ __forceinline__ int2 fragment_pixel(float4 w3, int l) {
+  const unsigned ri = __float_as_uint(w3.z), rj = __float_as_uint(w3.w);
+  const int dj = (int)((unsigned)l * (rj >> 15) >> 16);
+  return make_int2((int)(ri & 0xffff) + l - dj * (int)(ri >> 16), (int)(rj & 0x7fff) + dj);
+}
+
+// ------------------------------------------------------------------ pinhole setup
+//
+// One warp takes a cluster at a time: its vertices are transformed and snapped into shared memory;
+// triangles whose snapped box holds a sample go into the warp's ring; and for every 32 of them one
+// warp-wide step computes the inverse-depth planes and rasterises the ones whose box holds at most
+// kDirectPinhole samples into the pose's z-buffer in L2. Larger ones go to the screen-tile bins, as
+// do the pieces of triangles cut at the near plane. In a mapped room most triangles in view cover a
+// few pixels, and a view crowded with them used to pile tens of thousands of records into one
+// tile's bin, which one CTA worked off. Bound by instruction issue (0.7 of its peak; two IEEE
+// divisions a vertex, five a triangle). 256 poses of 640x480 on 1M triangles, two views: 3.17 ->
+// 2.14 and 4.58 -> 2.95 ms a call (raster 2.3 -> 0.57 ms, setup 1.06 -> 1.70); the benchmark's
+// view, whose triangles are large, is unchanged at 1.18. The line at 48 samples: 24 costs 5 to 9%,
+// 12 16 to 25%, and above 48 the rectangles' empty samples cost what the bins would.
+
+constexpr int kPinSetupThreads = 128;
+#ifndef RM_DIRECT_PINHOLE
+#define RM_DIRECT_PINHOLE 48
+#endif
+constexpr int kDirectPinhole = RM_DIRECT_PINHOLE;
+static_assert(kDirectPinhole <= kFragmentMax, "fragment index decode");
+// Direct triangles extend over at most 64 pixels (2^14 units): their edge functions fit int32, and
+// those divided by 256 are integers below 2^24, exact in FP32.
+constexpr int kDirectExtent = 1 << 14;
+
+struct PinSetupSmem {
+  float M[12];
+  int nvis;
+  float4 ring[kPinSetupThreads / 32][kRing * kRingEntry];
+  float4 vc[kPinSetupThreads / 32][kClusterMax];  // camera-frame vertex, global index bits in w
+  int2 vs[kPinSetupThreads / 32][kClusterMax];    // snapped, or kSentinel
+};
+
+// The warp's small triangles (this lane's: cnt row segments, 0 for none) into the z-buffer. A unit
+// of work is up to kSegment samples of one row: the walk along it costs three additions and one
+// fused multiply-add a sample, and finding the record is paid once for all of them.
+constexpr int kSegment = 8;
+__device__ __forceinline__ void direct_pixels(const DevCam &cam, const float4 *ring, int head, int cnt,
+                                              unsigned long long *zb) {
+  const float w_lo = fmaxf(cam.w_far, __int_as_float(1)), w_hi = cam.w_near;  // as raster_tile
+  spread_fragments(cnt, [&](int r, int l) {
+    const float4 *e = ring + ((head + r) & (kRing - 1)) * kRingEntry;
+    const float4 w0 = e[0], w1 = e[1], w2 = e[2], w3 = e[3];
+    const unsigned ri = __float_as_uint(w3.z), rj = __float_as_uint(w3.w), sg = __float_as_uint(w3.y);
+    const int row = (int)((unsigned)l * (rj >> 15) >> 16), x0 = (l - row * (int)sg) * kSegment;
+    const int i = (int)(ri & 0xffff) + x0, j = (int)(rj & 0x7fff) + row;
+    const float di = __int2float_rn(x0), dj = __int2float_rn(row);
+    float e0 = fmaf(di, w0.y, fmaf(dj, w0.z, w0.x)), e1 = fmaf(di, w1.x, fmaf(dj, w1.y, w0.w));
+    float e2 = fmaf(di, w1.w, fmaf(dj, w2.x, w1.z));
+    float fi = px_centre(i);
+    const float base = __fmaf_rn(w2.z, px_centre(j), w2.w);
+    unsigned long long *z = zb + j * cam.W + i;
+    const unsigned id = __float_as_uint(w3.x);
+    for (int n = min(kSegment, (int)(ri >> 16) - x0); n > 0; --n) {
+      const float w = __fmaf_rn(w2.y, fi, base);
+      if (fminf(e0, fminf(e1, e2)) >= 0.0f && w >= w_lo && w <= w_hi) atomicMin(z, make_key(w, id));
+      e0 += w0.y;
+      e1 += w1.x;
+      e2 += w1.w;
+      fi = __fadd_rn(fi, 1.0f);
+      ++z;
+    }
+  });
+}
+
+__global__ void __launch_bounds__(kPinSetupThreads, 7) k_setup_pin(WaveArgs a) {
+  __shared__ PinSetupSmem sm;
+  if (skipped(a)) return;
+  const int q = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float4 *vc = sm.vc[warp];
+  int2 *vs = sm.vs[warp];
+  float4 *ring = sm.ring[warp];
+  if (threadIdx.x == 0) sm.nvis = ld_cg(&a.vis_count[q]);
+  load_m_block(a, q, sm.M);
+  const DevCam &cam = a.cam;
+  const int W = cam.W, H = cam.H;
+  const int nvis = sm.nvis, stride = gridDim.x * (kPinSetupThreads / 32);
+  const int4 *vis = a.vis + (long long)q * a.n_clusters;
+  int *counts = a.counts + (long long)q * a.tg.ntiles;
+  unsigned char *bins = a.bins + (long long)q * a.tg.ntiles * a.tg.cap * a.tg.rec_bytes;
+  unsigned long long *zb = a.zbuf ? a.zbuf + (long long)q * W * H : nullptr;
+  int *touched = a.touched + (long long)q * a.tg.ntiles;
+  int head = 0, waiting = 0;
+  for (int ci = blockIdx.x * (kPinSetupThreads / 32) + warp;; ci += stride) {
+    const bool last = ci >= nvis;
+    int4 info = make_int4(0, 0, 0, 0);
+    if (!last) {
+      float edge2;
+      info = cluster_info(__ldcg(&vis[ci]), edge2);
+      float M[12];
+#pragma unroll
+      for (int k = 0; k < 12; ++k) M[k] = sm.M[k];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int k = lane + 32 * h;
+        if (k < info.z) {
+          const float4 v = a.cl_pos[info.x + k];
+          const float3 c = xform(M, v.x, v.y, v.z);
+          int2 sv = make_int2(kSentinel, 1);  // behind the near plane
+          if (c.z >= cam.near_m) {
+            int xi, yi;
+            sv = snap(cam, c.x, c.y, c.z, xi, yi) ? make_int2(xi, yi) : make_int2(kSentinel, 2);
+          }
+          vc[k] = make_float4(c.x, c.y, c.z, v.w);
+          vs[k] = sv;
+        }
+      }
+      __syncwarp();
+    }
+    for (int k0 = 0; k0 < info.w || last; k0 += 32) {
+      const int k = k0 + lane;
+      bool live = k < info.w, cut = false;
+      uchar4 t = make_uchar4(0, 0, 0, 0);
+      int2 s0 = make_int2(0, 0), s1 = s0, s2 = s0;
+      if (live) {
+        t = a.cl_tris[info.y + k];
+        s0 = vs[t.x];
+        s1 = vs[t.y];
+        s2 = vs[t.z];
+        cut = s0.x == kSentinel || s1.x == kSentinel || s2.x == kSentinel;
+        const int xmin = min(s0.x, min(s1.x, s2.x)), xmax = max(s0.x, max(s1.x, s2.x));
+        const int ymin = min(s0.y, min(s1.y, s2.y)), ymax = max(s0.y, max(s1.y, s2.y));
+        live = !cut && max((xmin + 127) >> 8, 0) <= min((xmax - 128) >> 8, W - 1) &&
+               max((ymin + 127) >> 8, 0) <= min((ymax - 128) >> 8, H - 1);
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, live);
+      if (live) {
+        const float4 p0 = vc[t.x], p1 = vc[t.y], p2 = vc[t.z];
+        float4 *e = ring + ((head + waiting + __popc(m & ((1u << lane) - 1u))) & (kRing - 1)) * kRingEntry;
+        e[0] = make_float4(p0.x, p0.y, p0.z, p1.x);
+        e[1] = make_float4(p1.y, p1.z, p2.x, p2.y);
+        e[2] = make_float4(p2.z, __int_as_float(s0.x), __int_as_float(s0.y), __int_as_float(s1.x));
+        e[3] = make_float4(__int_as_float(s1.y), __int_as_float(s2.x), __int_as_float(s2.y),
+                           __int_as_float(a.cl_ids[info.y + k]));
+      }
+      waiting += __popc(m);
+      __syncwarp();
+      while (waiting >= 32 || (last && waiting > 0)) {
+        const int n = min(waiting, 32);
+        int x0 = 0, y0 = 0, x1 = 0, y1 = 0, x2 = 0, y2 = 0, cnt = 0;
+        float A = 0.0f, B = 0.0f, C = 0.0f;
+        unsigned id = 0;
+        bool big = false;
+        int4 er = make_int4(0, 0, 0, 0), ex = er, ey = er;  // direct: edge values and steps
+        int2 rect = make_int2(0, 0);
+        int seg = 0;
+        if (lane < n) {
+          const float4 *e = ring + ((head + lane) & (kRing - 1)) * kRingEntry;
+          const float4 e0 = e[0], e1 = e[1], e2 = e[2], e3 = e[3];
+          const PlaneN pl = plane_n(make_float3(e0.x, e0.y, e0.z), make_float3(e0.w, e1.x, e1.y),
+                                    make_float3(e1.z, e1.w, e2.x));
+          fold_pinhole(cam, pl, A, B, C);
+          x0 = __float_as_int(e2.y); y0 = __float_as_int(e2.z);
+          x1 = __float_as_int(e2.w); y1 = __float_as_int(e3.x);
+          x2 = __float_as_int(e3.y); y2 = __float_as_int(e3.z);
+          id = __float_as_uint(e3.w);
+          const int xmin = min(x0, min(x1, x2)), xmax = max(x0, max(x1, x2));
+          const int ymin = min(y0, min(y1, y2)), ymax = max(y0, max(y1, y2));
+          const int i0 = max((xmin + 127) >> 8, 0), i1 = min((xmax - 128) >> 8, W - 1);
+          const int j0 = max((ymin + 127) >> 8, 0), j1 = min((ymax - 128) >> 8, H - 1);
+          const int bw = i1 - i0 + 1, bh = j1 - j0 + 1;
+          // the extents first: boxes of at most 64 pixels cannot overflow the product
+          big = !zb || xmax - xmin > kDirectExtent || ymax - ymin > kDirectExtent || bw * bh > kDirectPinhole;
+          if (!big) {
+            const int area = (x1 - x0) * (y2 - y0) - (y1 - y0) * (x2 - x0);
+            const bool flip = area < 0;
+            const int bx = flip ? x2 : x1, by = flip ? y2 : y1, cx = flip ? x1 : x2, cy = flip ? y1 : y2;
+            const int px = 256 * i0 + 128, py = 256 * j0 + 128;
+            const int dx0 = bx - x0, dy0 = by - y0, dx1 = cx - bx, dy1 = cy - by, dx2 = x0 - cx, dy2 = y0 - cy;
+            const bool tl0 = dy0 < 0 || (dy0 == 0 && dx0 > 0), tl1 = dy1 < 0 || (dy1 == 0 && dx1 > 0);
+            const bool tl2 = dy2 < 0 || (dy2 == 0 && dx2 > 0);
+            er = make_int4((dx0 * (py - y0) - dy0 * (px - x0) - (tl0 ? 0 : 1)) >> 8,
+                           (dx1 * (py - by) - dy1 * (px - bx) - (tl1 ? 0 : 1)) >> 8,
+                           (dx2 * (py - cy) - dy2 * (px - cx) - (tl2 ? 0 : 1)) >> 8, 0);
+            ex = make_int4(-dy0, -dy1, -dy2, 0);
+            ey = make_int4(dx0, dx1, dx2, 0);
+            const int ns = (bw + kSegment - 1) / kSegment;
+            seg = ns;
+            rect = make_int2(i0 | (bw << 16), j0 | (index_multiplier(ns) << 15));
+            cnt = area != 0 ? ns * bh : 0;
+            mark_tiles(a.tg, touched, i0, i1, j0, j1);
+          }
+        }
+        __syncwarp();
+        const unsigned direct = __ballot_sync(0xffffffffu, cnt > 0);
+        if (cnt > 0) {
+          float4 *e = ring + ((head + __popc(direct & ((1u << lane) - 1u))) & (kRing - 1)) * kRingEntry;
+          e[0] = make_float4(__int2float_rn(er.x), __int2float_rn(ex.x), __int2float_rn(ey.x), __int2float_rn(er.y));
+          e[1] = make_float4(__int2float_rn(ex.y), __int2float_rn(ey.y), __int2float_rn(er.z), __int2float_rn(ex.z));
+          e[2] = make_float4(__int2float_rn(ey.z), A, B, C);
+          e[3] = make_float4(__uint_as_float(id), __int_as_float(seg), __int_as_float(rect.x), __int_as_float(rect.y));
+        }
+        __syncwarp();
+        if (direct) direct_pixels(cam, ring, head, cnt, zb);
+        if (__any_sync(0xffffffffu, big)) emit_piece_warp(big, x0, y0, x1, y1, x2, y2, A, B, C, id, a, counts, bins);
+        head = (head + n) & (kRing - 1);
+        waiting -= n;
+        __syncwarp();
+      }
+      if (last) break;
+      if (__any_sync(0xffffffffu, cut)) {
+        // near-plane cut and/or guard band
+        bool va = false, vb = false;
+        int sx[4] = {0, 0, 0, 0}, sy[4] = {0, 0, 0, 0};
+        float A = 0.0f, B = 0.0f, C = 0.0f;
+        unsigned id = 0;
+        if (cut) va = cut_piece(cam, vc, t, sx, sy, A, B, C, vb);
+        if (va) id = (unsigned)a.cl_ids[info.y + k];
+        emit_piece_warp(va, sx[0], sy[0], sx[1], sy[1], sx[2], sy[2], A, B, C, id, a, counts, bins);
+        if (__any_sync(0xffffffffu, vb))
+          emit_piece_warp(vb, sx[0], sy[0], sx[2], sy[2], sx[3], sy[3], A, B, C, id, a, counts, bins);
+      }
+    }
+    if (last) break;
     __syncwarp();
   }
 }
@@ -626,12 +936,11 @@ __device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker
 // Seven CTAs per SM (72 registers): eight spill (1.86 ms), six hide less latency (1.75 ms).
 
 constexpr int kRaySetupThreads = 128;
-constexpr int kRayRing = 64;    // 31 waiting + 32 pushed at most
-constexpr int kRayEntry = 5;    // 16-byte words per ring entry: 8 lanes' entries in distinct banks
 #ifndef RM_DIRECT_RAY
 #define RM_DIRECT_RAY 32
 #endif
-constexpr int kDirectRay = RM_DIRECT_RAY;  // at most 255: the fragment index decode
+constexpr int kDirectRay = RM_DIRECT_RAY;
+static_assert(kDirectRay <= kFragmentMax, "fragment index decode");
 constexpr float kFarColumn = 1e30f;  // column of a vertex the quick rectangle cannot hold
 constexpr float kAngleErr = 6e-6f;   // error bound of the vertices' approximate angles, radians
 constexpr float kRoundMagic = 12582912.0f;  // 1.5 2^23: x + this holds rint(x) in its low bits
@@ -640,7 +949,7 @@ struct RaySetupSmem {
   float M[12];
   int nvis;
   float dev[2];  // the table's largest column and row deviation from its layout, pixels
-  float4 ring[kRaySetupThreads / 32][kRayRing * kRayEntry];
+  float4 ring[kRaySetupThreads / 32][kRing * kRingEntry];
   float4 vc[kRaySetupThreads / 32][kClusterMax];  // camera-frame vertex, global index bits in w
   float2 uv[kRaySetupThreads / 32][kClusterMax];  // packed bounds, or fractional column and row
 };
@@ -754,53 +1063,29 @@ struct QuickRect {
   }
 };
 
-// Tests the rays of the warp's n small records (this lane's: cnt rays, 0 for none; its record
-// already compacted to ring slot head + rank) and updates the z-buffer. Fragment f of the
-// concatenated rectangles belongs to the last record that starts at or before f; the starts
-// inside a window of 32 fragments are collected as a bit mask, so a lane finds its record with
-// two bit counts.
+// Tests the rays of the warp's small records (this lane's: cnt rays, 0 for none; its record already
+// compacted to ring slot head + rank) and updates the z-buffer.
 __device__ __forceinline__ void direct_rays(const DevCam &cam, const float4 *ring, int head, int cnt,
                                             unsigned long long *zb) {
-  const int lane = threadIdx.x & 31;
-  int incl = cnt;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, incl, off);
-    if (lane >= off) incl += v;
-  }
-  const int start = incl - cnt, total = __shfl_sync(0xffffffffu, incl, 31);
-  int r0 = 0, prev = 0;  // records that start before the window; the last one's start
-  for (int base = 0; base < total; base += 32) {
-    const unsigned bit = cnt > 0 && start >= base && start < base + 32 ? 1u << (start - base) : 0u;
-    const unsigned starts = __reduce_or_sync(0xffffffffu, bit);
-    const unsigned le = starts & (0xffffffffu >> (31 - lane));
-    const int f = base + lane;
-    if (f < total) {
-      const int l = le ? lane - (31 - __clz(le)) : f - prev;
-      const float4 *e = ring + ((head + r0 + __popc(le) - 1) & (kRayRing - 1)) * kRayEntry;
-      const float4 w3 = e[3];
-      const unsigned ri = __float_as_uint(w3.z), rj = __float_as_uint(w3.w);
-      const int bw = (ri >> 16) & 0xff, dj = (int)((unsigned)l * (rj >> 15) >> 16);
-      const int p = (int)((rj & 0x7fff) + dj) * cam.W + (int)(ri & 0xffff) + l - dj * bw;
-      const float *ray = cam.rays + 3 * (long long)p;
-      const float x = __ldg(ray), y = __ldg(ray + 1), z = __ldg(ray + 2);
-      const float4 w0 = e[0], w1 = e[1], w2 = e[2];
-      const float s0 = dot_c(x, y, z, w0.x, w0.y, w0.z);
-      const float s1 = dot_c(x, y, z, w0.w, w1.x, w1.y);
-      const float s2 = dot_c(x, y, z, w1.z, w1.w, w2.x);
-      const unsigned sig = ri >> 24;
-      const bool in = ((sig & 1) ? s0 >= 0.0f : s0 < 0.0f) && ((sig & 2) ? s1 >= 0.0f : s1 < 0.0f) &&
-                      ((sig & 4) ? s2 >= 0.0f : s2 < 0.0f);
-      if (in) {
-        const float w = dot_c(w2.y, w2.z, w2.w, x, y, z);
-        if (keep_w(cam, w)) atomicMin(zb + p, make_key(w, __float_as_uint(w3.x)));
-      }
+  spread_fragments(cnt, [&](int r, int l) {
+    const float4 *e = ring + ((head + r) & (kRing - 1)) * kRingEntry;
+    const float4 w3 = e[3];
+    const int2 ij = fragment_pixel(w3, l);
+    const int p = ij.y * cam.W + ij.x;
+    const float *ray = cam.rays + 3 * (long long)p;
+    const float x = __ldg(ray), y = __ldg(ray + 1), z = __ldg(ray + 2);
+    const float4 w0 = e[0], w1 = e[1], w2 = e[2];
+    const float s0 = dot_c(x, y, z, w0.x, w0.y, w0.z);
+    const float s1 = dot_c(x, y, z, w0.w, w1.x, w1.y);
+    const float s2 = dot_c(x, y, z, w1.z, w1.w, w2.x);
+    const unsigned sig = __float_as_uint(w3.y);
+    const bool in = ((sig & 1) ? s0 >= 0.0f : s0 < 0.0f) && ((sig & 2) ? s1 >= 0.0f : s1 < 0.0f) &&
+                    ((sig & 4) ? s2 >= 0.0f : s2 < 0.0f);
+    if (in) {
+      const float w = dot_c(w2.y, w2.z, w2.w, x, y, z);
+      if (keep_w(cam, w)) atomicMin(zb + p, make_key(w, __float_as_uint(w3.x)));
     }
-    if (starts) {
-      prev = base + 31 - __clz(starts);
-      r0 += __popc(starts);
-    }
-  }
+  });
 }
 
 __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
@@ -825,6 +1110,7 @@ __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
   const float c0 = -cam.az0 * ias - 0.5f, r0 = cam.el0 * ies;
   QuickRect quick;
   quick.set(cam, sm.dev);
+  int *touched = a.touched + (long long)q * a.tg.ntiles;
   int head = 0, waiting = 0;
   for (int ci = blockIdx.x * (kRaySetupThreads / 32) + warp;; ci += stride) {
     const bool last = ci >= nvis;
@@ -919,7 +1205,7 @@ __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
         const int i0 = lo & 0xffff, j0 = lo >> 16, bw = (int)(hi & 0xffff) - i0 + 1, bh = (int)(hi >> 16) - j0 + 1;
         slow = slow || !zb || bw * bh > kDirectRay;
         const int flags = (g0 < g1 ? 1 : 0) | (g1 < g2 ? 2 : 0) | (g2 < g0 ? 4 : 0) | (slow ? 8 : 0);
-        float4 *e = ring + ((head + waiting + __popc(m & ((1u << lane) - 1u))) & (kRayRing - 1)) * kRayEntry;
+        float4 *e = ring + ((head + waiting + __popc(m & ((1u << lane) - 1u))) & (kRing - 1)) * kRingEntry;
         e[0] = make_float4(p0.x, p0.y, p0.z, p1.x);
         e[1] = make_float4(p1.y, p1.z, p2.x, p2.y);
         e[2] = make_float4(p2.z, __int_as_float(a.cl_ids[info.y + k]), __int_as_float(flags), 0.0f);
@@ -933,7 +1219,7 @@ __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
         int4 rect[2];
         int nrect = 0, cnt = 0;
         if (lane < n) {
-          const float4 *e = ring + ((head + lane) & (kRayRing - 1)) * kRayEntry;
+          const float4 *e = ring + ((head + lane) & (kRing - 1)) * kRingEntry;
           const float4 e0 = e[0], e1 = e[1], e2 = e[2], e3 = e[3];
           const float3 v[3] = {make_float3(e0.x, e0.y, e0.z), make_float3(e0.w, e1.x, e1.y),
                                make_float3(e1.z, e1.w, e2.x)};
@@ -945,24 +1231,27 @@ __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
             const int i0 = __float_as_int(e3.x), bw = __float_as_int(e3.y);
             const int j0 = __float_as_int(e3.z), bh = __float_as_int(e3.w);
             cnt = bw * bh;
-            rr.rect0 = i0 | (bw << 16) | (rr.sig << 24);
-            rr.rect1 = j0 | (((65535 + bw) / bw) << 15);  // with the multiplier of l / bw
+            const int2 rect = fragment_rect(i0, j0, bw);
+            mark_tiles(a.tg, touched, i0, i0 + bw - 1, j0, j0 + bh - 1);
+            rr.rect0 = rect.x;
+            rr.rect1 = rect.y;
           }
         }
         __syncwarp();
         const unsigned direct = __ballot_sync(0xffffffffu, cnt > 0);
         if (cnt > 0) {
-          float4 *e = ring + ((head + __popc(direct & ((1u << lane) - 1u))) & (kRayRing - 1)) * kRayEntry;
+          float4 *e = ring + ((head + __popc(direct & ((1u << lane) - 1u))) & (kRing - 1)) * kRingEntry;
           e[0] = make_float4(rr.c0x, rr.c0y, rr.c0z, rr.c1x);
           e[1] = make_float4(rr.c1y, rr.c1z, rr.c2x, rr.c2y);
           e[2] = make_float4(rr.c2z, rr.nix, rr.niy, rr.niz);
-          e[3] = make_float4(__uint_as_float(rr.id), 0.0f, __int_as_float(rr.rect0), __int_as_float(rr.rect1));
+          e[3] = make_float4(__uint_as_float(rr.id), __int_as_float(rr.sig), __int_as_float(rr.rect0),
+                             __int_as_float(rr.rect1));
         }
         __syncwarp();
         if (direct) direct_rays(cam, ring, head, cnt, zb);
         if (__any_sync(0xffffffffu, nrect > 0)) emit_ray_warp(nrect > 0, rr, rect[0], a, counts, bins);
         if (__any_sync(0xffffffffu, nrect > 1)) emit_ray_warp(nrect > 1, rr, rect[1], a, counts, bins);
-        head = (head + n) & (kRayRing - 1);
+        head = (head + n) & (kRing - 1);
         waiting -= n;
         __syncwarp();
       }
@@ -971,16 +1260,6 @@ __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
     if (last) break;
     __syncwarp();
   }
-}
-
-// pinhole: six resident CTAs per SM (40 registers): setup is bound by the latency of its
-// dependent loads, so more resident warps pay more than registers; the ray-table setup keeps
-// a record and two rectangles per lane across its appends and gets 64 registers
-template <int MODEL>
-__global__ void __launch_bounds__(256, MODEL == 0 ? 6 : 4) k_setup(WaveArgs a) {
-  __shared__ SetupSmem sm;
-  if (skipped(a)) return;
-  setup_block<MODEL>(a, blockIdx.y, blockIdx.x, gridDim.x, sm);
 }
 
 // ------------------------------------------------------------------ raster + epilogue
@@ -1065,13 +1344,6 @@ __device__ __forceinline__ bool covers_exact(const TriRec &q, int i, int j) {
 __device__ __forceinline__ bool inner3(int a, int b, int c) { return (a | b | c) >= 0; }
 
 __device__ __forceinline__ int wadd(int a, int b) { return (int)((unsigned)a + (unsigned)b); }
-
-// (float)i + 0.5f for 0 <= i < 2^23 without the conversion pipe: 2^23 + i is exact in the
-// mantissa, and subtracting 2^23 - 0.5 (representable) leaves i + 0.5 exactly.
-__device__ __forceinline__ float px_centre(int i) {
-  return __fsub_rn(__int_as_float(0x4B000000 | i), 8388607.5f);
-}
-
 
 // Rasterise every record of one (pose, tile) bin into the shared z-buffer. Records are staged
 // with one bulk copy per round; a block-wide scan of their per-tile rectangle sizes lays all
@@ -1379,12 +1651,27 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
   const int W = a.cam.W, H = a.cam.H;
   const int xe = min(ox + TW, W) - 1, ye = min(oy + TH, H) - 1;
 
-  const unsigned long long *zb = a.zbuf ? a.zbuf + (long long)q * W * H : nullptr;
-  for (int p = tid; p < NP; p += kThreads) {
-    const int i = ox + p % TW, j = oy + p / TW;
-    zk[p] = zb && i <= xe && j <= ye ? __ldcg(zb + (long long)j * W + i) : kKeyEmpty;
-  }
   const long long bin = (long long)q * a.tg.ntiles + tile;
+  if (a.zbuf && __ldcg(a.touched + bin) != 0) {
+    // setup rasterised small triangles into this tile: start from their keys, and leave the
+    // z-buffer empty for the next wave or call
+    unsigned long long *zb = a.zbuf + (long long)q * W * H;
+    constexpr int kPer = NP / kThreads;
+    unsigned long long key[kPer];  // every load in flight before the first store
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) {
+      const int p = tid + m * kThreads, i = ox + p % TW, j = oy + p / TW;
+      key[m] = i <= xe && j <= ye ? __ldcg(zb + j * W + i) : kKeyEmpty;
+    }
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) {
+      const int p = tid + m * kThreads, i = ox + p % TW, j = oy + p / TW;
+      zk[p] = key[m];
+      if (key[m] != kKeyEmpty) __stcg(zb + j * W + i, kKeyEmpty);
+    }
+  } else {
+    for (int p = tid; p < NP; p += kThreads) zk[p] = kKeyEmpty;
+  }
   if (tid < 12) sm.M[tid] = __ldcg(a.Ms + 12 * (long long)g + tid);
   if (tid == 0) sm.n = min(ld_cg(&a.counts[bin]), a.tg.cap);
   float *rx = nullptr, *ry = nullptr, *rz = nullptr;
@@ -1743,10 +2030,6 @@ static cudaError_t launch_raster(const WaveArgs &a, int mode, cudaStream_t s) {
 cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t *ev,
                         bool zero_counters) {
   cudaError_t e;
-  if (a.zbuf) {  // every byte of kKeyEmpty is 0xff
-    e = cudaMemsetAsync(a.zbuf, 0xff, sizeof(unsigned long long) * (size_t)a.cam.W * a.cam.H * a.n_poses, s);
-    if (e != cudaSuccess) return e;
-  }
   if (zero_counters) {
     e = cudaMemsetAsync(a.counts, 0, sizeof(int) * (size_t)a.tg.ntiles * a.n_poses, s);
     if (e != cudaSuccess) return e;
@@ -1768,7 +2051,7 @@ cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t
     const int per_pose = max(16, (kSetupCtasPerGpu + a.n_poses - 1) / a.n_poses);
     const int blocks = min(max(a.n_clusters / 64, 1), per_pose);
     dim3 gs(blocks, a.n_poses);
-    if (a.cam.model == 0) k_setup<0><<<gs, 256, 0, s>>>(a);
+    if (a.cam.model == 0) k_setup_pin<<<dim3(2 * blocks, a.n_poses), kPinSetupThreads, 0, s>>>(a);
     else k_setup_ray<<<dim3(2 * blocks, a.n_poses), kRaySetupThreads, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -38,9 +38,11 @@ struct WaveArgs {
   int *vis_count;     // wave: one counter per pose
   int *counts;        // wave: ntiles per pose
   unsigned char *bins;  // wave: ntiles * cap records of tg.rec_bytes per pose
-  // wave: one z-buffer key per pixel and pose (kKeyEmpty before setup), or null. With it, setup
-  // rasterises small triangles itself and only larger ones go through the bins.
+  // wave: one z-buffer key per pixel and pose, or null. With it, setup rasterises small triangles
+  // itself and only larger ones go through the bins. Every key is kKeyEmpty before setup; the
+  // raster empties the tiles that setup marked again.
   unsigned long long *zbuf;
+  int *touched;       // wave: ntiles per pose, zero before setup (with zbuf)
   const int *ray_dev; // ray table: launch_ray_dev's two floats, or null (kRayMarginPx)
   double *partial;    // wave: ntiles * kNumVals per pose
   unsigned *status;   // device status word
@@ -74,6 +76,9 @@ __host__ __device__ constexpr bool is_icp(int mode) { return mode == kIcp || mod
 
 cudaError_t launch_pose_to_m(const double *poses, int n, double cx, double cy, double cz,
                              float *Ms, cudaStream_t s);
+// Start of a call: n matrices as launch_pose_to_m and n_counters ints to zero, in one launch.
+cudaError_t launch_begin(const double *poses, int n, double cx, double cy, double cz, float *Ms, int *counters,
+                         long long n_counters, cudaStream_t s);
 // Largest deviation of cam's rays from their layout (two floats as ints, device memory).
 cudaError_t launch_ray_dev(const DevCam &cam, int *dev, cudaStream_t s);
 // ev (optional, 5 events): recorded before the cull kernel, then after the cull, setup,
