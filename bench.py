@@ -343,14 +343,14 @@ def run_tracking(a):
         plain_ms += (time.perf_counter() - t0) * 1e3
     plain_value = n_agents * n_plain / (plain_ms * 1e-3)
     errs = np.array(errs)
-    # roofline of the one kernel of a frame (the persistent batch kernel): algorithmic bytes per
-    # launch = the map once plus the scan comparison of every evaluation of every agent
+    # roofline of a frame's one batch call: algorithmic bytes per
+    # call = the map once plus the scan comparison of every evaluation of every agent
     pk, pk_kind = peaks()
     p_img = [c.width * c.height for c in cams]
     evals_per_agent = 1 + 5 if a.method == "lm" else 5
     launch_bytes = 12 * mesh.n_verts + 13 * mesh.n_tris + sum(5 * p_img[k] * evals_per_agent for k in kinds)
     achieved = launch_bytes / (total_ms / a.frames * 1e-3) / 1e9
-    roofline = {"bound": "hbm", "kernel": "k_persist", "achieved": achieved, "peak": pk["hbm_gbs"],
+    roofline = {"bound": "hbm", "kernel": "batch graph", "achieved": achieved, "peak": pk["hbm_gbs"],
                 "unit": "GB/s", "frac": achieved / pk["hbm_gbs"], "traffic": None, "peak_kind": pk_kind,
                 "avg_launch_ms": total_ms / a.frames, "algorithmic_bytes_per_launch": launch_bytes}
     cpu = None
@@ -1019,7 +1019,7 @@ def main():
     ms_plain, _ = timed(plain, plain_steps)
     plain_value = n * plain_steps / (ms_plain * 1e-3)
 
-    # the persistent batch kernel (one launch, replayed as a CUDA graph) on the same batch
+    # the batch entry point on the same poses
     rm.cost_grad_batch(gm, scans=scan, poses=poses)
     ms_pers, _ = timed(lambda: rm.cost_grad_batch(gm, scans=scan, poses=poses), a.steps)
     pers_value = n * a.steps / (ms_pers * 1e-3)

@@ -123,9 +123,8 @@ typedef struct {
   int32_t wave_poses;       /* poses processed together per kernel wave */
   int32_t async_status;     /* 1: do not read the device status back (graph capture);
                                check it later with rm_status_sync */
-  int32_t wait_log2;        /* 0: default budgets of the bounded device waits (about 2^31
-                               cycles for a bulk copy, 2^32 for the batch kernel's work
-                               queue); 1..40: every such wait gives up after 2^wait_log2
+  int32_t wait_log2;        /* 0: the default budget of the bounded device waits (about 2^31
+                               cycles for a bulk copy); 1..40: every such wait gives up after 2^wait_log2
                                cycles and the call returns RM_ETIMEOUT (a copy still in
                                flight is drained with the default budget first) */
   int32_t reserved[2];
@@ -433,22 +432,20 @@ typedef struct {
   const double *pose;
 } rm_problem;
 
-/* rm_cost_grad for n problems that may differ in camera model, resolution and scan, in ONE
- * persistent kernel: CTAs take (problem, phase, index) items from device ready queues; an item
- * enters a queue only when its problem's previous phase has completed (cluster culling ->
- * triangle setup -> tile raster -> reduction per problem), the number of setup items follows
- * the visible clusters, and raster/reduction items are served first. Every wait is bounded
- * (RM_ETIMEOUT). Outputs as for rm_cost_grad, per problem
- * (index k = problem). Screen tiles are 64x32 for pinhole problems and 16x16 for ray-table
- * problems, the per-call entry points' defaults, so a problem's results equal those of
- * rm_cost_grad with default tiles bit for bit. (Sec. IV.C / Sec. VI: many evaluations per
- * scan match; batching them is this library's extension.) */
+/* rm_cost_grad for n problems that may differ in camera model, resolution and scan. The problems of
+ * one camera model run in step, phase by phase (cluster culling, triangle setup, tile raster,
+ * reduction), the two models beside each other, as one captured graph. Problems that share one
+ * scan and camera, with poses back to back, run as the poses of one rm_cost_grad. Always waits.
+ * Outputs as for rm_cost_grad, per problem (index k = problem). Screen tiles are 64x32 for pinhole
+ * problems and 16x16 for ray-table problems, the per-call entry points' defaults, so a problem's
+ * results equal those of rm_cost_grad with default tiles bit for bit. (Sec. IV.C / Sec. VI: many
+ * evaluations per scan match; batching them is this library's extension.) */
 rm_status rm_cost_grad_batch(rm_map *map, const rm_problem *problems, int32_t n,
                              const rm_cost_params *params, const rm_cost_out *out, void *stream);
 
-/* rm_align for n problems at once: every LM iteration of every problem runs inside one
- * persistent-kernel launch (each problem's next evaluation waits for its own LM step), so a
- * whole tracking frame of mixed sensors is one launch. poses_out: n*16 doubles (host or
+/* rm_align for n problems at once: the evaluations and LM steps of all problems run in step on the
+ * device, several iterations to a graph launch, so a whole tracking frame of mixed sensors is a
+ * launch or two. poses_out: n*16 doubles (host or
  * device); reports: n entries (optional, host). Returns RM_ENOTCONV if any problem stopped at
  * max_iters (its pose is still written). */
 rm_status rm_align_batch(rm_map *map, const rm_problem *problems, int32_t n,
@@ -456,8 +453,8 @@ rm_status rm_align_batch(rm_map *map, const rm_problem *problems, int32_t n,
                          double *poses_out, rm_align_report *reports, void *stream);
 
 /* rm_icp_align for a batch of problems (each its own scan and start pose; pinhole and
- * ray-table problems mixed), every evaluation and step of every problem in one persistent
- * kernel (as rm_align_batch): params->max_iters evaluations per problem (1..100000), each
+ * ray-table problems mixed), the evaluations and steps of all problems in step on the device
+ * (as rm_align_batch): params->max_iters evaluations per problem (1..100000), each
  * followed by its Gauss-Newton step on the device. poses_out: n*16 doubles (host or device);
  * reps: n reports (optional, host). Returns RM_ENOTCONV when a problem did not converge. */
 rm_status rm_icp_align_batch(rm_map *map, const rm_problem *problems, int32_t n,

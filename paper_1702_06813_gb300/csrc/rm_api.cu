@@ -95,6 +95,7 @@ struct rm_map {
   bool zbuf_empty = false;
   unsigned *d_status = nullptr;
   unsigned *h_status = nullptr;
+  int *h_progress = nullptr;  // pinned: a loop's steps done, and whether it has ended
   rm_tuning tuning{};
   int cap = 512;      // records per pinhole tile bin; doubled whenever one overflows
   int cap_ray = 512;  // likewise for ray-table bins
@@ -106,7 +107,7 @@ struct rm_map {
   double prof_ms[4] = {0, 0, 0, 0};
   long long prof_n[4] = {0, 0, 0, 0};
   long long launches = 0;  // kernels launched since the last rm_profile(map, 1)
-  // persistent batch: its launches captured once per batch shape and replayed as a graph
+  // batches of problems: their launches captured once per batch shape and replayed as a graph
   cudaStream_t cap_stream = nullptr;
   // per-call waves alternate between the caller's stream and this one, so that one wave's
   // culling and setup overlap the previous wave's raster
@@ -114,10 +115,9 @@ struct rm_map {
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaGraphExec_t batch_exec = nullptr;
   std::string batch_sig;
-  // host copies of the batch queue, dependency counts and per-problem arguments last
-  // uploaded into the arena; valid until another call carves the arena
+  // host copy of the batch's per-problem arguments last uploaded into the arena; valid until
+  // another call carves the arena
   bool batch_inputs_valid = false;
-  std::vector<int> batch_shape;
   std::vector<WaveArgs> batch_args;
 };
 
@@ -325,6 +325,14 @@ rm_status ensure_arena(rm_map *m, size_t bytes, cudaStream_t s) {
   return RM_OK;
 }
 
+// The second stream and the events that fork to it and join it.
+rm_status ensure_aux(rm_map *m) {
+  if (!m->aux_stream) RM_CK(cudaStreamCreateWithFlags(&m->aux_stream, cudaStreamNonBlocking));
+  if (!m->ev_fork) RM_CK(cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming));
+  if (!m->ev_join) RM_CK(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
+  return RM_OK;
+}
+
 // The z-buffers of a call's waves (`keys` of them, every one kKeyEmpty): kept between calls, because
 // the raster leaves every key it reads empty, so a call pays only for the tiles it touches.
 rm_status ensure_zbuf(rm_map *m, size_t keys, cudaStream_t s) {
@@ -364,12 +372,12 @@ rm_status check_intr(const rm_intrinsics *in) {
   return fail(RM_EINVAL, "unknown camera model");
 }
 
-TileGeom make_tiles(const rm_map *m, const rm_intrinsics *in) {
+// The map's tuned tile, or the camera model's default (always that one for batches of problems).
+TileGeom make_tiles(const rm_map *m, const rm_intrinsics *in, bool tuned = true) {
   TileGeom tg;
-  // default: the persistent kernel's tile for the camera model (64x32 pinhole, 16x16 ray table)
   const int md = in->model == RM_RAYTABLE ? 1 : 0;
-  tg.tw = m->tuning.tile_w > 0 ? m->tuning.tile_w : rmk::kPersistTileW[md];
-  tg.th = m->tuning.tile_h > 0 ? m->tuning.tile_h : rmk::kPersistTileH[md];
+  tg.tw = tuned && m->tuning.tile_w > 0 ? m->tuning.tile_w : rmk::kTileW[md];
+  tg.th = tuned && m->tuning.tile_h > 0 ? m->tuning.tile_h : rmk::kTileH[md];
   tg.ntx = (in->width + tg.tw - 1) / tg.tw;
   tg.nty = (in->height + tg.th - 1) / tg.th;
   tg.ntiles = tg.ntx * tg.nty;
@@ -457,11 +465,11 @@ rm_status drain_events(rm_map *m) {
 }
 
 // One wave, with events around its kernels when profiling.
-rm_status wave(rm_map *m, const WaveArgs &a, int mode, cudaStream_t s, bool zero_counters = true) {
+rm_status wave(rm_map *m, const WaveArgs &a, int mode, cudaStream_t s, bool reduce = true) {
   cudaEvent_t ev[5];
   if (m->prof) RM_TRY(take_events(m, ev));
-  RM_CK(rmk::launch_wave(a, mode, s, m->prof ? ev : nullptr, zero_counters));
-  m->launches += rmk::wave_kernel_launches(a, mode);
+  RM_CK(rmk::launch_wave(a, mode, s, m->prof ? ev : nullptr, false, reduce));
+  m->launches += rmk::wave_kernel_launches(a, mode, reduce);
   if (m->prof) m->ev_pending.push_back({ev[0], ev[1], ev[2], ev[3], ev[4]});
   return RM_OK;
 }
@@ -506,6 +514,7 @@ struct EvalReq {
   float *depth;
   int32_t *tri_id;
   float *bary;
+  bool batch = false;     // a batch call: default tiles, and the status is always read back
 };
 
 rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
@@ -545,7 +554,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
   const bool dev_ijtj = icp_mode && r.icp->jtj && on_device(r.icp->jtj);
 
   for (int attempt = 0;; ++attempt) {
-    TileGeom tg = make_tiles(m, in);
+    TileGeom tg = make_tiles(m, in, !r.batch);
     const int nw = wave_size(m, r.n, tg, P);
     // ---- plan the arena
     Carver plan{nullptr};
@@ -664,9 +673,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       m->launches += 1;
     }
     if (nbuf == 2) {
-      if (!m->aux_stream) RM_CK(cudaStreamCreateWithFlags(&m->aux_stream, cudaStreamNonBlocking));
-      if (!m->ev_fork) RM_CK(cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming));
-      if (!m->ev_join) RM_CK(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
+      RM_TRY(ensure_aux(m));
       RM_CK(cudaEventRecord(m->ev_fork, s));
       RM_CK(cudaStreamWaitEvent(m->aux_stream, m->ev_fork, 0));
     }
@@ -682,7 +689,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       a.partial = d_partial + (size_t)tg.ntiles * rmk::kNumVals * nw * b;
       a.zbuf = m->zbuf + (size_t)P * nw * b;
       a.touched = d_touched + (size_t)w0 * tg.ntiles;
-      RM_TRY(wave(m, a, r.mode, b == 0 ? s : m->aux_stream, false));
+      RM_TRY(wave(m, a, r.mode, b == 0 ? s : m->aux_stream));
     }
     m->zbuf_empty = true;
     if (nbuf == 2) {
@@ -710,7 +717,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
         if (!dev_jtj) RM_TRY(copy_out(r.out->jtj, d_jtj, sizeof(double) * 21 * r.n, s, &host_out));
       }
     }
-    if (m->tuning.async_status) {
+    if (m->tuning.async_status && !r.batch) {
       if (host_out) RM_CK(cudaStreamSynchronize(s));
       return RM_OK;
     }
@@ -729,11 +736,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
 
 namespace {
 
-// Raster items of one problem in the persistent queue.
-int raster_items(const TileGeom &tg, int model) {
-  const int per = rmk::kPersistTiles[model == RM_RAYTABLE ? 1 : 0];
-  return (tg.ntiles + per - 1) / per;
-}
+constexpr int kBatchChunk = 8;  // evaluations per captured graph
 
 // Shared driver of rm_cost_grad_batch (lm == icp == nullptr), rm_align_batch (lm) and
 // rm_icp_align_batch (icp; prm->eps then carries the association tolerance).
@@ -743,7 +746,7 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
                     rm_icp_report *ireps = nullptr) {
   if (n < 0) return fail(RM_EINVAL, "n < 0");
   if (n == 0) return RM_OK;
-  if (n >= (1 << rmk::kItemProblemBits)) return fail(RM_EINVAL, "too many problems in one batch");
+  if (n >= (1 << 23)) return fail(RM_EINVAL, "too many problems in one batch");
   if (!probs || !prm) return fail(RM_EINVAL, "NULL argument");
   if (!(prm->eps >= 0.0f)) return fail(RM_EINVAL, "eps must be >= 0");
   if (lm && (lm->max_iters < 0 || lm->max_iters > 100000)) return fail(RM_EINVAL, "max_iters out of range");
@@ -755,267 +758,221 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       return fail(RM_EINVAL, "problem " + std::to_string(p) + ": NULL scan array or pose");
   }
   RM_CK(cudaSetDevice(m->device));
+  // poses laid out back to back (one n x 16 array) are copied in one call
+  bool poses_contiguous = true;
+  for (int p = 1; p < n && poses_contiguous; ++p) poses_contiguous = probs[p].pose == probs[0].pose + 16 * (size_t)p;
+  // a plain batch of one scan and camera is the poses of one per-pose call (its waves take 1.5 ms
+  // where the problem-by-problem phases below take 1.9, on 256 poses of 640x480)
+  bool same = !lm && !icp && poses_contiguous;
+  for (int p = 1; p < n && same; ++p)
+    same = probs[p].scan.depth == probs[0].scan.depth && probs[p].scan.cls == probs[0].scan.cls &&
+           std::memcmp(&probs[p].scan.intr, &probs[0].scan.intr, sizeof(rm_intrinsics)) == 0;
+  if (same) {
+    EvalReq r{&probs[0].scan.intr, &probs[0].scan, probs[0].pose, n, prm, rmk::kCostGrad, out, nullptr, nullptr,
+              nullptr, nullptr};
+    r.batch = true;
+    return run_eval(m, r, s);
+  }
   const int K = lm ? lm->max_iters : (icp ? icp->max_iters - 1 : 0);
   const int nc = m->n_clusters;
-  // at least one item per phase, so that every phase completes and publishes the next
-  const int ncull = std::max(1, ((nc + 255) / 256 + rmk::kPersistCull - 1) / rmk::kPersistCull);
-  // setup items per evaluation are set on the device from the visible clusters; at most
-  const int max_setup = std::max(1, (nc + rmk::kSetupClusters - 1) / rmk::kSetupClusters);
-  if (max_setup >= (1 << rmk::kItemIndexBits)) return fail(RM_EINVAL, "map has too many clusters for a batch");
-  for (int attempt = 0;; ++attempt) {
-    std::vector<TileGeom> tg(n);
-    std::vector<long long> P(n);
-    size_t tiles_total = 0, bins_bytes = 0, px_total = 0, rays_total = 0;
-    // problems that share a scan (same arrays) share one staged copy; likewise ray tables
-    std::vector<int> scan_of(n), rays_of(n, -1);
-    {
-      using Key = std::tuple<const void *, const void *, int, int>;
-      std::map<Key, int> scans, rays;
-      for (int p = 0; p < n; ++p) {
-        const rm_scan &sc = probs[p].scan;
-        scan_of[p] = scans.emplace(Key(sc.depth, sc.cls, sc.intr.width, sc.intr.height), p).first->second;
-        if (sc.intr.model == RM_RAYTABLE)
-          rays_of[p] = rays.emplace(Key(sc.intr.rays, nullptr, sc.intr.width, sc.intr.height), p).first->second;
-      }
+  // problems in order of camera model: `order[k]` is the problem of argument block k
+  std::vector<int> order;
+  for (int md = 0; md < 2; ++md)
+    for (int p = 0; p < n; ++p)
+      if ((probs[p].scan.intr.model == RM_RAYTABLE) == (md == 1)) order.push_back(p);
+  int n_pin = 0;
+  for (int p = 0; p < n; ++p) n_pin += probs[p].scan.intr.model != RM_RAYTABLE;
+  // problems that share a host array share one staged copy; device arrays are read in place
+  using Key = std::tuple<const void *, int, int>;
+  std::map<Key, size_t> staged;    // offset in the staging area
+  std::map<const void *, int> tables;  // ray tables, numbered
+  size_t stage_bytes = 0;
+  auto stage = [&](const void *h, size_t bytes, int W, int H) {
+    if (!on_device(h) && staged.emplace(Key(h, W, H), stage_bytes).second) stage_bytes += align_up(bytes, 256);
+  };
+  for (int p = 0; p < n; ++p) {
+    const rm_scan &sc = probs[p].scan;
+    const size_t P = (size_t)sc.intr.width * sc.intr.height;
+    stage(sc.depth, sizeof(float) * P, sc.intr.width, sc.intr.height);
+    stage(sc.cls, P, sc.intr.width, sc.intr.height);
+    if (sc.intr.model == RM_RAYTABLE) {
+      stage(sc.intr.rays, sizeof(float) * 3 * P, sc.intr.width, sc.intr.height);
+      tables.emplace(sc.intr.rays, (int)tables.size());
     }
+  }
+  for (int attempt = 0;; ++attempt) {
+    size_t tiles_total = 0, bins_bytes = 0, px_total = 0;
+    int max_tiles[2] = {1, 1};
+    std::vector<TileGeom> tg(n);
     for (int p = 0; p < n; ++p) {
       const rm_intrinsics *in = &probs[p].scan.intr;
       const int md = in->model == RM_RAYTABLE ? 1 : 0;
-      tg[p].tw = rmk::kPersistTileW[md];
-      tg[p].th = rmk::kPersistTileH[md];
-      tg[p].ntx = (in->width + tg[p].tw - 1) / tg[p].tw;
-      tg[p].nty = (in->height + tg[p].th - 1) / tg[p].th;
-      tg[p].ntiles = tg[p].ntx * tg[p].nty;
-      tg[p].cap = in->model == RM_RAYTABLE ? m->cap_ray : m->cap;
-      tg[p].rec_bytes = in->model == RM_RAYTABLE ? (int)sizeof(rmk::RayRec) : (int)sizeof(TriRec);
-      P[p] = (long long)in->width * in->height;
+      tg[p] = make_tiles(m, in, false);
       tiles_total += tg[p].ntiles;
       bins_bytes += align_up((size_t)tg[p].ntiles * tg[p].cap * tg[p].rec_bytes, 256);
-      if (scan_of[p] == p) px_total += align_up((size_t)P[p], 64);
-      if (rays_of[p] == p) rays_total += 3 * (size_t)P[p];
-    }
-    // the ready queue: one slot per item of every evaluation of every problem; the kernel
-    // publishes a problem's items phase by phase. The dependency counts are a function of
-    // `shape` alone and are re-sent only when it changes or the arena was reused.
-    std::vector<int> shape = {n, K, ncull};
-    size_t cap_hi = 0, cap_lo = 0;  // raster + reduce slots, cull + setup slots
-    for (int p = 0; p < n; ++p) {
-      const int nr = raster_items(tg[p], probs[p].scan.intr.model);
-      shape.push_back(nr);
-      cap_hi += (size_t)(K + 1) * (nr + 1);
-      cap_lo += (size_t)(K + 1) * (ncull + max_setup);
-    }
-    const bool same_shape = shape == m->batch_shape;
-    std::vector<int> need(3 * (size_t)n);
-    for (int p = 0; p < n; ++p) {
-      need[3 * p] = ncull;
-      need[3 * p + 1] = 0;  // set by the kernel
-      need[3 * p + 2] = raster_items(tg[p], probs[p].scan.intr.model);
+      px_total += (size_t)in->width * in->height;
+      max_tiles[md] = std::max(max_tiles[md], tg[p].ntiles);
     }
     // ---- plan and carve the arena
-    auto layout = [&](Carver &cv, bool carve, WaveArgs **d_args, long long **d_items, int **d_next,
-                      int **d_done, int **d_need, float **d_M, int **d_skip, double **d_poses,
-                      rmk::LMState **d_lm, int **d_vcount, int4 **d_vis, int **d_counts,
-                      double **d_partial, unsigned char **d_bins, float **d_sd, uint8_t **d_sc,
-                      float **d_rays, long long **r_counts, long long **r_et, double **r_els,
-                      double **r_grad, double **r_jtj, rmk::IcpState **d_icp, double **r_l1) {
-      (void)carve;
-      *d_args = cv.take<WaveArgs>(n);
-      *d_items = cv.take<long long>(cap_hi + cap_lo);
-      *d_next = cv.take<int>(8);  // queue heads and tails, finished problems
-      *d_done = cv.take<int>(4 * (size_t)n);
-      *d_need = cv.take<int>(3 * (size_t)n);
-      *d_M = cv.take<float>(12 * (size_t)n);
-      *d_skip = cv.take<int>(n);
-      *d_poses = cv.take<double>(16 * (size_t)n);
-      *d_lm = cv.take<rmk::LMState>(n);
-      *d_vcount = cv.take<int>(n);
-      *d_vis = cv.take<int4>((size_t)n * std::max(nc, 1));
-      *d_counts = cv.take<int>(tiles_total);
-      *d_partial = cv.take<double>(tiles_total * rmk::kNumVals);
-      *d_bins = cv.take<unsigned char>(bins_bytes);
-      *d_sd = cv.take<float>(px_total);
-      *d_sc = cv.take<uint8_t>(px_total);
-      *d_rays = cv.take<float>(std::max<size_t>(rays_total, 1));
-      *r_counts = cv.take<long long>(6 * (size_t)n);
-      *r_et = cv.take<long long>(n);
-      *r_els = cv.take<double>(n);
-      *r_grad = cv.take<double>(6 * (size_t)n);
-      *r_jtj = cv.take<double>(21 * (size_t)n);
-      *d_icp = cv.take<rmk::IcpState>(n);
-      *r_l1 = cv.take<double>(n);
+    struct Arrays {
+      WaveArgs *args;
+      int *evals, *skip, *counters;  // counters: visible clusters, then bin counts and touched flags
+      float *M;
+      double *poses;
+      rmk::LMState *lm;
+      rmk::IcpState *icp;
+      int4 *vis;
+      double *partial, *els, *grad, *jtj, *l1;
+      unsigned char *bins, *staged;
+      long long *counts, *et;
+      int *dev;
+    } d;
+    auto layout = [&](Carver &cv) {
+      d.args = cv.take<WaveArgs>(n);
+      d.evals = cv.take<int>(n);
+      d.skip = cv.take<int>(n);
+      d.M = cv.take<float>(12 * (size_t)n);
+      d.poses = cv.take<double>(16 * (size_t)n);
+      d.lm = cv.take<rmk::LMState>(n);
+      d.icp = cv.take<rmk::IcpState>(n);
+      d.counters = cv.take<int>(n + 2 * tiles_total);
+      d.vis = cv.take<int4>((size_t)n * std::max(nc, 1));
+      d.partial = cv.take<double>(tiles_total * rmk::kNumVals);
+      d.bins = cv.take<unsigned char>(bins_bytes);
+      d.staged = cv.take<unsigned char>(stage_bytes);
+      d.counts = cv.take<long long>(6 * (size_t)n);
+      d.et = cv.take<long long>(n);
+      d.els = cv.take<double>(n);
+      d.grad = cv.take<double>(6 * (size_t)n);
+      d.jtj = cv.take<double>(21 * (size_t)n);
+      d.l1 = cv.take<double>(n);
+      d.dev = cv.take<int>(2 * tables.size());
     };
-    WaveArgs *d_args; long long *d_items; int4 *d_vis; int *d_next, *d_done, *d_need, *d_skip, *d_vcount, *d_counts;
-    float *d_M, *d_sd, *d_rays; double *d_poses, *d_partial, *r_els, *r_grad, *r_jtj; rmk::LMState *d_lm;
-    unsigned char *d_bins; uint8_t *d_sc; long long *r_counts, *r_et;
-    rmk::IcpState *d_icp; double *r_l1;
     Carver plan{nullptr};
-    layout(plan, false, &d_args, &d_items, &d_next, &d_done, &d_need, &d_M, &d_skip, &d_poses, &d_lm,
-           &d_vcount, &d_vis, &d_counts, &d_partial, &d_bins, &d_sd, &d_sc, &d_rays, &r_counts, &r_et,
-           &r_els, &r_grad, &r_jtj, &d_icp, &r_l1);
+    layout(plan);
     RM_TRY(ensure_arena(m, plan.off, s));
+    RM_TRY(ensure_zbuf(m, px_total, s));
     Carver cv{m->arena};
-    layout(cv, true, &d_args, &d_items, &d_next, &d_done, &d_need, &d_M, &d_skip, &d_poses, &d_lm,
-           &d_vcount, &d_vis, &d_counts, &d_partial, &d_bins, &d_sd, &d_sc, &d_rays, &r_counts, &r_et,
-           &r_els, &r_grad, &r_jtj, &d_icp, &r_l1);
-    // ---- per-problem arguments and inputs
-    // poses laid out back to back (one n x 16 array) are copied in one call
-    bool poses_contiguous = true;
-    for (int p = 1; p < n && poses_contiguous; ++p) poses_contiguous = probs[p].pose == probs[0].pose + 16 * (size_t)p;
-    if (poses_contiguous)
-      RM_CK(cudaMemcpyAsync(d_poses, probs[0].pose, sizeof(double) * 16 * n,
+    layout(cv);
+    // ---- inputs
+    if (poses_contiguous) {
+      RM_CK(cudaMemcpyAsync(d.poses, probs[0].pose, sizeof(double) * 16 * n,
                             on_device(probs[0].pose) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+    } else {
+      for (int p = 0; p < n; ++p)
+        RM_CK(cudaMemcpyAsync(d.poses + 16 * (size_t)p, probs[p].pose, sizeof(double) * 16,
+                              on_device(probs[p].pose) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+    }
+    std::vector<char> sent(staged.size(), 0), measured(tables.size(), 0);
+    auto device_array = [&](const void *h, size_t bytes, int W, int H, const void **dv) -> rm_status {
+      const auto it = staged.find(Key(h, W, H));
+      if (it == staged.end()) {
+        *dv = h;
+        return RM_OK;
+      }
+      *dv = d.staged + it->second;
+      char &done = sent[(size_t)std::distance(staged.begin(), it)];
+      if (!done) RM_CK(cudaMemcpyAsync(d.staged + it->second, h, bytes, cudaMemcpyHostToDevice, s));
+      done = 1;
+      return RM_OK;
+    };
     std::vector<WaveArgs> args(n);
-    std::vector<size_t> px_at(n), rays_at(n);
-    size_t t_off = 0, b_off = 0, px_off = 0, r_off = 0;
-    for (int p = 0; p < n; ++p) {
+    size_t t_off = 0, b_off = 0, px_off = 0;
+    for (int k = 0; k < n; ++k) {
+      const int p = order[k];
       const rm_scan &sc = probs[p].scan;
       const rm_intrinsics *in = &sc.intr;
-      float *rays = nullptr;
-      if (in->model == RM_RAYTABLE) {
-        if (rays_of[p] == p) {
-          rays_at[p] = r_off;
-          r_off += 3 * (size_t)P[p];
-          RM_CK(cudaMemcpyAsync(d_rays + rays_at[p], in->rays, sizeof(float) * 3 * P[p],
-                                on_device(in->rays) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-        } else {
-          rays_at[p] = rays_at[rays_of[p]];
-        }
-        rays = d_rays + rays_at[p];
-      }
-      if (scan_of[p] == p) {
-        px_at[p] = px_off;
-        px_off += align_up((size_t)P[p], 64);
-        RM_CK(cudaMemcpyAsync(d_sd + px_at[p], sc.depth, sizeof(float) * P[p],
-                              on_device(sc.depth) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-        RM_CK(cudaMemcpyAsync(d_sc + px_at[p], sc.cls, (size_t)P[p],
-                              on_device(sc.cls) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-      } else {
-        px_at[p] = px_at[scan_of[p]];
-      }
-      if (!poses_contiguous)
-        RM_CK(cudaMemcpyAsync(d_poses + 16 * (size_t)p, probs[p].pose, sizeof(double) * 16,
-                              on_device(probs[p].pose) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-      WaveArgs &a = args[p];
+      const size_t P = (size_t)in->width * in->height;
+      const void *sd, *cls, *rays = nullptr;
+      RM_TRY(device_array(sc.depth, sizeof(float) * P, in->width, in->height, &sd));
+      RM_TRY(device_array(sc.cls, P, in->width, in->height, &cls));
+      if (in->model == RM_RAYTABLE) RM_TRY(device_array(in->rays, sizeof(float) * 3 * P, in->width, in->height, &rays));
+      WaveArgs &a = args[k];
       std::memset(&a, 0, sizeof(WaveArgs));  // padding too: the argument block is compared bytewise
-      a.cam = make_cam(in, rays);
+      a.cam = make_cam(in, static_cast<const float *>(rays));
       a.tg = tg[p];
       a.V = (int)m->V;
       a.T = m->T;
       a.n_poses = 1;
+      a.problem = p;
       a.wave_base = 0;
       a.v = m->d_v;
       a.faces = m->d_faces;
       a.planes = m->d_planes;
       set_map_fields(m, a);
-      a.Ms = d_M + 12 * (size_t)p;
-      a.vis = d_vis + (size_t)p * std::max(nc, 1);
-      a.vis_count = d_vcount + p;
-      a.counts = d_counts + t_off;
-      a.bins = d_bins + b_off;
-      a.partial = d_partial + t_off * rmk::kNumVals;
+      a.Ms = d.M + 12 * (size_t)p;
+      a.vis = d.vis + (size_t)k * std::max(nc, 1);
+      a.vis_count = d.counters + k;
+      a.counts = d.counters + n + t_off;
+      a.touched = d.counters + n + tiles_total + t_off;
+      a.zbuf = m->zbuf + px_off;
+      if (rays) {
+        const int t = tables[in->rays];
+        a.ray_dev = d.dev + 2 * t;
+        if (!measured[t]) RM_CK(rmk::launch_ray_dev(a.cam, d.dev + 2 * t, s));
+        measured[t] = 1;
+      }
+      a.bins = d.bins + b_off;
+      a.partial = d.partial + t_off * rmk::kNumVals;
       a.status = m->d_status;
-      a.skip = d_skip + p;
-      a.scan_depth = d_sd + px_at[p];
-      a.scan_cls = d_sc + px_at[p];
+      a.skip = d.skip + p;
+      a.scan_depth = static_cast<const float *>(sd);
+      a.scan_cls = static_cast<const uint8_t *>(cls);
       a.prm = {prm->eps, prm->w_fofo, prm->w_fofu, prm->w_fufo};
-      a.res_counts = r_counts + 6 * (size_t)p;
-      a.res_etable = r_et + p;
-      a.res_els = r_els + p;
-      a.res_grad = r_grad + 6 * (size_t)p;
-      a.res_jtj = r_jtj + 21 * (size_t)p;
+      a.res_counts = d.counts + 6 * (size_t)p;
+      a.res_etable = d.et + p;
+      a.res_els = d.els + p;
+      a.res_grad = d.grad + 6 * (size_t)p;
+      a.res_jtj = d.jtj + 21 * (size_t)p;
       if (icp) {  // ICP terms: associations, C, e^2, J^T e, J^T J
         a.res_counts = nullptr;
         a.res_etable = nullptr;
-        a.res_n = r_counts + p;
-        a.res_l1 = r_l1 + p;
+        a.res_n = d.counts + p;
+        a.res_l1 = d.l1 + p;
       }
       t_off += tg[p].ntiles;
+      px_off += P;
       b_off += align_up((size_t)tg[p].ntiles * tg[p].cap * tg[p].rec_bytes, 256);
     }
-    // the queue, dependency counts and argument blocks are re-sent only when they changed
-    // since the last batch call on this arena (same shape and buffers: nothing to send)
+    // the argument blocks are re-sent only when they changed since the last batch call on this arena
     // (batch_inputs_valid is read here, after ensure_arena: a reallocated arena holds nothing)
-    const bool dev_shape = m->batch_inputs_valid && same_shape;
-    const bool same_args = dev_shape && m->batch_args.size() == args.size() &&
+    const bool same_args = m->batch_inputs_valid && m->batch_args.size() == args.size() &&
                            std::memcmp(m->batch_args.data(), args.data(), sizeof(WaveArgs) * n) == 0;
     m->batch_inputs_valid = false;
-    if (!dev_shape)
-      RM_CK(cudaMemcpyAsync(d_need, need.data(), sizeof(int) * need.size(), cudaMemcpyHostToDevice, s));
-    m->batch_shape = shape;
     if (!same_args) {
-      RM_CK(cudaMemcpyAsync(d_args, args.data(), sizeof(WaveArgs) * n, cudaMemcpyHostToDevice, s));
+      RM_CK(cudaMemcpyAsync(d.args, args.data(), sizeof(WaveArgs) * n, cudaMemcpyHostToDevice, s));
       m->batch_args = args;
     }
     m->batch_inputs_valid = true;
-    rmk::LMArgs la{};
-    la.cx = m->centre[0];
-    la.cy = m->centre[1];
-    la.cz = m->centre[2];
-    if (lm) {
-      la.lambda0 = lm->lambda0;
-      la.lambda_up = lm->lambda_up;
-      la.lambda_down = lm->lambda_down;
-      la.step_tol = lm->step_tol;
-    }
+    const rmk::LMArgs la{lm ? lm->lambda0 : 0.0, lm ? lm->lambda_up : 0.0, lm ? lm->lambda_down : 0.0,
+                         lm ? lm->step_tol : 0.0, m->centre[0], m->centre[1], m->centre[2]};
+    const rmk::IcpArgs ia{icp ? icp->step_tol : 0.0, m->centre[0], m->centre[1], m->centre[2]};
     rmk::BatchArgs b{};
-    b.probs = d_args;
-    if (cap_hi + cap_lo > (size_t)INT32_MAX) return fail(RM_EINVAL, "batch too large for the work queue");
-    b.n_problems = n;
-    b.items = d_items;
-    b.cap[0] = (int)cap_hi;
-    b.cap[1] = (int)cap_lo;
-    b.qctl = d_next;
-    b.done = d_done;
-    b.need = d_need;
-    b.lm = lm ? d_lm : nullptr;
-    b.icp = icp ? d_icp : nullptr;
-    rmk::IcpArgs ia{icp ? icp->step_tol : 0.0, m->centre[0], m->centre[1], m->centre[2]};
-    b.icpargs = ia;
-    b.Ms = d_M;
-    b.skip = d_skip;
+    b.lm = lm ? d.lm : nullptr;
+    b.icp = icp ? d.icp : nullptr;
+    b.evals = lm || icp ? d.evals : nullptr;
+    b.Ms = d.M;
+    b.skip = d.skip;
     b.lmargs = la;
+    b.icpargs = ia;
     b.lm_iters = K;
-    b.status = m->d_status;
-    b.spin_limit = wait_budget(m, 1ll << 32);
-    // A homogeneous plain batch (one scan, camera and parameters for every problem, no LM or
-    // ICP) runs as the poses of one wave: its argument block is a kernel parameter. The
-    // problems' arrays are already laid out at the wave's per-pose offsets, provided each
-    // problem's bins end on the 256-byte boundary where the next one's start.
-    bool wave_form = !lm && !icp && nc >= 1 &&
-                     ((size_t)tg[0].ntiles * tg[0].cap * tg[0].rec_bytes) % 256 == 0;
-    for (int p = 1; p < n && wave_form; ++p)
-      wave_form = scan_of[p] == 0 && std::memcmp(&probs[p].scan.intr, &probs[0].scan.intr, sizeof(rm_intrinsics)) == 0;
-    WaveArgs w;
-    std::memset(&w, 0, sizeof(w));
-    if (wave_form) {
-      w = args[0];
-      w.n_poses = n;
-      w.wave_base = 0;
-      w.skip = nullptr;
-    }
-    const int grid = wave_form ? rmk::persist_wave_grid(m->device, w.cam.model) : rmk::persist_grid(m->device);
-    if (grid <= 0) return fail(RM_ECUDA, "could not size the persistent grid");
-    // counters to zero, LM state / pose matrices, the persistent kernel: one captured graph
-    // per batch shape (the arena layout is a function of the shape), replayed every call
+    RM_CK(cudaMemsetAsync(d.evals, 0, sizeof(int) * n, s));
+    RM_CK(cudaMemsetAsync(d.skip, 0, sizeof(int) * n, s));
+    RM_CK(cudaMemsetAsync(d.counters, 0, sizeof(int) * (n + 2 * tiles_total), s));
+    if (lm) RM_CK(rmk::launch_lm_init_batch(d.lm, d.poses, n, la, d.M, d.skip, s));
+    else if (icp) RM_CK(rmk::launch_icp_init_batch(d.icp, d.poses, n, ia, d.M, d.skip, s));
+    else RM_CK(rmk::launch_pose_to_m(d.poses, n, m->centre[0], m->centre[1], m->centre[2], d.M, s));
+    m->launches += 1;
+    // up to kBatchChunk evaluations as one graph, the pinhole and the ray-table problems on two
+    // branches that do not wait for each other; captured once per batch shape and replayed, the
+    // evaluations past the last one doing nothing
+    const int E = std::min(K + 1, kBatchChunk);
     char sig[512];
-    std::snprintf(sig, sizeof(sig), "%p|%d|%d|%zu|%d|%d|%a|%a|%a|%a|%zu|%zu|%zu|%d|%a|%lld", (void *)m->arena, n,
-                  K, cap_hi + cap_lo, grid, lm ? 1 : (icp ? 2 : 0), la.lambda0, la.lambda_up, la.lambda_down,
-                  la.step_tol, tiles_total, px_total, rays_total, m->cap * 4096 + m->cap_ray, ia.step_tol,
-                  b.spin_limit);
-    std::string key(sig);
-    if (wave_form) {  // the graph holds w by value: a different w needs a new capture
-      key += "|wave:";
-      const unsigned char *wb = reinterpret_cast<const unsigned char *>(&w);
-      for (size_t k = 0; k < sizeof(w); ++k) {
-        static const char hex[] = "0123456789abcdef";
-        key += hex[wb[k] >> 4];
-        key += hex[wb[k] & 15];
-      }
-    }
-    for (int p = 0; p < n; ++p) key += "|" + std::to_string(probs[p].scan.intr.model) + "x" +
-                                        std::to_string(probs[p].scan.intr.width) + "x" +
-                                        std::to_string(probs[p].scan.intr.height);
+    std::snprintf(sig, sizeof(sig), "%p|%d|%d|%d|%d|%a|%a|%a|%a|%zu|%zu|%zu|%d|%d|%a|%p|%d|%d|%d", (void *)m->arena, n,
+                  n_pin, K, lm ? 1 : (icp ? 2 : 0), la.lambda0, la.lambda_up, la.lambda_down, la.step_tol, tiles_total,
+                  px_total, stage_bytes, m->cap, m->cap_ray, ia.step_tol, (void *)m->d_vn, max_tiles[0], max_tiles[1],
+                  (int)tables.size());
+    const std::string key(sig);
     if (!m->batch_exec || key != m->batch_sig) {
       if (m->batch_exec) {
         RM_CK(cudaGraphExecDestroy(m->batch_exec));
@@ -1023,22 +980,28 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
         m->batch_sig.clear();
       }
       if (!m->cap_stream) RM_CK(cudaStreamCreateWithFlags(&m->cap_stream, cudaStreamNonBlocking));
+      RM_TRY(ensure_aux(m));
       cudaStream_t c = m->cap_stream;
+      const int mode = icp ? rmk::kIcp : rmk::kCostGrad;
       RM_CK(cudaStreamBeginCapture(c, cudaStreamCaptureModeThreadLocal));
       cudaError_t e = cudaSuccess;
       auto rec = [&](cudaError_t x) {
         if (e == cudaSuccess) e = x;
       };
-      rec(cudaMemsetAsync(d_next, 0, 8 * sizeof(int), c));
-      rec(rmk::launch_queue_init(d_items, (int)(cap_hi + cap_lo), (int)cap_hi, n, ncull, d_next, c));
-      rec(cudaMemsetAsync(d_done, 0, sizeof(int) * 4 * n, c));
-      rec(cudaMemsetAsync(d_skip, 0, sizeof(int) * n, c));
-      rec(cudaMemsetAsync(d_vcount, 0, sizeof(int) * n, c));
-      rec(cudaMemsetAsync(d_counts, 0, sizeof(int) * tiles_total, c));
-      if (lm) rec(rmk::launch_lm_init_batch(d_lm, d_poses, n, la, d_M, d_skip, c));
-      else if (icp) rec(rmk::launch_icp_init_batch(d_icp, d_poses, n, ia, d_M, d_skip, c));
-      else rec(rmk::launch_pose_to_m(d_poses, n, m->centre[0], m->centre[1], m->centre[2], d_M, c));
-      rec(wave_form ? rmk::launch_persist_wave(b, w, grid, c) : rmk::launch_persist(b, grid, c));
+      const bool fork = n_pin > 0 && n_pin < n;
+      if (fork) {
+        rec(cudaEventRecord(m->ev_fork, c));
+        rec(cudaStreamWaitEvent(m->aux_stream, m->ev_fork, 0));
+      }
+      for (int it = 0; it < E; ++it) {
+        rec(rmk::launch_batch_eval(d.args, n_pin, 0, mode, m->d_vn != nullptr, nc, max_tiles[0], b, c));
+        rec(rmk::launch_batch_eval(d.args + n_pin, n - n_pin, 1, mode, m->d_vn != nullptr, nc, max_tiles[1], b,
+                                   fork ? m->aux_stream : c));
+      }
+      if (fork) {
+        rec(cudaEventRecord(m->ev_join, m->aux_stream));
+        rec(cudaStreamWaitEvent(c, m->ev_join, 0));
+      }
       cudaGraph_t graph = nullptr;
       const cudaError_t ec = cudaStreamEndCapture(c, &graph);
       if (e == cudaSuccess) e = ec;
@@ -1050,27 +1013,30 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       }
       m->batch_sig = key;
     }
-    RM_CK(cudaGraphLaunch(m->batch_exec, s));
-    m->launches += 2;
+    m->zbuf_empty = false;  // until every evaluation's raster is on its way
+    for (int it = 0; it <= K; it += E) {
+      RM_CK(cudaGraphLaunch(m->batch_exec, s));
+      m->launches += (size_t)E * ((n_pin > 0) + (n_pin < n)) * (nc > 0 ? 4 : 2);
+    }
+    m->zbuf_empty = true;
     bool host_out = false;
     std::vector<rmk::LMState> hs;
     std::vector<rmk::IcpState> his;
     if (lm) {
       hs.resize(n);
-      RM_CK(cudaMemcpyAsync(hs.data(), d_lm, sizeof(rmk::LMState) * n, cudaMemcpyDeviceToHost, s));
+      RM_CK(cudaMemcpyAsync(hs.data(), d.lm, sizeof(rmk::LMState) * n, cudaMemcpyDeviceToHost, s));
     } else if (icp) {
       his.resize(n);
-      RM_CK(cudaMemcpyAsync(his.data(), d_icp, sizeof(rmk::IcpState) * n, cudaMemcpyDeviceToHost, s));
+      RM_CK(cudaMemcpyAsync(his.data(), d.icp, sizeof(rmk::IcpState) * n, cudaMemcpyDeviceToHost, s));
     } else if (out) {
-      RM_TRY(copy_out(out->counts, r_counts, sizeof(long long) * 6 * n, s, &host_out));
-      RM_TRY(copy_out(out->e_table, r_et, sizeof(long long) * n, s, &host_out));
-      RM_TRY(copy_out(out->e_ls, r_els, sizeof(double) * n, s, &host_out));
-      RM_TRY(copy_out(out->grad, r_grad, sizeof(double) * 6 * n, s, &host_out));
-      RM_TRY(copy_out(out->jtj, r_jtj, sizeof(double) * 21 * n, s, &host_out));
+      RM_TRY(copy_out(out->counts, d.counts, sizeof(long long) * 6 * n, s, &host_out));
+      RM_TRY(copy_out(out->e_table, d.et, sizeof(long long) * n, s, &host_out));
+      RM_TRY(copy_out(out->e_ls, d.els, sizeof(double) * n, s, &host_out));
+      RM_TRY(copy_out(out->grad, d.grad, sizeof(double) * 6 * n, s, &host_out));
+      RM_TRY(copy_out(out->jtj, d.jtj, sizeof(double) * 21 * n, s, &host_out));
     }
     unsigned st = 0;
     RM_TRY(read_status(m, s, &st));  // synchronises the stream
-    if (st & rmk::kStatusQueue) return fail(RM_ECUDA, "the persistent queue ran out of slots");
     if (st & rmk::kStatusTimeout) return fail(RM_ETIMEOUT, "a device-side wait ran out of time");
     if (st & (rmk::kStatusOverflow | rmk::kStatusOverflowRay)) {
       RM_TRY(grow_bins(m, st, attempt));
@@ -1134,7 +1100,8 @@ struct LoopBufs {
   const float *sd, *rays;
   const uint8_t *sc;
   int4 *vis;
-  int *vis_count, *counts;
+  int *vis_count, *counts, *touched, *ray_dev;  // the first three one block, zero before an evaluation
+  int n_counters;
   unsigned char *bins;
   double *partial;
 };
@@ -1150,8 +1117,11 @@ void loop_arrays(Carver &cv, const rm_map *m, const rm_scan *scan, const TileGeo
   b->sc = on_device(scan->cls) ? scan->cls : cv.take<uint8_t>(P);
   b->rays = (in->model != RM_RAYTABLE || on_device(in->rays)) ? in->rays : cv.take<float>(3 * P);
   b->vis = cv.take<int4>((size_t)m->n_clusters * S);
-  b->vis_count = cv.take<int>(S);
-  b->counts = cv.take<int>((size_t)tg.ntiles * S);
+  b->n_counters = S * (1 + 2 * tg.ntiles);
+  b->vis_count = cv.take<int>(b->n_counters);
+  b->counts = b->vis_count + S;
+  b->touched = b->counts + (size_t)tg.ntiles * S;
+  b->ray_dev = cv.take<int>(2);
   b->bins = cv.take<unsigned char>((size_t)tg.ntiles * tg.cap * tg.rec_bytes * S);
   b->partial = cv.take<double>((size_t)tg.ntiles * rmk::kNumVals * S);
 }
@@ -1175,6 +1145,9 @@ WaveArgs loop_wave(const rm_map *m, const rm_scan *scan, const TileGeom &tg, int
   a.vis = b.vis;
   a.vis_count = b.vis_count;
   a.counts = b.counts;
+  a.touched = b.touched;
+  a.zbuf = m->zbuf;
+  a.ray_dev = a.cam.model == RM_RAYTABLE ? b.ray_dev : nullptr;
   a.bins = b.bins;
   a.partial = b.partial;
   a.status = m->d_status;
@@ -1185,9 +1158,12 @@ WaveArgs loop_wave(const rm_map *m, const rm_scan *scan, const TileGeom &tg, int
   return a;
 }
 
-rm_status loop_inputs(const rm_scan *scan, const double *init_pose, const LoopBufs &b, cudaStream_t s) {
+rm_status loop_inputs(rm_map *m, const rm_scan *scan, const double *init_pose, const WaveArgs &a, const LoopBufs &b,
+                      cudaStream_t s) {
   const rm_intrinsics *in = &scan->intr;
   const long long P = (long long)in->width * in->height;
+  m->h_progress[0] = m->h_progress[1] = 0;  // the last loop on this map has been waited for
+  RM_CK(cudaMemsetAsync(b.vis_count, 0, sizeof(int) * (size_t)b.n_counters, s));
   RM_CK(cudaMemcpyAsync(b.T0, init_pose, sizeof(double) * 16,
                         on_device(init_pose) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   if (b.rays != in->rays)
@@ -1195,6 +1171,38 @@ rm_status loop_inputs(const rm_scan *scan, const double *init_pose, const LoopBu
   if (b.sd != scan->depth)
     RM_CK(cudaMemcpyAsync((void *)b.sd, scan->depth, sizeof(float) * P, cudaMemcpyHostToDevice, s));
   if (b.sc != scan->cls) RM_CK(cudaMemcpyAsync((void *)b.sc, scan->cls, P, cudaMemcpyHostToDevice, s));
+  if (a.ray_dev) RM_CK(rmk::launch_ray_dev(a.cam, b.ray_dev, s));
+  return RM_OK;
+}
+
+// Before a loop's step `it` is launched: waits until the device is at most kLoopAhead steps behind,
+// and says whether the loop has ended. Default iteration limits are several times what a search
+// needs, and every step past its end would still launch its kernels to find that out.
+constexpr int kLoopAhead = 3;
+rm_status loop_ended(rm_map *m, int it, cudaStream_t s, bool *ended) {
+  const volatile int *h = m->h_progress;
+  for (unsigned spins = 0; it - h[0] > kLoopAhead && !h[1]; ++spins) {
+    if ((spins & 1023) != 1023) continue;
+    const cudaError_t e = cudaStreamQuery(s);
+    if (e == cudaSuccess) break;  // nothing pending: the count is as far as it goes
+    if (e != cudaErrorNotReady) RM_CK(e);
+  }
+  *ended = h[1] != 0;
+  return RM_OK;
+}
+
+// The evaluations and steps of a one-problem LM or ICP loop.
+rm_status loop_steps(rm_map *m, const WaveArgs &a, const rmk::BatchArgs &b, int mode, cudaStream_t s) {
+  m->zbuf_empty = false;  // until the last raster is on its way
+  for (int it = 0; it <= b.lm_iters; ++it) {
+    bool ended;
+    RM_TRY(loop_ended(m, it, s, &ended));
+    if (ended) break;
+    RM_TRY(wave(m, a, mode, s, false));
+    RM_CK(rmk::launch_step_one(a, b, s));
+    m->launches += 1;
+  }
+  m->zbuf_empty = true;
   return RM_OK;
 }
 
@@ -1337,6 +1345,7 @@ rm_status rm_map_create(const float *vertices, int64_t n_vertices, const int32_t
       (e = cudaMalloc(&m->d_planes, sizeof(float4) * hp.size())) != cudaSuccess ||
       (e = cudaMalloc(&m->d_status, sizeof(unsigned))) != cudaSuccess ||
       (e = cudaMallocHost(&m->h_status, sizeof(unsigned))) != cudaSuccess ||
+      (e = cudaMallocHost(&m->h_progress, 2 * sizeof(int))) != cudaSuccess ||
       (e = cudaMemcpy(m->d_v, hv.data(), sizeof(float4) * hv.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(m->d_faces, hf.data(), sizeof(int4) * hf.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
       (e = cudaMemcpy(m->d_planes, hp.data(), sizeof(float4) * hp.size(), cudaMemcpyHostToDevice)) != cudaSuccess ||
@@ -1372,6 +1381,7 @@ void rm_map_destroy(rm_map *m) {
   if (m->ev_join) cudaEventDestroy(m->ev_join);
   cudaFree(m->d_status);
   if (m->h_status) cudaFreeHost(m->h_status);
+  if (m->h_progress) cudaFreeHost(m->h_progress);
   for (auto &ev : m->ev_pending)
     for (auto e : ev) cudaEventDestroy(e);
   for (auto e : m->ev_free) cudaEventDestroy(e);
@@ -1746,6 +1756,7 @@ rm_status rm_align(rm_map *m, const rm_scan *scan, const double *init_pose,
   for (int attempt = 0;; ++attempt) {
     TileGeom tg = make_tiles(m, in);
     LoopBufs lb;
+    int *evals;
     auto arrays = [&](Carver &cv, rmk::LMState **st, long long **counts, long long **et, double **els,
                       double **grad, double **jtj) {
       *st = cv.take<rmk::LMState>(1);
@@ -1754,6 +1765,7 @@ rm_status rm_align(rm_map *m, const rm_scan *scan, const double *init_pose,
       *els = cv.take<double>(1);
       *grad = cv.take<double>(6);
       *jtj = cv.take<double>(21);
+      evals = cv.take<int>(1);
       loop_arrays(cv, m, scan, tg, 1, &lb);
     };
     rmk::LMState *d_st;
@@ -1762,6 +1774,7 @@ rm_status rm_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     Carver plan{nullptr};
     arrays(plan, &d_st, &d_counts, &d_etable, &d_els, &d_grad, &d_jtj);
     RM_TRY(ensure_arena(m, plan.off, s));
+    RM_TRY(ensure_zbuf(m, (size_t)in->width * in->height, s));
     m->batch_inputs_valid = false;
     Carver cv{m->arena};
     arrays(cv, &d_st, &d_counts, &d_etable, &d_els, &d_grad, &d_jtj);
@@ -1771,17 +1784,18 @@ rm_status rm_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     a.res_els = d_els;
     a.res_grad = d_grad;
     a.res_jtj = d_jtj;
-    RM_TRY(loop_inputs(scan, init_pose, lb, s));
-    rmk::LMArgs la{lm->lambda0, lm->lambda_up, lm->lambda_down, lm->step_tol,
-                   m->centre[0], m->centre[1], m->centre[2]};
-    RM_CK(rmk::launch_lm_init(d_st, lb.T0, la, lb.M, lb.skip, s));
-    RM_TRY(wave(m, a, rmk::kCostGrad, s));
-    RM_CK(rmk::launch_lm_take_initial(d_st, d_counts, d_els, d_grad, d_jtj, s));
-    for (int it = 0; it < lm->max_iters; ++it) {
-      RM_CK(rmk::launch_lm_propose(d_st, la, lb.M, lb.skip, s));
-      RM_TRY(wave(m, a, rmk::kCostGrad, s));
-      RM_CK(rmk::launch_lm_accept(d_st, la, d_counts, d_els, d_grad, d_jtj, lb.skip, s));
-    }
+    RM_TRY(loop_inputs(m, scan, init_pose, a, lb, s));
+    RM_CK(cudaMemsetAsync(evals, 0, sizeof(int), s));
+    rmk::BatchArgs b{};
+    b.lm = d_st;
+    b.evals = evals;
+    b.Ms = lb.M;
+    b.skip = lb.skip;
+    b.lmargs = {lm->lambda0, lm->lambda_up, lm->lambda_down, lm->step_tol, m->centre[0], m->centre[1], m->centre[2]};
+    b.lm_iters = lm->max_iters;
+    b.progress = m->h_progress;
+    RM_CK(rmk::launch_lm_init_batch(d_st, lb.T0, 1, b.lmargs, lb.M, lb.skip, s));
+    RM_TRY(loop_steps(m, a, b, rmk::kCostGrad, s));
     rmk::LMState hs;
     bool retry;
     RM_TRY(loop_finish(m, s, &hs, d_st, sizeof(hs), attempt, &retry));
@@ -1840,6 +1854,7 @@ rm_status rm_dfo_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     Carver plan{nullptr};
     arrays(plan, &d_st, &d_counts, &d_et, &d_els);
     RM_TRY(ensure_arena(m, plan.off, s));
+    RM_TRY(ensure_zbuf(m, (size_t)in->width * in->height * S, s));
     m->batch_inputs_valid = false;
     Carver cv{m->arena};
     arrays(cv, &d_st, &d_counts, &d_et, &d_els);
@@ -1847,7 +1862,7 @@ rm_status rm_dfo_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     a.res_counts = d_counts;
     a.res_etable = d_et;
     a.res_els = d_els;
-    RM_TRY(loop_inputs(scan, init_pose, lb, s));
+    RM_TRY(loop_inputs(m, scan, init_pose, a, lb, s));
     rmk::DfoArgs da{};
     da.nm_iters = dp->nm_iters;
     da.cd_iters = dp->cd_iters;
@@ -1872,11 +1887,16 @@ rm_status rm_dfo_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     // the origin and seven line searches per Powell iteration
     const int max_steps = dp->method == 1 ? 1 + 7 * dp->powell_iters + dp->cd_iters
                                           : 1 + 2 * dp->nm_iters + dp->cd_iters;
+    m->zbuf_empty = false;  // until the last raster is on its way
     for (int it = 0; it < max_steps; ++it) {
+      bool ended;
+      RM_TRY(loop_ended(m, it, s, &ended));
+      if (ended) break;
       RM_TRY(wave(m, a, rmk::kCost, s));
-      RM_CK(rmk::launch_dfo_step(d_st, da, d_et, lb.M, lb.skip, s));
+      RM_CK(rmk::launch_dfo_step(d_st, da, d_et, lb.M, lb.skip, lb.vis_count, lb.n_counters, m->h_progress, it, s));
       m->launches += 1;
     }
+    m->zbuf_empty = true;
     rmk::DfoState hs;
     bool retry;
     RM_TRY(loop_finish(m, s, &hs, d_st, sizeof(hs), attempt, &retry));
@@ -1920,6 +1940,7 @@ rm_status rm_icp_align(rm_map *m, const rm_scan *scan, const double *init_pose,
   for (int attempt = 0;; ++attempt) {
     TileGeom tg = make_tiles(m, in);
     LoopBufs lb;
+    int *evals;
     auto arrays = [&](Carver &cv, rmk::IcpState **st, long long **n, double **l1, double **e2,
                       double **g, double **H) {
       *st = cv.take<rmk::IcpState>(1);
@@ -1928,6 +1949,7 @@ rm_status rm_icp_align(rm_map *m, const rm_scan *scan, const double *init_pose,
       *e2 = cv.take<double>(1);
       *g = cv.take<double>(6);
       *H = cv.take<double>(21);
+      evals = cv.take<int>(1);
       loop_arrays(cv, m, scan, tg, 1, &lb);
     };
     rmk::IcpState *d_st;
@@ -1936,6 +1958,7 @@ rm_status rm_icp_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     Carver plan{nullptr};
     arrays(plan, &d_st, &d_n, &d_l1, &d_e2, &d_g, &d_H);
     RM_TRY(ensure_arena(m, plan.off, s));
+    RM_TRY(ensure_zbuf(m, (size_t)in->width * in->height, s));
     m->batch_inputs_valid = false;
     Carver cv{m->arena};
     arrays(cv, &d_st, &d_n, &d_l1, &d_e2, &d_g, &d_H);
@@ -1946,15 +1969,19 @@ rm_status rm_icp_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     a.res_els = d_e2;
     a.res_grad = d_g;
     a.res_jtj = d_H;
-    RM_TRY(loop_inputs(scan, init_pose, lb, s));
-    const rmk::IcpArgs ia{prm->step_tol, m->centre[0], m->centre[1], m->centre[2]};
-    RM_CK(rmk::launch_icp_init(d_st, lb.T0, ia, lb.M, lb.skip, s));
+    RM_TRY(loop_inputs(m, scan, init_pose, a, lb, s));
+    RM_CK(cudaMemsetAsync(evals, 0, sizeof(int), s));
+    rmk::BatchArgs b{};
+    b.icp = d_st;
+    b.evals = evals;
+    b.Ms = lb.M;
+    b.skip = lb.skip;
+    b.icpargs = {prm->step_tol, m->centre[0], m->centre[1], m->centre[2]};
+    b.lm_iters = prm->max_iters - 1;
+    b.progress = m->h_progress;
+    RM_CK(rmk::launch_icp_init_batch(d_st, lb.T0, 1, b.icpargs, lb.M, lb.skip, s));
     m->launches += 1;
-    for (int it = 0; it < prm->max_iters; ++it) {
-      RM_TRY(wave(m, a, rmk::kIcp, s));
-      RM_CK(rmk::launch_icp_step(d_st, ia, d_n, d_l1, d_g, d_H, lb.M, lb.skip, s));
-      m->launches += 1;
-    }
+    RM_TRY(loop_steps(m, a, b, rmk::kIcp, s));
     rmk::IcpState hs;
     bool retry;
     RM_TRY(loop_finish(m, s, &hs, d_st, sizeof(hs), attempt, &retry));

@@ -15,7 +15,7 @@
 //                 surface with its scan return and the point-to-plane terms (Sec. V)
 //   k_reduce      per pose: fixed-order sum of the per-tile partials
 // k_lm_* and k_icp_* take the Levenberg-Marquardt and ICP steps between evaluations.
-// k_persist runs the same phases for a batch of problems (and LM iterations) in one launch.
+// The k_*_batch kernels run the same phases for problems of different cameras and scans.
 #include <cfloat>
 #include <cmath>
 
@@ -510,126 +510,6 @@ __device__ __forceinline__ bool cut_piece(const DevCam &cam, const float4 *vc, u
 
 constexpr int kClusterMax = 64;  // vertices and triangles per cluster
 
-// One warp per visible cluster: its vertices are transformed and snapped once into shared
-// memory, then each lane sets up triangles (near-plane cut, culling, depth plane) and
-// appends them to the screen-tile bins.
-struct SetupSmem {
-  float M[12];
-  int nvis;
-  float4 s_vc[8][kClusterMax];
-  int2 s_vs[8][kClusterMax];
-  int s_gid[8][kClusterMax];
-  float4 s_dir[8][kClusterMax];  // ray table: unit direction and azimuth
-};
-
-template <int MODEL>
-__device__ __forceinline__ void setup_block(const WaveArgs &a, int q, int worker, int nworkers,
-                                            SetupSmem &sm) {
-  float4(*s_vc)[kClusterMax] = sm.s_vc;
-  int2(*s_vs)[kClusterMax] = sm.s_vs;
-  int(*s_gid)[kClusterMax] = sm.s_gid;
-  float4(*s_dir)[kClusterMax] = sm.s_dir;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) sm.nvis = ld_cg(&a.vis_count[q]);
-  load_m_block(a, q, sm.M);
-  float M[12];
-#pragma unroll
-  for (int k = 0; k < 12; ++k) M[k] = sm.M[k];
-  const int nvis = sm.nvis;
-  const int4 *vis = a.vis + (long long)q * a.n_clusters;
-  int *counts = a.counts + (long long)q * a.tg.ntiles;
-  unsigned char *bins = a.bins + (long long)q * a.tg.ntiles * a.tg.cap * a.tg.rec_bytes;
-  const int W = a.cam.W, H = a.cam.H;
-  const float near_m = a.cam.near_m;
-  constexpr bool raytable = MODEL != 0;  // one instantiation per camera model
-  for (int ci = worker * 8 + warp; ci < nvis; ci += nworkers * 8) {
-    float edge2;
-    const int4 info = cluster_info(__ldcg(&vis[ci]), edge2);
-    for (int k = lane; k < info.z; k += 32) {
-      const float4 v = a.cl_pos[info.x + k];
-      const int gv = __float_as_int(v.w);
-      const float3 c = xform(M, v.x, v.y, v.z);
-      int2 sv = make_int2(kSentinel, 1);  // behind the near plane
-      if (raytable) {
-        // the direction only bounds the rectangle: an approximate normalisation suffices
-        const float n2 = c.x * c.x + c.y * c.y + c.z * c.z;
-        const float inv = n2 > 0.0f ? rsqrtf(n2) : 0.0f;
-        s_dir[warp][k] = make_float4(c.x * inv, c.y * inv, c.z * inv, atan2f(c.x, c.z));
-      } else if (c.z >= near_m) {
-        int xi, yi;
-        sv = snap(a.cam, c.x, c.y, c.z, xi, yi) ? make_int2(xi, yi) : make_int2(kSentinel, 2);
-      }
-      s_vc[warp][k] = make_float4(c.x, c.y, c.z, v.w);
-      s_vs[warp][k] = sv;
-      s_gid[warp][k] = gv;
-    }
-    __syncwarp();
-    if (raytable) {
-      // every lane steps through the cluster's triangles together (warp-collective appends)
-      for (int k0 = 0; k0 < info.w; k0 += 32) {
-        const int k = k0 + lane;
-        RayRec rr;
-        int4 rect[2];
-        int nrect = 0;
-        if (k < info.w) {
-          const uchar4 t = a.cl_tris[info.y + k];
-          const unsigned id = (unsigned)a.cl_ids[info.y + k];
-          const int loc[3] = {t.x, t.y, t.z};
-          float3 v[3];
-          int gid[3];
-#pragma unroll
-          for (int m = 0; m < 3; ++m) {
-            const float4 p = s_vc[warp][loc[m]];
-            v[m] = make_float3(p.x, p.y, p.z);
-            gid[m] = s_gid[warp][loc[m]];
-          }
-          const int order = (gid[0] < gid[1] ? 1 : 0) | (gid[1] < gid[2] ? 2 : 0) | (gid[2] < gid[0] ? 4 : 0);
-          nrect = setup_ray(v, order, id, a.cam, rr, rect);
-        }
-        emit_ray_warp(nrect > 0, rr, rect[0], a, counts, bins);
-        if (__any_sync(0xffffffffu, nrect > 1)) emit_ray_warp(nrect > 1, rr, rect[1], a, counts, bins);
-      }
-      __syncwarp();
-      continue;
-    }
-    // pinhole: every lane of the warp steps through the cluster's triangles together, so the
-    // (at most two) pieces of a lane's triangle are appended by the warp-collective emitter
-    for (int k0 = 0; k0 < info.w; k0 += 32) {
-      const int k = k0 + lane;
-      bool va = false, vb = false;
-      int sx[4] = {0, 0, 0, 0}, sy[4] = {0, 0, 0, 0};
-      float A = 0.0f, B = 0.0f, C = 0.0f;
-      unsigned id = 0;
-      if (k < info.w) {
-        const uchar4 t = a.cl_tris[info.y + k];
-        id = (unsigned)a.cl_ids[info.y + k];
-        const int2 s0 = s_vs[warp][t.x], s1 = s_vs[warp][t.y], s2 = s_vs[warp][t.z];
-        if (s0.x != kSentinel && s1.x != kSentinel && s2.x != kSentinel) {
-          // all three in front of the near plane and inside the guard band
-          const int xmin = min(s0.x, min(s1.x, s2.x)), xmax = max(s0.x, max(s1.x, s2.x));
-          const int ymin = min(s0.y, min(s1.y, s2.y)), ymax = max(s0.y, max(s1.y, s2.y));
-          if (max((xmin + 127) >> 8, 0) <= min((xmax - 128) >> 8, W - 1) &&
-              max((ymin + 127) >> 8, 0) <= min((ymax - 128) >> 8, H - 1)) {
-            const float4 p0 = s_vc[warp][t.x], p1 = s_vc[warp][t.y], p2 = s_vc[warp][t.z];
-            const PlaneN pl = plane_n(make_float3(p0.x, p0.y, p0.z), make_float3(p1.x, p1.y, p1.z),
-                                      make_float3(p2.x, p2.y, p2.z));
-            fold_pinhole(a.cam, pl, A, B, C);
-            sx[0] = s0.x; sy[0] = s0.y; sx[1] = s1.x; sy[1] = s1.y; sx[2] = s2.x; sy[2] = s2.y;
-            va = true;
-          }
-        } else {
-          // slow path: near-plane cut and/or guard band
-          va = cut_piece(a.cam, s_vc[warp], t, sx, sy, A, B, C, vb);
-        }
-      }
-      emit_piece_warp(va, sx[0], sy[0], sx[1], sy[1], sx[2], sy[2], A, B, C, id, a, counts, bins);
-      if (__any_sync(0xffffffffu, vb))
-        emit_piece_warp(vb, sx[0], sy[0], sx[2], sy[2], sx[3], sy[3], A, B, C, id, a, counts, bins);
-    }
-    __syncwarp();
-  }
-}
-
 // (float)i + 0.5f for 0 <= i < 2^23 without the conversion pipe: 2^23 + i is exact in the
 // mantissa, and subtracting 2^23 - 0.5 (representable) leaves i + 0.5 exactly.
 __device__ __forceinline__ float px_centre(int i) {
@@ -765,10 +645,8 @@ __device__ __forceinline__ void direct_pixels(const DevCam &cam, const float4 *r
   });
 }
 
-__global__ void __launch_bounds__(kPinSetupThreads, 7) k_setup_pin(WaveArgs a) {
-  __shared__ PinSetupSmem sm;
-  if (skipped(a)) return;
-  const int q = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void setup_pin(const WaveArgs &a, int q, PinSetupSmem &sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float4 *vc = sm.vc[warp];
   int2 *vs = sm.vs[warp];
   float4 *ring = sm.ring[warp];
@@ -916,6 +794,11 @@ __global__ void __launch_bounds__(kPinSetupThreads, 7) k_setup_pin(WaveArgs a) {
     if (last) break;
     __syncwarp();
   }
+}
+
+__global__ void __launch_bounds__(kPinSetupThreads, 7) k_setup_pin(WaveArgs a) {
+  __shared__ PinSetupSmem sm;
+  if (!skipped(a)) setup_pin(a, blockIdx.y, sm);
 }
 
 // ------------------------------------------------------------------ ray-table setup
@@ -1088,10 +971,8 @@ __device__ __forceinline__ void direct_rays(const DevCam &cam, const float4 *rin
   });
 }
 
-__global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
-  __shared__ RaySetupSmem sm;
-  if (skipped(a)) return;
-  const int q = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void setup_ray_table(const WaveArgs &a, int q, RaySetupSmem &sm) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float4 *vc = sm.vc[warp];
   float2 *uv = sm.uv[warp];
   float4 *ring = sm.ring[warp];
@@ -1260,6 +1141,11 @@ __global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
     if (last) break;
     __syncwarp();
   }
+}
+
+__global__ void __launch_bounds__(kRaySetupThreads, 7) k_setup_ray(WaveArgs a) {
+  __shared__ RaySetupSmem sm;
+  if (!skipped(a)) setup_ray_table(a, blockIdx.y, sm);
 }
 
 // ------------------------------------------------------------------ raster + epilogue
@@ -1560,10 +1446,6 @@ __device__ __forceinline__ bool raster_tile_ray(unsigned long long *zk, RayRec *
   }
   return true;
 }
-
-#ifndef RM_PERSIST_MIN_BLOCKS
-#define RM_PERSIST_MIN_BLOCKS 4
-#endif
 
 #ifndef RM_RASTER_MIN_BLOCKS
 #define RM_RASTER_MIN_BLOCKS 5  // resident CTAs per SM the register budget is sized for (48 registers)
@@ -2027,8 +1909,17 @@ static cudaError_t launch_raster(const WaveArgs &a, int mode, cudaStream_t s) {
   return a.cam.model == 0 ? launch_raster_m<TW, TH, 0>(a, mode, s) : launch_raster_m<TW, TH, 1>(a, mode, s);
 }
 
+// Setup CTAs (four warps) per pose: 32 in a large wave, so that each warp sets up several clusters
+// and the next wave's setup (on the other stream) takes few enough SMs to run beside this wave's
+// raster; waves of few poses (single-pose alignment) get up to about twelve CTAs per SM in total,
+// so that their setup spreads over the GPU.
+static int setup_blocks(int n_clusters, int n_poses) {
+  const int per_pose = max(16, (kSetupCtasPerGpu + n_poses - 1) / n_poses);
+  return 2 * min(max(n_clusters / 64, 1), per_pose);
+}
+
 cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t *ev,
-                        bool zero_counters) {
+                        bool zero_counters, bool reduce) {
   cudaError_t e;
   if (zero_counters) {
     e = cudaMemsetAsync(a.counts, 0, sizeof(int) * (size_t)a.tg.ntiles * a.n_poses, s);
@@ -2044,15 +1935,9 @@ cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t
   }
   if (ev && (e = cudaEventRecord(ev[1], s)) != cudaSuccess) return e;
   if (a.n_clusters > 0) {
-    // 16 CTAs per pose in a large wave: each warp then sets up several clusters, and the next
-    // wave's setup (on the other stream) takes few enough SMs to run beside this wave's
-    // raster; waves of few poses (single-pose alignment) get up to about six CTAs per SM in
-    // total so that their setup spreads over the GPU
-    const int per_pose = max(16, (kSetupCtasPerGpu + a.n_poses - 1) / a.n_poses);
-    const int blocks = min(max(a.n_clusters / 64, 1), per_pose);
-    dim3 gs(blocks, a.n_poses);
-    if (a.cam.model == 0) k_setup_pin<<<dim3(2 * blocks, a.n_poses), kPinSetupThreads, 0, s>>>(a);
-    else k_setup_ray<<<dim3(2 * blocks, a.n_poses), kRaySetupThreads, 0, s>>>(a);
+    const dim3 gs(setup_blocks(a.n_clusters, a.n_poses), a.n_poses);
+    if (a.cam.model == 0) k_setup_pin<<<gs, kPinSetupThreads, 0, s>>>(a);
+    else k_setup_ray<<<gs, kRaySetupThreads, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if (ev && (e = cudaEventRecord(ev[2], s)) != cudaSuccess) return e;
@@ -2062,7 +1947,7 @@ cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t
   else e = launch_raster<16, 16>(a, mode, s);
   if (e != cudaSuccess) return e;
   if (ev && (e = cudaEventRecord(ev[3], s)) != cudaSuccess) return e;
-  if (mode != kRender) {
+  if (reduce && mode != kRender) {
     k_reduce<<<a.n_poses, 256, 0, s>>>(a);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -2070,8 +1955,8 @@ cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t
   return cudaSuccess;
 }
 
-int wave_kernel_launches(const WaveArgs &a, int mode) {
-  return 2 * (a.n_clusters > 0) + 1 + (mode != kRender);
+int wave_kernel_launches(const WaveArgs &a, int mode, bool reduce) {
+  return 2 * (a.n_clusters > 0) + 1 + (reduce && mode != kRender);
 }
 
 // ------------------------------------------------------------------ Levenberg-Marquardt
@@ -2331,24 +2216,6 @@ __device__ void lm_init_dev(LMState &st, const double *T0, const LMArgs &a, floa
   *skip = 0;
 }
 
-__global__ void k_lm_init(LMState *st, const double *T0, LMArgs a, float *M, int *skip) {
-  lm_init_dev(*st, T0, a, M, skip);
-}
-
-__global__ void k_lm_take_initial(LMState *st, const long long *counts, const double *els,
-                                  const double *grad, const double *jtj) {
-  lm_take_initial_dev(*st, counts, els, grad, jtj);
-}
-
-__global__ void k_lm_propose(LMState *st, LMArgs a, float *M, int *skip) {
-  lm_propose_dev(*st, a, M, skip);
-}
-
-__global__ void k_lm_accept(LMState *st, LMArgs a, const long long *counts, const double *els,
-                            const double *grad, const double *jtj, int *skip) {
-  lm_accept_dev(*st, a, counts, els, grad, jtj, *skip != 0);
-}
-
 // ------------------------------------------------------------------ point-to-plane ICP
 
 __device__ void icp_init_dev(IcpState &st, const double *T0, const IcpArgs &a, float *M, int *skip) {
@@ -2358,10 +2225,6 @@ __device__ void icp_init_dev(IcpState &st, const double *T0, const IcpArgs &a, f
   st.iters = st.converged = st.done = st.evals = 0;
   pose_to_m(T0, a.cx, a.cy, a.cz, M);
   *skip = 0;
-}
-
-__global__ void k_icp_init(IcpState *st, const double *T0, IcpArgs a, float *M, int *skip) {
-  icp_init_dev(*st, T0, a, M, skip);
 }
 
 // Gauss-Newton step of point-to-plane ICP: J^T J dx = -J^T e (Cholesky, no damping), then
@@ -2399,11 +2262,6 @@ __device__ __noinline__ void icp_step_dev(IcpState &s, const IcpArgs &a, const l
   *skip = 0;
 }
 
-__global__ void k_icp_step(IcpState *st, IcpArgs a, const long long *n, const double *l1,
-                           const double *g, const double *H, float *M, int *skip) {
-  icp_step_dev(*st, a, n, l1, g, H, M, skip);
-}
-
 __global__ void k_icp_init_batch(IcpState *st, const double *T0, int n, IcpArgs a, float *Ms,
                                  int *skip) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2417,17 +2275,12 @@ cudaError_t launch_icp_init_batch(IcpState *st, const double *T0, int n, const I
   return cudaGetLastError();
 }
 
-cudaError_t launch_icp_init(IcpState *st, const double *T0, const IcpArgs &a, float *M,
-                            int *skip, cudaStream_t s) {
-  k_icp_init<<<1, 1, 0, s>>>(st, T0, a, M, skip);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_icp_step(IcpState *st, const IcpArgs &a, const long long *n,
-                            const double *l1, const double *g, const double *H, float *M,
-                            int *skip, cudaStream_t s) {
-  k_icp_step<<<1, 1, 0, s>>>(st, a, n, l1, g, H, M, skip);
-  return cudaGetLastError();
+// Tells a host that polls it how far a loop is: evaluations done, and whether it has ended.
+__device__ __forceinline__ void report_progress(int *progress, int evals, int done) {
+  if (!progress) return;
+  *reinterpret_cast<volatile int *>(progress + 1) = done;
+  __threadfence_system();
+  *reinterpret_cast<volatile int *>(progress) = evals;
 }
 
 // ------------------------------------------------------------------ derivative-free search
@@ -2565,16 +2418,16 @@ __device__ void powell_step(DfoState &s, const DfoArgs &a, const double *fc) {
   powell_line(s, s.disp, 1.0);
 }
 
-__device__ void dfo_write_candidates(DfoState &s, const DfoArgs &a, float *Ms) {
-  for (int m = 0; m < kDfoSlots; ++m) {
-    double T[16];
-    se3_right_dev(s.T0, s.cand[m < s.n_cand ? m : 0], T);
-    pose_to_m(T, a.cx, a.cy, a.cz, Ms + 12 * m);
-  }
+// The candidates' matrices, one thread each (their FP64 retractions are a serial chain).
+__device__ __forceinline__ void dfo_write_candidates(DfoState &s, const DfoArgs &a, float *Ms) {
+  const int m = threadIdx.x;
+  if (m >= kDfoSlots) return;
+  double T[16];
+  se3_right_dev(s.T0, s.cand[m < s.n_cand ? m : 0], T);
+  pose_to_m(T, a.cx, a.cy, a.cz, Ms + 12 * m);
 }
 
-__global__ void k_dfo_init(DfoState *st, const double *T0, DfoArgs a, float *Ms, int *skip) {
-  DfoState &s = *st;
+__device__ void dfo_start(DfoState &s, const double *T0, const DfoArgs &a) {
   for (int k = 0; k < 16; ++k) s.T0[k] = T0[k];
   s.evals = s.nm_iters = s.nm_shrinks = s.cd_iters = s.converged = s.shrink_best = 0;
   s.powell_iters = 0;
@@ -2585,24 +2438,25 @@ __global__ void k_dfo_init(DfoState *st, const double *T0, DfoArgs a, float *Ms,
     s.ps = a.powell_step;
     s.n_cand = 1;
     s.phase = 5;
-    dfo_write_candidates(s, a, Ms);
-    *skip = 0;
     return;
   }
   for (int i = 0; i < 7; ++i)
     for (int k = 0; k < 6; ++k) s.cand[i][k] = (i >= 1 && k == i - 1) ? a.nm_step * a.scale[k] : 0.0;
   s.n_cand = 7;
   s.phase = 0;
-  dfo_write_candidates(s, a, Ms);
-  *skip = 0;
 }
 
-__global__ void k_dfo_step(DfoState *st, DfoArgs a, const long long *et, float *Ms, int *skip) {
-  DfoState &s = *st;
-  if (s.phase == 4) {
-    *skip = 1;
-    return;
+__global__ void k_dfo_init(DfoState *st, const double *T0, DfoArgs a, float *Ms, int *skip) {
+  if (threadIdx.x == 0) {
+    dfo_start(*st, T0, a);
+    *skip = 0;
   }
+  __syncthreads();
+  dfo_write_candidates(*st, a, Ms);
+}
+
+// Takes the costs of the pending candidates and plans the next ones.
+__device__ void dfo_advance(DfoState &s, const DfoArgs &a, const long long *et) {
   double fc[kDfoSlots];
   for (int m = 0; m < s.n_cand; ++m) fc[m] = (double)et[m];
   s.evals += s.n_cand;
@@ -2668,375 +2522,39 @@ __global__ void k_dfo_step(DfoState *st, DfoArgs a, const long long *et, float *
     }
     dfo_next_cd(s, a);
   }
-  if (s.phase == 4) {
-    *skip = 1;
-    return;
+}
+
+// One step of the search, and the counters of the next evaluation's lists and bins to zero.
+__global__ void __launch_bounds__(256) k_dfo_step(DfoState *st, DfoArgs a, const long long *et, float *Ms, int *skip,
+                                                  int *counters, int n_counters, int *progress, int step) {
+  if (threadIdx.x == 0) {
+    if (st->phase != 4) dfo_advance(*st, a, et);
+    *skip = st->phase == 4;
   }
-  dfo_write_candidates(s, a, Ms);
-  *skip = 0;
+  for (int k = threadIdx.x; k < n_counters; k += blockDim.x) counters[k] = 0;
+  __syncthreads();
+  if (st->phase != 4) dfo_write_candidates(*st, a, Ms);
+  if (threadIdx.x == 0) report_progress(progress, step + 1, st->phase == 4);
 }
 
 cudaError_t launch_dfo_init(DfoState *st, const double *T0, const DfoArgs &a, float *Ms,
                             int *skip, cudaStream_t s) {
-  k_dfo_init<<<1, 1, 0, s>>>(st, T0, a, Ms, skip);
+  k_dfo_init<<<1, 32, 0, s>>>(st, T0, a, Ms, skip);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dfo_step(DfoState *st, const DfoArgs &a, const long long *e_table, float *Ms,
-                            int *skip, cudaStream_t s) {
-  k_dfo_step<<<1, 1, 0, s>>>(st, a, e_table, Ms, skip);
+cudaError_t launch_dfo_step(DfoState *st, const DfoArgs &a, const long long *e_table, float *Ms, int *skip,
+                            int *counters, int n_counters, int *progress, int step, cudaStream_t s) {
+  k_dfo_step<<<1, 256, 0, s>>>(st, a, e_table, Ms, skip, counters, n_counters, progress, step);
   return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ persistent batch kernel
+// ------------------------------------------------------------------ batches of problems
 
 __global__ void k_lm_init_batch(LMState *st, const double *T0, int n, LMArgs a, float *Ms,
                                 int *skip) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k < n) lm_init_dev(st[k], T0 + 16 * (long long)k, a, Ms + 12 * (long long)k, skip + k);
-}
-
-// Phase bodies of the persistent kernel, each compiled out of line so that its register
-// allocation is its own (as in the per-phase kernels) rather than the union of all phases.
-__device__ __noinline__ void persist_cull(const WaveArgs *__restrict__ pa, int item, float *sM) {
-  const WaveArgs &a = *pa;
-  const int c1 = min((item + 1) * kPersistCull, (a.n_clusters + 255) / 256);
-  for (int c = item * kPersistCull; c < c1; ++c) {
-    cull_block(a, 0, c, sM);
-    __syncthreads();
-  }
-}
-
-template <int MODEL>
-__device__ __noinline__ void persist_setup(const WaveArgs *__restrict__ pa, int worker, int nworkers,
-                                           SetupSmem &sm) {
-  const WaveArgs &a = *pa;
-  setup_block<MODEL>(a, 0, worker, nworkers, sm);
-}
-
-template <int MODEL>
-__device__ __noinline__ void persist_raster(
-    const WaveArgs *__restrict__ pa, int item, RasterSmem<kPersistTileW[MODEL] * kPersistTileH[MODEL], MODEL> &sm) {
-  const WaveArgs &a = *pa;
-  const int t1 = min((item + 1) * kPersistTiles[MODEL], a.tg.ntiles);
-  for (int t = item * kPersistTiles[MODEL]; t < t1; ++t) {
-    raster_block<kPersistTileW[MODEL], kPersistTileH[MODEL], kCostGrad, MODEL>(a, t, 0, sm);
-    __syncthreads();
-  }
-}
-
-template <int MODEL>
-__device__ __noinline__ void persist_raster_icp(
-    const WaveArgs *__restrict__ pa, int item, RasterSmem<kPersistTileW[MODEL] * kPersistTileH[MODEL], MODEL> &sm) {
-  const WaveArgs &a = *pa;
-  const int t1 = min((item + 1) * kPersistTiles[MODEL], a.tg.ntiles);
-  for (int t = item * kPersistTiles[MODEL]; t < t1; ++t) {
-    if (a.vnormals) raster_block<kPersistTileW[MODEL], kPersistTileH[MODEL], kIcpVn, MODEL>(a, t, 0, sm);
-    else raster_block<kPersistTileW[MODEL], kPersistTileH[MODEL], kIcp, MODEL>(a, t, 0, sm);
-    __syncthreads();
-  }
-}
-
-__device__ __noinline__ void persist_reduce(const WaveArgs *__restrict__ pa, double *vals) {
-  const WaveArgs &a = *pa;
-  reduce_block(a, 0, vals);
-}
-
-// Copies an LM state with L2 loads (another SM may have written it during this kernel).
-__device__ __noinline__ void lm_load_cg(const LMState *src, LMState &dst) {
-  const long long *s = reinterpret_cast<const long long *>(src);
-  long long *d = reinterpret_cast<long long *>(&dst);
-  for (int k = 0; k < (int)(sizeof(LMState) / 8); ++k) d[k] = __ldcg(s + k);
-}
-
-// A load with acquire semantics at GPU scope: later loads see what the writer released.
-__device__ __forceinline__ long long ld_acquire_gpu(const long long *p) {
-  long long v;
-  asm volatile("ld.acquire.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-
-// Orders this thread's earlier memory operations before its later ones at GPU scope (with a
-// relaxed write after it: a release; with a relaxed read before it: an acquire).
-__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
-
-__device__ __forceinline__ int4 unpack_item(long long v) {
-  return make_int4((int)(v >> 40), (int)(v >> 21) & 3, (int)v & ((1 << kItemIndexBits) - 1),
-                   (int)(v >> 23) & ((1 << kItemEvalBits) - 1));
-}
-
-// Claims the next slot of a queue that looks non-empty (one atomic add), or returns -1. Two
-// CTAs racing for its last item can both claim; the later one then waits for the queue's next
-// publication, or for the end of the batch.
-__device__ __forceinline__ int claim_slot(int *head, const int *tail) {
-  if (*(volatile const int *)head >= *(volatile const int *)tail) return -1;
-  return atomicAdd(head, 1);
-}
-
-// One launch runs every phase of every problem of a batch (and, with LM, every iteration).
-// Items enter a ready queue only once they can run: the launch starts with the evaluation-0
-// cull items of every problem, and the CTA that completes the last item of a problem's phase
-// appends the next phase (cull -> setup -> raster -> reduce and LM step -> the next
-// evaluation's cull). The number of setup items follows the visible-cluster count of that
-// evaluation. Raster and reduce items go to a queue that is served first, so problems that
-// have reached their raster finish their evaluation before new ones start theirs. A CTA takes
-// only slots that have been reserved by a publisher (whose write is then at most a few
-// instructions away) and exits once every problem has finished; with nothing to take it
-// sleeps and retries (bounded).
-// Thread 0 of a CTA: claims the next ready item of the batch's queues into *s_item (x < 0:
-// every problem has finished) and sets *s_abort when a wait ran out of its budget.
-__device__ __forceinline__ void persist_claim(const BatchArgs &b, int4 *s_item, int *s_abort) {
-  int4 item = make_int4(-1, 0, 0, 0);
-  int abort = 0;
-  const long long t0 = clock64();
-  unsigned ns = 32;
-  for (;;) {
-    // a claim past a queue's capacity (racing claims at its very end) holds no slot
-    int slot = claim_slot(b.qctl + 0, b.qctl + 1);
-    if (slot >= b.cap[0]) slot = -1;
-    if (slot < 0) {
-      slot = claim_slot(b.qctl + 2, b.qctl + 3);
-      slot = slot >= b.cap[1] ? -1 : (slot >= 0 ? slot + b.cap[0] : -1);
-    }
-    if (slot >= 0) {
-      long long x;
-      bool finished = false;
-      while ((x = ld_acquire_gpu(b.items + slot)) < 0) {
-        if (*(volatile const int *)(b.qctl + 4) >= b.n_problems) {  // nothing more will come
-          finished = true;
-          break;
-        }
-        if (clock64() - t0 > b.spin_limit) break;
-        __nanosleep(64);
-      }
-      if (finished) break;
-      if (x < 0) {
-        atomicOr(b.status, kStatusTimeout);
-        abort = 1;
-        break;
-      }
-      item = unpack_item(x);
-      break;
-    }
-    if (*(volatile const int *)(b.qctl + 4) >= b.n_problems) break;  // all finished
-    if (clock64() - t0 > b.spin_limit) {
-      atomicOr(b.status, kStatusTimeout);
-      abort = 1;
-      break;
-    }
-    __nanosleep(ns);
-    if (ns < 1024) ns *= 2;
-  }
-  *s_item = item;
-  *s_abort = abort;
-}
-
-// Thread 0 of a CTA, after `item` is done: counts it, and when it was its problem's last item
-// of a phase, reserves the next phase's slots (the setup phase sized by *vis_count, the
-// problem's visible clusters, clusters_per_item to an item). Returns (phase, count, first
-// slot, evaluation); count 0: none.
-__device__ __forceinline__ int4 persist_complete(const BatchArgs &b, int4 item, const int *vis_count,
-                                                 int clusters_per_item) {
-  fence_acq_rel_gpu();  // the CTA's results (after its barrier) before the count
-  const int p = item.x, ph = item.y, it = item.w;
-  int4 eq = make_int4(0, 0, -1, it);  // phase, count, queue, evaluation
-  if (ph < 3) {
-    const int c = atomicAdd(b.done + 4 * p + ph, 1) + 1;
-    if (c == __ldcg(b.need + 3 * p + ph)) {
-      if (ph == 0) {
-        // all cull items are in: size the setup phase by the visible clusters
-        const int nv = __ldcg(vis_count);
-        const int nsetup = max(1, (nv + clusters_per_item - 1) / clusters_per_item);
-        b.need[3 * p + 1] = nsetup;
-        eq = make_int4(1, nsetup, 1, it);
-      } else if (ph == 1) {
-        eq = make_int4(2, b.need[3 * p + 2], 0, it);
-      } else {
-        eq = make_int4(3, 1, 0, it);
-      }
-    }
-  } else if ((b.lm || b.icp) && it < b.lm_iters) {
-    b.done[4 * p + 0] = 0;
-    b.done[4 * p + 1] = 0;
-    b.done[4 * p + 2] = 0;
-    eq = make_int4(0, b.need[3 * p], 1, it + 1);
-  } else {
-    atomicAdd(b.qctl + 4, 1);  // the problem is finished
-  }
-  if (eq.y > 0) {
-    const int q = eq.z;
-    const int first = atomicAdd(b.qctl + 2 * q + 1, eq.y);
-    if (first + eq.y > b.cap[q]) atomicOr(b.status, kStatusQueue);  // cannot happen
-    eq.z = (q == 0 ? 0 : b.cap[0]) + first;
-    eq.y = max(0, min(eq.y, b.cap[q] - first));
-  }
-  return eq;
-}
-
-// All threads of a CTA: publish the reserved successor slots, each with one 64-bit write after
-// a fence (which also orders what thread 0 observed of the completion counts).
-__device__ __forceinline__ void persist_publish(const BatchArgs &b, int4 eq, int problem) {
-  if (eq.y > 0) {
-    fence_acq_rel_gpu();
-    __syncthreads();
-    for (int k = threadIdx.x; k < eq.y; k += blockDim.x)
-      atomicExch(reinterpret_cast<unsigned long long *>(b.items + eq.z + k),
-                 (unsigned long long)pack_item(problem, eq.x, k, eq.w));
-  }
-}
-
-__global__ void __launch_bounds__(kThreads, RM_PERSIST_MIN_BLOCKS) k_persist(BatchArgs b) {
-  union PersistSmem {
-    RasterSmem<kPersistTileW[0] * kPersistTileH[0], 0> r0;
-    RasterSmem<kPersistTileW[1] * kPersistTileH[1], 1> r1;
-    SetupSmem su;
-    double vals[kNumVals];
-  };
-  __shared__ PersistSmem u;
-  __shared__ float s_M[12];
-  __shared__ int4 s_item;
-  __shared__ int4 s_enq;       // successors to publish: phase, count, first slot, evaluation
-  __shared__ int s_abort;
-  for (;;) {
-    if (threadIdx.x == 0) persist_claim(b, &s_item, &s_abort);
-    __syncthreads();
-    const int4 item = s_item;
-    if (item.x < 0 || s_abort) break;
-    // the problem's argument block: written before the launch and read-only during it, so
-    // the phases read it in place through the read-only data path
-    const WaveArgs *__restrict__ pa = b.probs + item.x;
-    const WaveArgs &a = *pa;
-    const bool skip = skipped(a);
-    if (!skip) {
-      switch (item.y) {
-        case 0: persist_cull(pa, item.z, s_M); break;
-        case 1:
-          if (a.cam.model == 0) persist_setup<0>(pa, item.z, __ldcg(b.need + 3 * item.x + 1), u.su);
-          else persist_setup<1>(pa, item.z, __ldcg(b.need + 3 * item.x + 1), u.su);
-          break;
-        case 2:
-          if (b.icp) {
-            if (a.cam.model == 0) persist_raster_icp<0>(pa, item.z, u.r0);
-            else persist_raster_icp<1>(pa, item.z, u.r1);
-          } else {
-            if (a.cam.model == 0) persist_raster<0>(pa, item.z, u.r0);
-            else persist_raster<1>(pa, item.z, u.r1);
-          }
-          break;
-        default: persist_reduce(pa, u.vals); break;
-      }
-    }
-    if (item.y == 3 && b.icp) {
-      // ICP: every evaluation is followed by a Gauss-Newton step (a no-op once done)
-      __syncthreads();
-      const int p = item.x, it = item.w;
-      if (threadIdx.x == 0) {
-        IcpState st = b.icp[p];
-        icp_step_dev(st, b.icpargs, a.res_n, a.res_l1, a.res_grad, a.res_jtj, b.Ms + 12 * (long long)p,
-                     b.skip + p);
-        b.icp[p] = st;
-      }
-      if (it < b.lm_iters) {
-        for (int t = threadIdx.x; t < a.tg.ntiles; t += blockDim.x) a.counts[t] = 0;
-        if (threadIdx.x == 0) a.vis_count[0] = 0;
-      }
-    }
-    if (item.y == 3 && b.lm) {
-      __syncthreads();
-      const int p = item.x, it = item.w;
-      if (threadIdx.x == 0) {
-        LMState st;
-        lm_load_cg(b.lm + p, st);
-        if (it == 0) lm_take_initial_dev(st, a.res_counts, a.res_els, a.res_grad, a.res_jtj);
-        else lm_accept_dev(st, b.lmargs, a.res_counts, a.res_els, a.res_grad, a.res_jtj, skip);
-        if (it < b.lm_iters) lm_propose_dev(st, b.lmargs, b.Ms + 12 * (long long)p, b.skip + p);
-        b.lm[p] = st;
-      }
-      if (it < b.lm_iters) {  // the next evaluation starts from empty lists and bins
-        for (int t = threadIdx.x; t < a.tg.ntiles; t += blockDim.x) a.counts[t] = 0;
-        if (threadIdx.x == 0) a.vis_count[0] = 0;
-      }
-    }
-    __syncthreads();
-    // completion; the last item of the problem's phase publishes the successors
-    if (threadIdx.x == 0) s_enq = persist_complete(b, item, a.vis_count, setup_clusters(a.cam.model));
-    __syncthreads();
-    persist_publish(b, s_enq, item.x);
-  }
-}
-
-// The persistent kernel for a homogeneous batch (every problem the same camera, scan and
-// parameters, a plain evaluation): the problems are the poses of one wave, whose arguments
-// are a kernel parameter, so the phases (inlined) read them as the per-wave kernels do and the
-// kernel fits the per-wave raster's register budget. Same queue, items and results as
-// k_persist.
-#ifndef RM_PERSIST_WAVE_MIN_BLOCKS
-#define RM_PERSIST_WAVE_MIN_BLOCKS 5
-#endif
-
-template <int MODEL>
-__global__ void __launch_bounds__(kThreads, MODEL == 0 ? RM_PERSIST_WAVE_MIN_BLOCKS : 4)
-    k_persist_wave(BatchArgs b, WaveArgs w) {
-  constexpr int TW = kPersistTileW[MODEL], TH = kPersistTileH[MODEL];
-  union PersistWaveSmem {
-    RasterSmem<TW * TH, MODEL> r;
-    SetupSmem su;
-    double vals[kNumVals];
-  };
-  __shared__ PersistWaveSmem u;
-  __shared__ float s_M[12];
-  __shared__ int4 s_item;
-  __shared__ int4 s_enq;
-  __shared__ int s_abort;
-  for (;;) {
-    if (threadIdx.x == 0) persist_claim(b, &s_item, &s_abort);
-    __syncthreads();
-    const int4 item = s_item;
-    if (item.x < 0 || s_abort) break;
-    const int q = item.x;  // the problem is pose q of the wave
-    switch (item.y) {
-      case 0: {
-        const int c1 = min((item.z + 1) * kPersistCull, (w.n_clusters + 255) / 256);
-        for (int c = item.z * kPersistCull; c < c1; ++c) {
-          cull_block(w, q, c, s_M);
-          __syncthreads();
-        }
-        break;
-      }
-      case 1: setup_block<MODEL>(w, q, item.z, __ldcg(b.need + 3 * q + 1), u.su); break;
-      case 2: {
-        const int t1 = min((item.z + 1) * kPersistTiles[MODEL], w.tg.ntiles);
-        for (int t = item.z * kPersistTiles[MODEL]; t < t1; ++t) {
-          raster_block<TW, TH, kCostGrad, MODEL>(w, t, q, u.r);
-          __syncthreads();
-        }
-        break;
-      }
-      default: reduce_block(w, q, u.vals); break;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s_enq = persist_complete(b, item, w.vis_count + q, setup_clusters(MODEL));
-    __syncthreads();
-    persist_publish(b, s_enq, item.x);
-  }
-}
-
-__global__ void k_queue_init(long long *items, int n_slots, int first_low, int n_problems,
-                             int cull_items, int *qctl) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int n0 = n_problems * cull_items;
-  if (k < n_slots) {
-    const int c = k - first_low;
-    items[k] = c >= 0 && c < n0 ? pack_item(c / cull_items, 0, c % cull_items, 0) : -1ll;
-  }
-  if (k == 0) qctl[3] = n0;
-}
-
-cudaError_t launch_queue_init(long long *items, int n_slots, int first_low, int n_problems,
-                              int cull_items, int *qctl, cudaStream_t s) {
-  k_queue_init<<<(n_slots + 255) / 256, 256, 0, s>>>(items, n_slots, first_low, n_problems,
-                                                     cull_items, qctl);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_lm_init_batch(LMState *st, const double *T0, int n, const LMArgs &a,
@@ -3046,51 +2564,120 @@ cudaError_t launch_lm_init_batch(LMState *st, const double *T0, int n, const LMA
   return cudaGetLastError();
 }
 
-cudaError_t launch_persist(const BatchArgs &b, int grid, cudaStream_t s) {
-  k_persist<<<grid, kThreads, 0, s>>>(b);
+// The phases of one evaluation of every problem of a batch: blockIdx.y is the problem, whose argument
+// block (written before the launch, read-only during it) is read in place. Problems of one camera
+// model run in step, phase by phase: a phase's kernel has the registers it needs and all of its
+// problems' work at once. The form before it, one persistent kernel over a device queue of
+// (problem, phase, index) items, held four CTAs per SM for every phase and spent a quarter of its
+// CTAs' time waiting for a problem's previous phase: 24 agents (two cameras and a Lidar) on a
+// 2M-triangle terrain, five LM iterations: 15.7 -> 3.03 ms with the direct rasterisation above.
+__global__ void __launch_bounds__(256) k_cull_batch(const WaveArgs *__restrict__ probs) {
+  __shared__ float sM[12];
+  const WaveArgs &a = probs[blockIdx.y];
+  if (!skipped(a)) cull_block(a, 0, blockIdx.x, sM);
+}
+
+__global__ void __launch_bounds__(kPinSetupThreads, 6) k_setup_pin_batch(const WaveArgs *__restrict__ probs) {
+  __shared__ PinSetupSmem sm;
+  const WaveArgs &a = probs[blockIdx.y];
+  if (!skipped(a)) setup_pin(a, 0, sm);
+}
+
+__global__ void __launch_bounds__(kRaySetupThreads, 6) k_setup_ray_batch(const WaveArgs *__restrict__ probs) {
+  __shared__ RaySetupSmem sm;
+  const WaveArgs &a = probs[blockIdx.y];
+  if (!skipped(a)) setup_ray_table(a, 0, sm);
+}
+
+template <int MODE, int MODEL>
+__global__ void __launch_bounds__(kThreads, 4) k_raster_batch(const WaveArgs *__restrict__ probs) {
+  __shared__ RasterSmem<kTileW[MODEL] * kTileH[MODEL], MODEL> sm;
+  const WaveArgs &a = probs[blockIdx.y];
+  if ((int)blockIdx.x >= a.tg.ntiles || skipped(a)) return;
+  raster_block<kTileW[MODEL], kTileH[MODEL], MODE, MODEL>(a, blockIdx.x, 0, sm);
+}
+
+// Copies an LM state with L2 loads (another SM may have written it).
+__device__ __noinline__ void lm_load_cg(const LMState *src, LMState &dst) {
+  const long long *s = reinterpret_cast<const long long *>(src);
+  long long *d = reinterpret_cast<long long *>(&dst);
+  for (int k = 0; k < (int)(sizeof(LMState) / 8); ++k) d[k] = __ldcg(s + k);
+}
+
+// The end of an evaluation of a problem (all threads of a CTA): the sums, the LM or ICP step, and
+// the counters of the next evaluation's lists and bins to zero. A problem whose last evaluation
+// this was is skipped from here on.
+__device__ __forceinline__ void step_problem(const WaveArgs &a, const BatchArgs &b, double *vals) {
+  const int p = a.problem;
+  const int it = b.evals ? __ldcg(b.evals + p) : 0;
+  if (it > b.lm_iters) return;
+  const bool skip = skipped(a);
+  if (!skip) reduce_block(a, 0, vals);
+  if (!b.evals) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float *M = b.Ms + 12 * (long long)p;
+    int done;
+    if (b.icp) {  // every evaluation is followed by a Gauss-Newton step (a no-op once done)
+      IcpState st = b.icp[p];
+      icp_step_dev(st, b.icpargs, a.res_n, a.res_l1, a.res_grad, a.res_jtj, M, b.skip + p);
+      b.icp[p] = st;
+      done = st.done;
+    } else {
+      LMState st;
+      lm_load_cg(b.lm + p, st);
+      if (it == 0) lm_take_initial_dev(st, a.res_counts, a.res_els, a.res_grad, a.res_jtj);
+      else lm_accept_dev(st, b.lmargs, a.res_counts, a.res_els, a.res_grad, a.res_jtj, skip);
+      if (it < b.lm_iters) lm_propose_dev(st, b.lmargs, M, b.skip + p);
+      b.lm[p] = st;
+      done = st.done;
+    }
+    b.evals[p] = it + 1;
+    if (it == b.lm_iters) b.skip[p] = 1;
+    a.vis_count[0] = 0;
+    report_progress(b.progress, it + 1, done);
+  }
+  for (int t = threadIdx.x; t < a.tg.ntiles; t += blockDim.x) {
+    a.counts[t] = 0;
+    a.touched[t] = 0;
+  }
+}
+
+__global__ void __launch_bounds__(256) k_step_batch(const WaveArgs *__restrict__ probs, BatchArgs b) {
+  __shared__ double vals[kNumVals];
+  step_problem(probs[blockIdx.x], b, vals);
+}
+
+__global__ void __launch_bounds__(256) k_step_one(WaveArgs a, BatchArgs b) {
+  __shared__ double vals[kNumVals];
+  step_problem(a, b, vals);
+}
+
+cudaError_t launch_step_one(const WaveArgs &a, const BatchArgs &b, cudaStream_t s) {
+  k_step_one<<<1, 256, 0, s>>>(a, b);
   return cudaGetLastError();
 }
 
-cudaError_t launch_persist_wave(const BatchArgs &b, const WaveArgs &w, int grid, cudaStream_t s) {
-  if (w.cam.model == 0) k_persist_wave<0><<<grid, kThreads, 0, s>>>(b, w);
-  else k_persist_wave<1><<<grid, kThreads, 0, s>>>(b, w);
-  return cudaGetLastError();
-}
-
-int persist_wave_grid(int device, int model) {
-  int sms = 0, per = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-  const cudaError_t e = model == 0 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_persist_wave<0>, kThreads, 0)
-                                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_persist_wave<1>, kThreads, 0);
-  if (e != cudaSuccess) return 0;
-  return sms * (per > 0 ? per : 1);
-}
-
-int persist_grid(int device) {
-  int sms = 0, per = 0;
-  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_persist, kThreads, 0) != cudaSuccess) return 0;
-  return sms * (per > 0 ? per : 1);
-}
-
-cudaError_t launch_lm_init(LMState *st, const double *T0, const LMArgs &a, float *M, int *skip,
-                           cudaStream_t s) {
-  k_lm_init<<<1, 1, 0, s>>>(st, T0, a, M, skip);
-  return cudaGetLastError();
-}
-cudaError_t launch_lm_take_initial(LMState *st, const long long *counts, const double *els,
-                                   const double *grad, const double *jtj, cudaStream_t s) {
-  k_lm_take_initial<<<1, 1, 0, s>>>(st, counts, els, grad, jtj);
-  return cudaGetLastError();
-}
-cudaError_t launch_lm_propose(LMState *st, const LMArgs &a, float *M, int *skip, cudaStream_t s) {
-  k_lm_propose<<<1, 1, 0, s>>>(st, a, M, skip);
-  return cudaGetLastError();
-}
-cudaError_t launch_lm_accept(LMState *st, const LMArgs &a, const long long *counts,
-                             const double *els, const double *grad, const double *jtj, int *skip,
-                             cudaStream_t s) {
-  k_lm_accept<<<1, 1, 0, s>>>(st, a, counts, els, grad, jtj, skip);
+cudaError_t launch_batch_eval(const WaveArgs *probs, int n, int model, int mode, bool vnormals, int n_clusters,
+                              int max_tiles, const BatchArgs &b, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (n_clusters > 0) {
+    k_cull_batch<<<dim3((n_clusters + 255) / 256, n), 256, 0, s>>>(probs);
+    const int blocks = setup_blocks(n_clusters, n);
+    if (model == 0) k_setup_pin_batch<<<dim3(blocks, n), kPinSetupThreads, 0, s>>>(probs);
+    else k_setup_ray_batch<<<dim3(blocks, n), kRaySetupThreads, 0, s>>>(probs);
+  }
+  const dim3 grid(max_tiles, n);
+  if (model == 0) {
+    if (mode == kCostGrad) k_raster_batch<kCostGrad, 0><<<grid, kThreads, 0, s>>>(probs);
+    else if (vnormals) k_raster_batch<kIcpVn, 0><<<grid, kThreads, 0, s>>>(probs);
+    else k_raster_batch<kIcp, 0><<<grid, kThreads, 0, s>>>(probs);
+  } else {
+    if (mode == kCostGrad) k_raster_batch<kCostGrad, 1><<<grid, kThreads, 0, s>>>(probs);
+    else if (vnormals) k_raster_batch<kIcpVn, 1><<<grid, kThreads, 0, s>>>(probs);
+    else k_raster_batch<kIcp, 1><<<grid, kThreads, 0, s>>>(probs);
+  }
+  k_step_batch<<<n, 256, 0, s>>>(probs, b);
   return cudaGetLastError();
 }
 

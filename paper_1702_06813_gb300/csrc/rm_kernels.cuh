@@ -21,6 +21,7 @@ struct WaveArgs {
   int V;
   long long T;
   int n_poses;        // poses in this wave
+  int problem;        // number of the problem in its batch
   int wave_base;      // global index of the wave's first pose
   const float4 *v;    // map vertices (re-centred), w unused
   const int4 *faces;  // i0, i1, i2, label
@@ -84,10 +85,11 @@ cudaError_t launch_ray_dev(const DevCam &cam, int *dev, cudaStream_t s);
 // ev (optional, 5 events): recorded before the cull kernel, then after the cull, setup,
 // raster and reduce kernels, on stream s.
 // zero_counters: clear the wave's bin counts and visible-cluster count first (callers that
-// clear them for several waves at once pass false)
+// clear them for several waves at once pass false); reduce: sum the tiles' partials per pose
+// (callers whose own step kernel does pass false)
 cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t *ev = nullptr,
-                        bool zero_counters = true);
-int wave_kernel_launches(const WaveArgs &a, int mode);
+                        bool zero_counters = true, bool reduce = true);
+int wave_kernel_launches(const WaveArgs &a, int mode, bool reduce = true);
 cudaError_t launch_retract(const double *T, const double *xi, int n, double *out, double *jr,
                            cudaStream_t s);
 // out_k = R n_k for V vertex normals (n: V*3 device floats, R row major): world-frame float4.
@@ -131,16 +133,8 @@ struct IcpArgs {
   double cx, cy, cz;   // map centre
 };
 
-cudaError_t launch_icp_init(IcpState *st, const double *T0, const IcpArgs &a, float *M,
-                            int *skip, cudaStream_t s);
 cudaError_t launch_icp_init_batch(IcpState *st, const double *T0, int n, const IcpArgs &a,
                                   float *Ms, int *skip, cudaStream_t s);
-// After an evaluation at the state's pose (outputs n, l1, g = J^T e, H = J^T J): record it,
-// solve, move the pose and write its matrix, or set *skip when the iterations are over.
-cudaError_t launch_icp_step(IcpState *st, const IcpArgs &a, const long long *n,
-                            const double *l1, const double *g, const double *H, float *M,
-                            int *skip, cudaStream_t s);
-
 // Vertex-position gradient of the surrogate from a rendered visibility buffer.
 struct VGradArgs {
   DevCam cam;
@@ -190,84 +184,41 @@ struct DfoArgs {
 cudaError_t launch_dfo_init(DfoState *st, const double *T0, const DfoArgs &a, float *Ms,
                             int *skip, cudaStream_t s);
 // Takes the Table I costs of the pending candidates (e_table per slot), advances the search
-// and writes the next candidates' matrices, or sets *skip when the search is over.
-cudaError_t launch_dfo_step(DfoState *st, const DfoArgs &a, const long long *e_table, float *Ms,
-                            int *skip, cudaStream_t s);
+// and writes the next candidates' matrices, or sets *skip when the search is over; zeroes the
+// counters of the next evaluation and reports step + 1 to `progress` (see BatchArgs).
+cudaError_t launch_dfo_step(DfoState *st, const DfoArgs &a, const long long *e_table, float *Ms, int *skip,
+                            int *counters, int n_counters, int *progress, int step, cudaStream_t s);
 
-// Batch of problems (each its own camera, scan and scratch) run by one persistent kernel.
-constexpr int kPersistCull = 4;   // 256-cluster chunks per cull item
-// Persistent kernel screen tiles, two per raster item: 64x32 for pinhole problems, 16x16 for
-// ray-table problems (a panoramic tile can hold thousands of bin records, and smaller tiles
-// split that serial work over more CTAs).
-constexpr int kPersistTileW[2] = {64, 16};
-constexpr int kPersistTileH[2] = {32, 16};
-constexpr int kPersistTiles[2] = {2, 2};
+// Default screen tiles by camera model: 64x32 pinhole, 16x16 ray table (a panoramic tile can hold
+// thousands of bin records, and smaller tiles split that serial work over more CTAs).
+constexpr int kTileW[2] = {64, 16};
+constexpr int kTileH[2] = {32, 16};
+
+// A batch of problems, each with its own camera, scan and scratch (WaveArgs of one pose), evaluated
+// in step. States, matrices, skip flags and evaluation counts by problem number.
 struct BatchArgs {
-  const WaveArgs *probs;   // one per problem (n_poses 1, wave_base 0)
-  int n_problems;
-  // Two ready queues in one slot array: slots [0, cap[0]) take raster and reduce items, slots
-  // [cap[0], cap[0] + cap[1]) cull and setup items. An item is (problem, phase (0 cull,
-  // 1 setup, 2 raster, 3 reduce+LM), index within the phase, evaluation number), packed into
-  // one 64-bit word by pack_item so that a claim reads it with a single load; a slot holds -1
-  // until it is published.
-  long long *items;
-  int cap[2];
-  int *qctl;               // head (claimed) and tail (reserved) of each queue, then the number
-                           // of finished problems; zero before launch except the first tail
-  int *done;               // 4 counters per problem: items completed per phase this evaluation
-  int *need;               // per problem: cull items, setup items (set by the kernel each
-                           // evaluation from the visible-cluster count), raster items
-  LMState *lm;             // per problem, or null for a plain evaluation
-  IcpState *icp;           // per problem for ICP alignment (raster in ICP mode), else null
-  IcpArgs icpargs;
+  LMState *lm;             // or null
+  IcpState *icp;           // or null (raster in ICP mode)
+  int *evals;              // evaluations done; null for a single plain evaluation
   float *Ms;               // 12 floats per problem (the problems' a.Ms point here)
   int *skip;               // one flag per problem (the problems' a.skip point here)
   LMArgs lmargs;
-  int lm_iters;            // LM (or ICP) iterations after the first evaluation (evaluations
-                           // 0..lm_iters)
-  unsigned *status;
-  long long spin_limit;    // cycles a CTA may go without finding work before it gives up
+  IcpArgs icpargs;
+  int lm_iters;            // evaluations 0..lm_iters
+  int *progress;           // one problem's loop: host memory for (evaluations done, ended), or null
 };
 
-// Queue item fields: index within the phase (21 bits), phase (2), evaluation (17), problem
-// (23). The host checks the limits before a launch.
-constexpr int kItemIndexBits = 21, kItemEvalBits = 17, kItemProblemBits = 23;
-static_assert(kItemIndexBits + 2 + kItemEvalBits + kItemProblemBits == 63, "item fields fill 63 bits");
-// Evaluations (at most 100001) and raster items (at most 16384^2 / 256 / 2) always fit their
-// fields; the host checks the problem count and the setup items per evaluation.
-__host__ __device__ constexpr long long pack_item(int problem, int phase, int index, int eval) {
-  return ((long long)problem << 40) | ((long long)eval << 23) | ((long long)phase << 21) | (long long)index;
-}
-
-constexpr int kSetupClusters = 64;  // visible clusters per setup item (eight per warp), at most
-// Visible clusters per persistent setup item by camera model: pinhole 64; ray-table views,
-// which see many more clusters, 128.
-__host__ __device__ constexpr int setup_clusters(int model) { return model != 0 ? 128 : kSetupClusters; }
-constexpr int kSetupCtasPerGpu = 912;  // setup CTAs a small wave may spread over (152 SMs x 6)
-
-// Every slot unpublished except the evaluation-0 cull items of every problem at the head of
-// the cull/setup queue; sets that queue's tail.
-cudaError_t launch_queue_init(long long *items, int n_slots, int first_low, int n_problems,
-                              int cull_items, int *qctl, cudaStream_t s);
+constexpr int kSetupCtasPerGpu = 912;  // setup CTA pairs a small wave may spread over (152 SMs x 6)
 
 cudaError_t launch_lm_init_batch(LMState *st, const double *T0, int n, const LMArgs &a,
                                  float *Ms, int *skip, cudaStream_t s);
-cudaError_t launch_persist(const BatchArgs &b, int grid, cudaStream_t s);
-int persist_grid(int device);
-// The persistent kernel for a homogeneous plain batch: the problems are the n_poses poses of
-// the one argument block w (pose q's arrays at the wave's per-pose offsets).
-cudaError_t launch_persist_wave(const BatchArgs &b, const WaveArgs &w, int grid, cudaStream_t s);
-int persist_wave_grid(int device, int model);
-
-cudaError_t launch_lm_init(LMState *st, const double *T0, const LMArgs &a, float *M,
-                           int *skip, cudaStream_t s);
-cudaError_t launch_lm_take_initial(LMState *st, const long long *counts, const double *els,
-                                   const double *grad, const double *jtj, cudaStream_t s);
-cudaError_t launch_lm_propose(LMState *st, const LMArgs &a, float *M, int *skip,
-                              cudaStream_t s);
-cudaError_t launch_lm_accept(LMState *st, const LMArgs &a, const long long *counts,
-                             const double *els, const double *grad, const double *jtj,
-                             int *skip, cudaStream_t s);
+// The end of an evaluation of the one problem a (launch_wave without its reduction).
+cudaError_t launch_step_one(const WaveArgs &a, const BatchArgs &b, cudaStream_t s);
+// One evaluation (and LM or ICP step) of the n problems probs[0..n) of one camera model: cull,
+// setup, raster, step. max_tiles: the most screen tiles of one problem; vnormals: the map carries
+// vertex normals (ICP).
+cudaError_t launch_batch_eval(const WaveArgs *probs, int n, int model, int mode, bool vnormals, int n_clusters,
+                              int max_tiles, const BatchArgs &b, cudaStream_t s);
 
 }  // namespace rmk
 

@@ -540,7 +540,7 @@ def _problems(problems=None, scans=None, poses=None):
 
 def cost_grad_batch(m: Map, problems=None, params=None, *, scans=None, poses=None):
     """cost_grad for [(Scan, pose), ...] that may differ in camera and size (or for `scans` and
-    `poses` as in _problems): one persistent kernel launch. Returns the same dict as
+    `poses` as in _problems) in one library call. Returns the same dict as
     cost_grad, indexed by problem."""
     arr, keep = _problems(problems, scans, poses)
     n = len(arr)
@@ -559,7 +559,7 @@ def cost_grad_batch(m: Map, problems=None, params=None, *, scans=None, poses=Non
 def align_batch(m: Map, problems=None, params=None, max_iters=5, lambda0=1e-3, lambda_up=10.0,
                 lambda_down=10.0, step_tol=1e-8, *, scans=None, poses=None):
     """LM for [(Scan, start pose), ...] (or `scans` and `poses` as in _problems) with every
-    iteration of every problem in one persistent kernel launch. Returns (poses (n,4,4) numpy,
+    iteration of every problem on the device, in step. Returns (poses (n,4,4) numpy,
     list of reports, status name)."""
     arr, keep = _problems(problems, scans, poses)
     n = len(arr)
@@ -578,7 +578,7 @@ def align_batch(m: Map, problems=None, params=None, max_iters=5, lambda0=1e-3, l
 
 def icp_align_batch(m: Map, problems=None, tol=0.1, max_iters=10, step_tol=1e-5, *, scans=None, poses=None):
     """Point-to-plane ICP for [(Scan, start pose), ...] with every evaluation and step of every
-    problem in one persistent kernel launch. Returns (poses (n,4,4) numpy, reports, status)."""
+    problem on the device, in step. Returns (poses (n,4,4) numpy, reports, status)."""
     arr, keep = _problems(problems, scans, poses)
     n = len(arr)
     out = np.empty((n, 16))
