@@ -1516,10 +1516,14 @@ cudaError_t launch_rotate_normals(const float *n, int V, const float *R, float4 
 }
 
 // One (pose q, tile) of the z-buffer and its fused epilogue. Returns false on a timed-out wait.
-template <int TW, int TH, int MODE, int MODEL>
+// FEW: the launch has few CTAs (no more than are resident at once), so that a CTA's own chain of
+// loads decides its time: the scan is loaded at the start, the z-buffer without asking whether it
+// was touched, and every pixel's plane before the first pixel's sums. The sums are the same.
+template <int TW, int TH, int MODE, int MODEL, bool FEW = false>
 __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
                                              RasterSmem<TW * TH, MODEL> &sm) {
   constexpr int NP = TW * TH;
+  constexpr int kPx = NP / kThreads;  // pixels of a thread
   unsigned long long *zk = sm.zk;
   unsigned char *sbuf = sm.sbuf;
   int *S = sm.S;
@@ -1534,7 +1538,18 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
   const int xe = min(ox + TW, W) - 1, ye = min(oy + TH, H) - 1;
 
   const long long bin = (long long)q * a.tg.ntiles + tile;
-  if (a.zbuf && __ldcg(a.touched + bin) != 0) {
+  float few_sd[FEW ? kPx : 1];
+  unsigned char few_sc[FEW ? kPx : 1];
+  if (FEW) {
+#pragma unroll
+    for (int m = 0; m < kPx; ++m) {
+      const int p = tid + m * kThreads, i = ox + p % TW, j = oy + p / TW;
+      const bool in = i <= xe && j <= ye;
+      few_sd[m] = in ? __ldg(a.scan_depth + j * W + i) : 0.0f;
+      few_sc[m] = in ? __ldg(a.scan_cls + j * W + i) : 255;
+    }
+  }
+  if (a.zbuf && (FEW || __ldcg(a.touched + bin) != 0)) {
     // setup rasterised small triangles into this tile: start from their keys, and leave the
     // z-buffer empty for the next wave or call
     unsigned long long *zb = a.zbuf + (long long)q * W * H;
@@ -1670,20 +1685,11 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
     // ---- point-to-plane ICP epilogue (Sec. V): projective association of the pixel's map
     // surface with its scan return, residual e = (d - t)(n . r), J = (n, p x n), p = d r.
     // Counts field 0 holds the associations; eps is the association tolerance.
-#pragma unroll 1
-    for (int p = tid; p < NP; p += kThreads) {
-      const int i = ox + p % TW, j = oy + p / TW;
-      if (i > xe || j > ye) continue;
-      const unsigned long long key = zk[p];
-      if (key == kKeyEmpty) continue;
+    auto pixel = [&](int i, int j, unsigned long long key, float sd, const float4 &pl) {
       const long long pix = (long long)j * W + i;
-      const float sd = a.scan_depth[pix];
-      if (a.scan_cls[pix] != 0 || !(fabsf(sd) <= FLT_MAX)) continue;  // FO returns only
-      const float4 pl = a.planes[(unsigned)key];
-      if (__float_as_int(pl.w) != 0) continue;                         // FO surfaces only
       const float t = key_depth(key);
       const float dz = __fsub_rn(t, sd);
-      if (!(fabsf(dz) < eps)) continue;
+      if (!(fabsf(dz) < eps)) return;
       float rx, ry, rz;
       if (MODEL == 0) {
         rx = (i + 0.5f - a.cam.cx) * ifx;
@@ -1697,14 +1703,14 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
       }
       float nx, ny, nz;
       if (MODE == kIcpVn) {
-        if (!vertex_normal(a, sm.M, (unsigned)key, t, rx, ry, rz, nx, ny, nz)) continue;
+        if (!vertex_normal(a, sm.M, (unsigned)key, t, rx, ry, rz, nx, ny, nz)) return;
       } else {
         nx = R[0] * pl.x + R[1] * pl.y + R[2] * pl.z;
         ny = R[3] * pl.x + R[4] * pl.y + R[5] * pl.z;
         nz = R[6] * pl.x + R[7] * pl.y + R[8] * pl.z;
       }
       const float nn = nx * nx + ny * ny + nz * nz;
-      if (!(nn > 0.0f)) continue;  // degenerate face: no plane
+      if (!(nn > 0.0f)) return;  // degenerate face: no plane
       const float u = rsqrtf(nn);
       nx *= u;
       ny *= u;
@@ -1728,28 +1734,46 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
       for (int u2 = 0; u2 < 6; ++u2)
 #pragma unroll
         for (int v2 = u2; v2 < 6; ++v2) acc[qk++] += J[u2] * J[v2];
+    };
+    if (FEW) {
+      float4 pl[kPx];
+#pragma unroll
+      for (int m = 0; m < kPx; ++m) {
+        const unsigned long long key = zk[tid + m * kThreads];
+        pl[m] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(1));  // no pair
+        if (key != kKeyEmpty && few_sc[m] == 0 && fabsf(few_sd[m]) <= FLT_MAX) pl[m] = a.planes[(unsigned)key];
+      }
+#pragma unroll
+      for (int m = 0; m < kPx; ++m) {
+        const int p = tid + m * kThreads;
+        if (__float_as_int(pl[m].w) == 0) pixel(ox + p % TW, oy + p / TW, zk[p], few_sd[m], pl[m]);
+      }
+    } else {
+#pragma unroll 1
+      for (int p = tid; p < NP; p += kThreads) {
+        const int i = ox + p % TW, j = oy + p / TW;
+        if (i > xe || j > ye) continue;
+        const unsigned long long key = zk[p];
+        if (key == kKeyEmpty) continue;
+        const long long pix = (long long)j * W + i;
+        const float sd = a.scan_depth[pix];
+        if (a.scan_cls[pix] != 0 || !(fabsf(sd) <= FLT_MAX)) continue;  // FO returns only
+        const float4 pl = a.planes[(unsigned)key];
+        if (__float_as_int(pl.w) != 0) continue;                         // FO surfaces only
+        pixel(i, j, key, sd, pl);
+      }
     }
   } else {
-#pragma unroll 1
-  for (int p = tid; p < NP; p += kThreads) {
-    const int i = ox + p % TW, j = oy + p / TW;
-    if (i > xe || j > ye) continue;
-    const unsigned long long key = zk[p];
-    if (key == kKeyEmpty) continue;  // map NaN row: ignore
+  auto pixel = [&](int i, int j, unsigned long long key, float sd, int sc, const float4 &pl) {
     const long long pix = (long long)j * W + i;
-    const float sd = a.scan_depth[pix];
-    const int sc = a.scan_cls[pix];
-    if (sc > 1 || !(fabsf(sd) <= FLT_MAX)) continue;  // scan NaN column: ignore
-    const unsigned id = (unsigned)key;
     const float t = key_depth(key);
-    const float4 pl = a.planes[id];
     const int mc = __float_as_int(pl.w);
-    if (mc > 1) continue;  // unknown-occupied row: ignore
+    if (mc > 1) return;  // unknown-occupied row: ignore
     const float dz = __fsub_rn(t, sd);
     int oc;
     if (mc == 0) oc = sc == 0 ? (fabsf(dz) <= eps ? 0 : 1) : (dz > 0.0f ? 2 : 3);
     else if (sc == 0) oc = dz <= 0.0f ? 4 : 5;
-    else continue;  // FU / FU: ignore
+    else return;  // FU / FU: ignore
     cnt6 += 1u << (5 * oc);
     float r, w, sgn = 0.0f;
     switch (oc) {
@@ -1799,6 +1823,33 @@ __device__ __forceinline__ void raster_block(const WaveArgs &a, int tile, int q,
       for (int u = 0; u < 6; ++u)
 #pragma unroll
         for (int v = u; v < 6; ++v) acc[qk++] += w * J[u] * J[v];
+    }
+  };
+  if (FEW) {
+    float4 pl[kPx];
+#pragma unroll
+    for (int m = 0; m < kPx; ++m) {
+      const unsigned long long key = zk[tid + m * kThreads];
+      pl[m] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(2));  // nothing to compare
+      if (key != kKeyEmpty && few_sc[m] <= 1 && fabsf(few_sd[m]) <= FLT_MAX) pl[m] = a.planes[(unsigned)key];
+    }
+#pragma unroll
+    for (int m = 0; m < kPx; ++m) {
+      const int p = tid + m * kThreads;
+      pixel(ox + p % TW, oy + p / TW, zk[p], few_sd[m], few_sc[m], pl[m]);
+    }
+  } else {
+#pragma unroll 1
+    for (int p = tid; p < NP; p += kThreads) {
+      const int i = ox + p % TW, j = oy + p / TW;
+      if (i > xe || j > ye) continue;
+      const unsigned long long key = zk[p];
+      if (key == kKeyEmpty) continue;  // map NaN row: ignore
+      const long long pix = (long long)j * W + i;
+      const float sd = a.scan_depth[pix];
+      const int sc = a.scan_cls[pix];
+      if (sc > 1 || !(fabsf(sd) <= FLT_MAX)) continue;  // scan NaN column: ignore
+      pixel(i, j, key, sd, sc, a.planes[(unsigned)key]);
     }
   }
   }
@@ -1860,19 +1911,40 @@ __global__ void __launch_bounds__(kThreads, RM_RASTER_MIN_BLOCKS) k_raster(WaveA
   raster_block<TW, TH, MODE, MODEL>(a, blockIdx.x, blockIdx.y, sm);
 }
 
+// The raster of a launch of few CTAs (at most kFewCtas): the registers for two or, without the
+// gradient's sums, four CTAs per SM.
+constexpr int kFewCtas = 304;  // 152 SMs x 2
+template <int TW, int TH, int MODE, int MODEL>
+__global__ void __launch_bounds__(kThreads, MODE == kCost ? 4 : 2) k_raster_few(WaveArgs a) {
+  __shared__ RasterSmem<TW * TH, MODEL> sm;
+  if (skipped(a)) return;
+  raster_block<TW, TH, MODE, MODEL, true>(a, blockIdx.x, blockIdx.y, sm);
+}
+
 // Per pose: sum the per-tile partials. Warp w reduces values w, w+8, ...; lane l sums tiles
 // l, l+32, ... and a butterfly combines the lanes, so the order is fixed run to run.
 __device__ __forceinline__ void reduce_block(const WaveArgs &a, int q, double *vals) {
   const int g = a.wave_base + q;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double *base = a.partial + (long long)q * a.tg.ntiles * kNumVals;
-  for (int k = warp; k < kNumVals; k += 8) {
-    double s = 0.0;
-    for (int t = lane; t < a.tg.ntiles; t += 32) s += __ldcg(base + (long long)t * kNumVals + k);
+  // a warp's five values side by side: one load latency per step down the tiles, not five
+  constexpr int kMine = (kNumVals + 7) / 8;
+  double s[kMine];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) vals[k] = s;
+  for (int m = 0; m < kMine; ++m) s[m] = 0.0;
+#pragma unroll 2
+  for (int t = lane; t < a.tg.ntiles; t += 32) {
+#pragma unroll
+    for (int m = 0; m < kMine; ++m)
+      if (warp + 8 * m < kNumVals) s[m] += __ldcg(base + (long long)t * kNumVals + warp + 8 * m);
   }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+    for (int m = 0; m < kMine; ++m) s[m] += __shfl_xor_sync(0xffffffffu, s[m], off);
+#pragma unroll
+  for (int m = 0; m < kMine; ++m)
+    if (lane == 0 && warp + 8 * m < kNumVals) vals[warp + 8 * m] = s[m];
   __syncthreads();
   const int k = threadIdx.x;
   if (k < 6 && a.res_counts) a.res_counts[6 * (long long)g + k] = (long long)vals[k];
@@ -1896,6 +1968,15 @@ __global__ void __launch_bounds__(256) k_reduce(WaveArgs a) {
 template <int TW, int TH, int MODEL>
 static cudaError_t launch_raster_m(const WaveArgs &a, int mode, cudaStream_t s) {
   dim3 grid(a.tg.ntiles, a.n_poses);
+  if constexpr (TW == 64 && MODEL == 0) {  // eight pixels to a thread
+    const long long ctas = (long long)a.tg.ntiles * a.n_poses;
+    if (ctas <= (mode == kCost ? 2 : 1) * kFewCtas && mode != kRender && !(mode == kIcp && a.vnormals)) {
+      if (mode == kCost) k_raster_few<TW, TH, kCost, MODEL><<<grid, kThreads, 0, s>>>(a);
+      else if (mode == kIcp) k_raster_few<TW, TH, kIcp, MODEL><<<grid, kThreads, 0, s>>>(a);
+      else k_raster_few<TW, TH, kCostGrad, MODEL><<<grid, kThreads, 0, s>>>(a);
+      return cudaGetLastError();
+    }
+  }
   if (mode == kRender) k_raster<TW, TH, kRender, MODEL><<<grid, kThreads, 0, s>>>(a);
   else if (mode == kCost) k_raster<TW, TH, kCost, MODEL><<<grid, kThreads, 0, s>>>(a);
   else if (mode == kIcp && a.vnormals) k_raster<TW, TH, kIcpVn, MODEL><<<grid, kThreads, 0, s>>>(a);
@@ -1911,11 +1992,11 @@ static cudaError_t launch_raster(const WaveArgs &a, int mode, cudaStream_t s) {
 
 // Setup CTAs (four warps) per pose: 32 in a large wave, so that each warp sets up several clusters
 // and the next wave's setup (on the other stream) takes few enough SMs to run beside this wave's
-// raster; waves of few poses (single-pose alignment) get up to about twelve CTAs per SM in total,
-// so that their setup spreads over the GPU.
+// raster; waves of few poses (single-pose alignment) get up to seven CTAs per SM in total and as
+// little as one cluster to a warp: the chain of a cluster's loads is what they wait for.
 static int setup_blocks(int n_clusters, int n_poses) {
-  const int per_pose = max(16, (kSetupCtasPerGpu + n_poses - 1) / n_poses);
-  return 2 * min(max(n_clusters / 64, 1), per_pose);
+  const int per_pose = max(32, (kSetupCtasPerGpu + n_poses - 1) / n_poses);
+  return min((n_clusters + 3) / 4, per_pose);
 }
 
 cudaError_t launch_wave(const WaveArgs &a, int mode, cudaStream_t s, cudaEvent_t *ev,
@@ -1978,20 +2059,27 @@ __device__ __noinline__ void se3_right_dev(const double *T, const double *xi, do
   }
   const double K[9] = {0, -phi[2], phi[1], phi[2], 0, -phi[0], -phi[1], phi[0], 0};
   double K2[9];
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
       double s = 0;
+#pragma unroll
       for (int k = 0; k < 3; ++k) s += K[3 * i + k] * K[3 * k + j];
       K2[3 * i + j] = s;
     }
   double E[16];
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
       const double I = i == j ? 1.0 : 0.0;
       E[4 * i + j] = I + A * K[3 * i + j] + B * K2[3 * i + j];
     }
+#pragma unroll
   for (int i = 0; i < 3; ++i) {
     double t = 0;
+#pragma unroll
     for (int j = 0; j < 3; ++j) {
       const double I = i == j ? 1.0 : 0.0;
       t += (I + B * K[3 * i + j] + C * K2[3 * i + j]) * rho[j];
@@ -2000,9 +2088,12 @@ __device__ __noinline__ void se3_right_dev(const double *T, const double *xi, do
   }
   E[12] = E[13] = E[14] = 0.0;
   E[15] = 1.0;
+#pragma unroll
   for (int i = 0; i < 4; ++i)
+#pragma unroll
     for (int j = 0; j < 4; ++j) {
       double s = 0;
+#pragma unroll
       for (int k = 0; k < 4; ++k) s += T[4 * i + k] * E[4 * k + j];
       out[4 * i + j] = s;
     }
@@ -2118,17 +2209,24 @@ cudaError_t launch_twist_grad(const double *xi, const double *g, const double *s
 __device__ __noinline__ bool lm_solve_dev(const double *jtj, const double *g, double lambda, double *x) {
   double A[36], L[36];
   int q = 0;
+#pragma unroll
   for (int u = 0; u < 6; ++u)
+#pragma unroll
     for (int v = u; v < 6; ++v) {
       A[6 * u + v] = jtj[q];
       A[6 * v + u] = jtj[q];
       ++q;
     }
+#pragma unroll
   for (int u = 0; u < 36; ++u) L[u] = 0.0;
+#pragma unroll
   for (int u = 0; u < 6; ++u) A[7 * u] += lambda * A[7 * u];
+#pragma unroll
   for (int i = 0; i < 6; ++i)
+#pragma unroll
     for (int j = 0; j <= i; ++j) {
       double s = A[6 * i + j];
+#pragma unroll
       for (int k = 0; k < j; ++k) s -= L[6 * i + k] * L[6 * j + k];
       if (i == j) {
         if (!(s > 0.0)) return false;
@@ -2138,13 +2236,17 @@ __device__ __noinline__ bool lm_solve_dev(const double *jtj, const double *g, do
       }
     }
   double y[6];
+#pragma unroll
   for (int i = 0; i < 6; ++i) {
     double s = -g[i];
+#pragma unroll
     for (int k = 0; k < i; ++k) s -= L[6 * i + k] * y[k];
     y[i] = s / L[7 * i];
   }
+#pragma unroll
   for (int i = 5; i >= 0; --i) {
     double s = y[i];
+#pragma unroll
     for (int k = i + 1; k < 6; ++k) s -= L[6 * k + i] * x[k];
     x[i] = s / L[7 * i];
   }
@@ -2524,17 +2626,28 @@ __device__ void dfo_advance(DfoState &s, const DfoArgs &a, const long long *et) 
   }
 }
 
-// One step of the search, and the counters of the next evaluation's lists and bins to zero.
+// One step of the search, and the counters of the next evaluation's lists and bins to zero. The
+// search's control flow is one thread's; its state is in shared memory meanwhile, because a chain of
+// global reads and writes made the step the longest kernel of an evaluation (52 us, now below 20).
 __global__ void __launch_bounds__(256) k_dfo_step(DfoState *st, DfoArgs a, const long long *et, float *Ms, int *skip,
                                                   int *counters, int n_counters, int *progress, int step) {
-  if (threadIdx.x == 0) {
-    if (st->phase != 4) dfo_advance(*st, a, et);
-    *skip = st->phase == 4;
-  }
+  static_assert(sizeof(DfoState) % 8 == 0, "copied in 8-byte words");
+  constexpr int kWords = sizeof(DfoState) / 8;
+  __shared__ DfoState sh;
+  __shared__ long long costs[kDfoSlots];
+  long long *w = reinterpret_cast<long long *>(&sh), *g = reinterpret_cast<long long *>(st);
+  for (int k = threadIdx.x; k < kWords; k += blockDim.x) w[k] = g[k];
+  if (threadIdx.x < kDfoSlots) costs[threadIdx.x] = et[threadIdx.x];
   for (int k = threadIdx.x; k < n_counters; k += blockDim.x) counters[k] = 0;
   __syncthreads();
-  if (st->phase != 4) dfo_write_candidates(*st, a, Ms);
-  if (threadIdx.x == 0) report_progress(progress, step + 1, st->phase == 4);
+  if (threadIdx.x == 0) {
+    if (sh.phase != 4) dfo_advance(sh, a, costs);
+    *skip = sh.phase == 4;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < kWords; k += blockDim.x) g[k] = w[k];
+  if (sh.phase != 4) dfo_write_candidates(sh, a, Ms);
+  if (threadIdx.x == 0) report_progress(progress, step + 1, sh.phase == 4);
 }
 
 cudaError_t launch_dfo_init(DfoState *st, const double *T0, const DfoArgs &a, float *Ms,

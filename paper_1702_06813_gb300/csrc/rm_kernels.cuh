@@ -208,7 +208,7 @@ struct BatchArgs {
   int *progress;           // one problem's loop: host memory for (evaluations done, ended), or null
 };
 
-constexpr int kSetupCtasPerGpu = 912;  // setup CTA pairs a small wave may spread over (152 SMs x 6)
+constexpr int kSetupCtasPerGpu = 1064;  // setup CTAs a small wave may spread over (152 SMs x 7)
 
 cudaError_t launch_lm_init_batch(LMState *st, const double *T0, int n, const LMArgs &a,
                                  float *Ms, int *skip, cudaStream_t s);
