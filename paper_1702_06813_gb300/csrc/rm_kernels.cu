@@ -2387,55 +2387,70 @@ __device__ __forceinline__ void report_progress(int *progress, int evals, int do
 
 // ------------------------------------------------------------------ derivative-free search
 
-// Vertex order by value, ties by slot (stable insertion sort).
+// The search's control flow runs on one warp over a state in shared memory: every lane follows the
+// same branches, the lanes share the element-wise work (FP64 divisions and square roots take
+// hundreds of cycles, one after the other, on a single thread), lane 0 writes the scalars. Each
+// function expects the state to be settled (a __syncwarp since the last write) and leaves it so.
+
+// Vertex order by value, ties by slot: o[rank] = slot.
 __device__ void dfo_order(const double *f, int *o) {
-  for (int i = 0; i < 7; ++i) o[i] = i;
-  for (int i = 1; i < 7; ++i)
-    for (int j = i; j > 0 && f[o[j]] < f[o[j - 1]]; --j) {
-      const int t = o[j];
-      o[j] = o[j - 1];
-      o[j - 1] = t;
-    }
+  const int i = threadIdx.x & 31;
+  if (i < 7) {
+    int rank = 0;
+    for (int j = 0; j < 7; ++j) rank += f[j] < f[i] || (f[j] == f[i] && j < i);
+    o[rank] = i;
+  }
+  __syncwarp();
+}
+
+__device__ __forceinline__ double warp_max_d(double x) {
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, off));
+  return x;
 }
 
 // Coordinate descent: converged, out of iterations, or the 12 moves +-step per axis.
 __device__ void dfo_next_cd(DfoState &s, const DfoArgs &a) {
-  if (s.cd_iters >= a.cd_iters) {
-    s.phase = 4;
-    return;
-  }
-  double smax = 0.0;
-  for (int k = 0; k < 6; ++k) smax = fmax(smax, s.st[k] / a.scale[k]);
-  if (smax < a.cd_tol) {
-    s.converged = 1;
-    s.phase = 4;
-    return;
-  }
-  for (int m = 0; m < 12; ++m)
-    for (int k = 0; k < 6; ++k)
+  const int lane = threadIdx.x & 31;
+  const bool out = s.cd_iters >= a.cd_iters;
+  const double smax = out ? 0.0 : warp_max_d(lane < 6 ? fmax(0.0, s.st[lane] / a.scale[lane]) : 0.0);
+  const bool conv = !out && smax < a.cd_tol;
+  if (!out && !conv)
+    for (int e = lane; e < 72; e += 32) {
+      const int m = e / 6, k = e % 6;
       s.cand[m][k] = s.xc[k] + (k == m / 2 ? (m % 2 ? -s.st[k] : s.st[k]) : 0.0);
-  s.n_cand = 12;
-  s.phase = 3;
+    }
+  __syncwarp();
+  if (lane == 0) {
+    if (conv) s.converged = 1;
+    s.phase = out || conv ? 4 : 3;
+    if (!out && !conv) s.n_cand = 12;
+  }
+  __syncwarp();
 }
 
 // Next Nelder-Mead iteration (the four candidates), or the switch to coordinate descent.
-__device__ void dfo_next_nm(DfoState &s, const DfoArgs &a) {
-  int o[7];
+__device__ void dfo_next_nm(DfoState &s, const DfoArgs &a, int *o) {
+  const int lane = threadIdx.x & 31;
   dfo_order(s.f, o);
   double diam = 0.0;
-  for (int i = 1; i < 7; ++i)
-    for (int k = 0; k < 6; ++k) diam = fmax(diam, fabs(s.x[o[i]][k] - s.x[o[0]][k]) / a.scale[k]);
+  for (int e = lane; e < 36; e += 32) {
+    const int i = 1 + e / 6, k = e % 6;
+    diam = fmax(diam, fabs(s.x[o[i]][k] - s.x[o[0]][k]) / a.scale[k]);
+  }
+  diam = warp_max_d(diam);
   if (s.nm_iters >= a.nm_iters || diam < a.nm_tol) {
-    for (int k = 0; k < 6; ++k) {
-      s.xc[k] = s.x[o[0]][k];
-      s.st[k] = a.cd_step * a.scale[k];
+    if (lane < 6) {
+      s.xc[lane] = s.x[o[0]][lane];
+      s.st[lane] = a.cd_step * a.scale[lane];
     }
-    s.fcur = s.f[o[0]];
+    if (lane == 0) s.fcur = s.f[o[0]];
+    __syncwarp();
     dfo_next_cd(s, a);
     return;
   }
-  const int h = o[6];
-  for (int k = 0; k < 6; ++k) {
+  if (lane < 6) {
+    const int k = lane, h = o[6];
     double sum = 0.0;
     for (int i = 0; i < 6; ++i) sum += s.x[o[i]][k];
     const double c = sum / 6.0, d = c - s.x[h][k];
@@ -2444,8 +2459,11 @@ __device__ void dfo_next_nm(DfoState &s, const DfoArgs &a) {
     s.cand[2][k] = c + 0.5 * d;
     s.cand[3][k] = c - 0.5 * d;
   }
-  s.n_cand = 4;
-  s.phase = 1;
+  if (lane == 0) {
+    s.n_cand = 4;
+    s.phase = 1;
+  }
+  __syncwarp();
 }
 
 // Powell's line search from xc along d: the 12 points xc + (a step) d, products and sums
@@ -2453,71 +2471,90 @@ __device__ void dfo_next_nm(DfoState &s, const DfoArgs &a) {
 __constant__ double kPowellA[12] = {0.25, -0.25, 0.5, -0.5, 1.0, -1.0, 2.0, -2.0, 4.0, -4.0, 8.0, -8.0};
 
 __device__ void powell_line(DfoState &s, const double *d, double step) {
-  for (int m = 0; m < 12; ++m) {
-    const double am = __dmul_rn(kPowellA[m], step);
-    for (int k = 0; k < 6; ++k) s.cand[m][k] = __dadd_rn(s.xc[k], __dmul_rn(am, d[k]));
+  const int lane = threadIdx.x & 31;
+  for (int e = lane; e < 72; e += 32) {
+    const int m = e / 6, k = e % 6;
+    s.cand[m][k] = __dadd_rn(s.xc[k], __dmul_rn(__dmul_rn(kPowellA[m], step), d[k]));
   }
-  s.n_cand = 12;
-  s.phase = 6;
+  if (lane == 0) {
+    s.n_cand = 12;
+    s.phase = 6;
+  }
+  __syncwarp();
 }
 
 // The next Powell iteration (its first axis search), or the switch to coordinate descent from
 // Powell's end point once out of iterations or below the step tolerance.
 __device__ void powell_next(DfoState &s, const DfoArgs &a) {
+  const int lane = threadIdx.x & 31;
   if (s.powell_iters >= a.powell_iters || !(s.ps >= a.powell_tol)) {
-    for (int k = 0; k < 6; ++k) s.st[k] = a.cd_step * a.scale[k];
+    if (lane < 6) s.st[lane] = a.cd_step * a.scale[lane];
+    __syncwarp();
     dfo_next_cd(s, a);
     return;
   }
-  for (int k = 0; k < 6; ++k) s.x0[k] = s.xc[k];
-  s.best_drop = 0.0;
-  s.best_dir = 0;
-  s.pdir = 0;
+  if (lane < 6) s.x0[lane] = s.xc[lane];
+  if (lane == 0) {
+    s.best_drop = 0.0;
+    s.best_dir = 0;
+    s.pdir = 0;
+  }
+  __syncwarp();
   powell_line(s, s.D[0], s.ps);
 }
 
 // One finished Powell line search: take its lowest point if it lowers the value, then the
 // next direction, the displacement search, or the next iteration.
 __device__ void powell_step(DfoState &s, const DfoArgs &a, const double *fc) {
+  const int lane = threadIdx.x & 31;
   int best = 0;
   for (int m = 1; m < 12; ++m)
     if (fc[m] < fc[best]) best = m;
-  double drop = 0.0;
-  if (fc[best] < s.fcur) {
-    drop = s.fcur - fc[best];
-    for (int k = 0; k < 6; ++k) s.xc[k] = s.cand[best][k];
-    s.fcur = fc[best];
-  }
-  if (s.pdir == 6) {  // the displacement search: replace the direction of largest decrease
+  const bool lower = fc[best] < s.fcur;
+  const double drop = lower ? s.fcur - fc[best] : 0.0;
+  const int pdir = s.pdir;
+  __syncwarp();
+  if (lower && lane < 6) s.xc[lane] = s.cand[best][lane];
+  if (lower && lane == 0) s.fcur = fc[best];
+  if (pdir == 6) {  // the displacement search: replace the direction of largest decrease
     const double n = __dsqrt_rn(s.n2);
-    for (int k = 0; k < 6; ++k) s.D[s.best_dir][k] = __ddiv_rn(s.disp[k], n);
+    if (lane < 6) s.D[s.best_dir][lane] = __ddiv_rn(s.disp[lane], n);
+    __syncwarp();
     powell_next(s, a);
     return;
   }
-  if (drop > s.best_drop) {
-    s.best_drop = drop;
-    s.best_dir = s.pdir;
+  if (lane == 0) {
+    if (drop > s.best_drop) {
+      s.best_drop = drop;
+      s.best_dir = pdir;
+    }
+    s.pdir = pdir + 1;
+    if (pdir == 5) s.powell_iters += 1;
   }
-  s.pdir += 1;
-  if (s.pdir < 6) {
-    powell_line(s, s.D[s.pdir], s.ps);
+  __syncwarp();
+  if (pdir < 5) {
+    powell_line(s, s.D[pdir + 1], s.ps);
     return;
   }
-  s.powell_iters += 1;
+  double u2 = 0.0;
+  if (lane < 6) {
+    const double d = __dsub_rn(s.xc[lane], s.x0[lane]), u = __ddiv_rn(d, a.scale[lane]);
+    s.disp[lane] = d;
+    u2 = __dmul_rn(u, u);
+  }
   double n2 = 0.0;
-  for (int k = 0; k < 6; ++k) {
-    s.disp[k] = __dsub_rn(s.xc[k], s.x0[k]);
-    const double u = __ddiv_rn(s.disp[k], a.scale[k]);
-    n2 = __dadd_rn(n2, __dmul_rn(u, u));
+  for (int k = 0; k < 6; ++k) n2 = __dadd_rn(n2, __shfl_sync(0xffffffffu, u2, k));
+  if (lane == 0) {
+    if (n2 == 0.0) {
+      s.ps = 0.5 * s.ps;
+    } else {
+      s.n2 = n2;
+      s.pdir = 6;
+    }
   }
-  if (n2 == 0.0) {
-    s.ps = 0.5 * s.ps;
-    powell_next(s, a);
-    return;
-  }
-  s.n2 = n2;
-  s.pdir = 6;
-  powell_line(s, s.disp, 1.0);
+  __syncwarp();
+  if (n2 == 0.0) powell_next(s, a);
+  else powell_line(s, s.disp, 1.0);
 }
 
 // The candidates' matrices, one thread each (their FP64 retractions are a serial chain).
@@ -2558,96 +2595,101 @@ __global__ void k_dfo_init(DfoState *st, const double *T0, DfoArgs a, float *Ms,
 }
 
 // Takes the costs of the pending candidates and plans the next ones.
-__device__ void dfo_advance(DfoState &s, const DfoArgs &a, const long long *et) {
-  double fc[kDfoSlots];
-  for (int m = 0; m < s.n_cand; ++m) fc[m] = (double)et[m];
-  s.evals += s.n_cand;
-  if (s.phase == 0) {
-    s.f_init = fc[0];
-    for (int i = 0; i < 7; ++i) {
-      for (int k = 0; k < 6; ++k) s.x[i][k] = s.cand[i][k];
-      s.f[i] = fc[i];
-    }
-    dfo_next_nm(s, a);
-  } else if (s.phase == 1) {
-    s.nm_iters += 1;
-    int o[7];
+__device__ void dfo_advance(DfoState &s, const DfoArgs &a, const double *fc, int *o) {
+  const int lane = threadIdx.x & 31, phase = s.phase;
+  if (lane == 0) s.evals += s.n_cand;
+  __syncwarp();
+  if (phase == 0) {
+    for (int e = lane; e < 42; e += 32) s.x[e / 6][e % 6] = s.cand[e / 6][e % 6];
+    if (lane < 7) s.f[lane] = fc[lane];
+    if (lane == 0) s.f_init = fc[0];
+    __syncwarp();
+    dfo_next_nm(s, a, o);
+  } else if (phase == 1) {
+    if (lane == 0) s.nm_iters += 1;
     dfo_order(s.f, o);
-    const int h = o[6];
-    const double fb = s.f[o[0]], fs = s.f[o[5]], fh = s.f[h];
+    const int h = o[6], b = o[0];
+    const double fb = s.f[b], fs = s.f[o[5]], fh = s.f[h];
     int take;
     if (fc[0] < fb) take = fc[1] < fc[0] ? 1 : 0;
     else if (fc[0] < fs) take = 0;
     else if (fc[0] < fh) take = fc[2] <= fc[0] ? 2 : -1;
     else take = fc[3] < fh ? 3 : -1;
+    __syncwarp();
     if (take >= 0) {
-      for (int k = 0; k < 6; ++k) s.x[h][k] = s.cand[take][k];
-      s.f[h] = fc[take];
-      dfo_next_nm(s, a);
+      if (lane < 6) s.x[h][lane] = s.cand[take][lane];
+      if (lane == 0) s.f[h] = fc[take];
+      __syncwarp();
+      dfo_next_nm(s, a, o);
     } else {
-      const int b = o[0];
-      int m = 0;
-      for (int i = 0; i < 7; ++i) {
-        if (i == b) continue;
-        for (int k = 0; k < 6; ++k) s.cand[m][k] = s.x[b][k] + 0.5 * (s.x[i][k] - s.x[b][k]);
-        ++m;
+      for (int e = lane; e < 36; e += 32) {
+        const int m = e / 6, k = e % 6, i = m < b ? m : m + 1;
+        s.cand[m][k] = s.x[b][k] + 0.5 * (s.x[i][k] - s.x[b][k]);
       }
-      s.shrink_best = b;
-      s.n_cand = 6;
-      s.phase = 2;
+      if (lane == 0) {
+        s.shrink_best = b;
+        s.n_cand = 6;
+        s.phase = 2;
+      }
+      __syncwarp();
     }
-  } else if (s.phase == 2) {
-    s.nm_shrinks += 1;
-    int m = 0;
-    for (int i = 0; i < 7; ++i) {
-      if (i == s.shrink_best) continue;
-      for (int k = 0; k < 6; ++k) s.x[i][k] = s.cand[m][k];
-      s.f[i] = fc[m];
-      ++m;
+  } else if (phase == 2) {
+    const int b = s.shrink_best;
+    for (int e = lane; e < 36; e += 32) {
+      const int m = e / 6, k = e % 6, i = m < b ? m : m + 1;
+      s.x[i][k] = s.cand[m][k];
+      if (k == 0) s.f[i] = fc[m];
     }
-    dfo_next_nm(s, a);
-  } else if (s.phase == 5) {
-    s.f_init = s.fcur = fc[0];
+    if (lane == 0) s.nm_shrinks += 1;
+    __syncwarp();
+    dfo_next_nm(s, a, o);
+  } else if (phase == 5) {
+    if (lane == 0) s.f_init = s.fcur = fc[0];
+    __syncwarp();
     powell_next(s, a);
-  } else if (s.phase == 6) {
+  } else if (phase == 6) {
     powell_step(s, a, fc);
   } else {
-    s.cd_iters += 1;
     int best = 0;
     for (int m = 1; m < 12; ++m)
       if (fc[m] < fc[best]) best = m;
-    if (fc[best] < s.fcur) {
-      for (int k = 0; k < 6; ++k) s.xc[k] = s.cand[best][k];
-      s.fcur = fc[best];
-    } else {
-      for (int k = 0; k < 6; ++k) s.st[k] *= 0.5;
+    const bool lower = fc[best] < s.fcur;
+    __syncwarp();
+    if (lane < 6) {
+      if (lower) s.xc[lane] = s.cand[best][lane];
+      else s.st[lane] *= 0.5;
     }
+    if (lane == 0) {
+      s.cd_iters += 1;
+      if (lower) s.fcur = fc[best];
+    }
+    __syncwarp();
     dfo_next_cd(s, a);
   }
 }
 
-// One step of the search, and the counters of the next evaluation's lists and bins to zero. The
-// search's control flow is one thread's; its state is in shared memory meanwhile, because a chain of
-// global reads and writes made the step the longest kernel of an evaluation (52 us, now below 20).
+// One step of the search, and the counters of the next evaluation's lists and bins to zero: 51 us
+// after a Nelder-Mead evaluation while one thread did it all, 19 us on a warp.
 __global__ void __launch_bounds__(256) k_dfo_step(DfoState *st, DfoArgs a, const long long *et, float *Ms, int *skip,
                                                   int *counters, int n_counters, int *progress, int step) {
   static_assert(sizeof(DfoState) % 8 == 0, "copied in 8-byte words");
   constexpr int kWords = sizeof(DfoState) / 8;
   __shared__ DfoState sh;
-  __shared__ long long costs[kDfoSlots];
+  __shared__ double fc[kDfoSlots];
+  __shared__ int order[7];
   long long *w = reinterpret_cast<long long *>(&sh), *g = reinterpret_cast<long long *>(st);
   for (int k = threadIdx.x; k < kWords; k += blockDim.x) w[k] = g[k];
-  if (threadIdx.x < kDfoSlots) costs[threadIdx.x] = et[threadIdx.x];
+  if (threadIdx.x < kDfoSlots) fc[threadIdx.x] = (double)et[threadIdx.x];
   for (int k = threadIdx.x; k < n_counters; k += blockDim.x) counters[k] = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (sh.phase != 4) dfo_advance(sh, a, costs);
-    *skip = sh.phase == 4;
-  }
+  if (threadIdx.x < 32 && sh.phase != 4) dfo_advance(sh, a, fc, order);
   __syncthreads();
   for (int k = threadIdx.x; k < kWords; k += blockDim.x) g[k] = w[k];
   if (sh.phase != 4) dfo_write_candidates(sh, a, Ms);
-  if (threadIdx.x == 0) report_progress(progress, step + 1, sh.phase == 4);
+  if (threadIdx.x == 0) {
+    *skip = sh.phase == 4;
+    report_progress(progress, step + 1, sh.phase == 4);
+  }
 }
 
 cudaError_t launch_dfo_init(DfoState *st, const double *T0, const DfoArgs &a, float *Ms,
