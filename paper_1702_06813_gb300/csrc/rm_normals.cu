@@ -1,16 +1,21 @@
 // rm_normals.cu -- rm_depth_normals: surface normals of depth images (Eq. 2, Sec. V).
 //
-// One CTA per (64x16 output tile, image), fused: the tile's depths with a halo of r + 1
-// pixels are staged in shared memory as depths and validity weights (invalid pixels
-// contribute neither), smoothed with the separable Gaussian as a normalised convolution (a
-// horizontal pass of weighted sums and weight sums, four outputs per thread sliding along a
-// row, then a vertical pass, six per thread down a column; one instantiation per radius, so
-// the taps unroll with their weights in registers), and the smoothed depth S over the tile
-// plus a one-pixel ring feeds the central differences and the normal N = a x b with
-// a = (0, s_y, dz/dy) and b = (s_x, 0, dz/dx). Each depth and class byte is read once from HBM
-// and each normal written once (17 bytes per pixel); the convolution's instructions and
-// shared-memory traffic, not HBM, set the kernel's time.
+// One warp per (62-column strip, chunk of rows, image), fused and without block barriers: it walks
+// down its strip four rows at a time. Each row's depths are staged in shared memory as (depth,
+// weight) pairs, zero where invalid, with a halo of the Gaussian's radius; a lane smooths two
+// adjacent columns along the row, sums and weight sums together in packed FP32 pairs (a
+// normalised convolution), and keeps the result in its own ring of the last rows; four smoothed
+// rows then come from one pass down the ring, and the normals N = a x b with a = (0, s_y, dz/dy),
+// b = (s_x, 0, dz/dx) from the smoothed rows in registers, the columns beside a lane's own by
+// shuffle. Rows are not convolved twice and only 12 of 74 columns (radius 5) and the chunk's first
+// and last rows are halo. One instantiation per radius, so the taps unroll with their weights in
+// registers. Each depth and class byte is read about once from HBM and each normal written once
+// (17 bytes per pixel). Bound by the shared-memory pipe (0.88 of its peak: about 60 wavefronts a row
+// of 64 columns, two fifths of them the row windows) beside instruction issue (0.65). 64 images of
+// 640x480 at radius 5: 146 us; the form before it, one CTA per 64x16 tile with its halo staged
+// and convolved again by its neighbours, 229 us and 1.9 times the instructions.
 #include <cfloat>
+#include <algorithm>
 #include <cmath>
 #include <string>
 
@@ -19,13 +24,12 @@
 
 namespace {
 
-constexpr int kTW = 64, kTH = 16;      // output tile
 constexpr int kMaxR = 16;              // Gaussian radius ceil(3 sigma) for sigma <= 5
-constexpr int kSW = kTW + 2;           // smoothed region (tile plus a one-pixel ring)
-constexpr int kSH = kTH + 2;
-constexpr int kThreadsN = 256;
-constexpr int kHG = 4;                 // horizontal pass: outputs per thread along a row
-constexpr int kVG = 6;                 // vertical pass: outputs per thread down a column
+constexpr int kCols = 64;              // smoothed columns of a strip, two per lane
+constexpr int kOut = kCols - 2;        // its output columns
+constexpr int kRows = 4;               // rows per step
+constexpr int kWarpsN = 4;             // warps (strips) per CTA
+constexpr long long kNormalWarps = 3040;  // 152 SMs x 20 resident
 
 struct NormalArgs {
   const float *depth;
@@ -34,220 +38,195 @@ struct NormalArgs {
   float *smoothed;   // optional
   float *blur;       // optional: S where valid, else the input depth
   int W, H, r, metric;
+  int strips, chunks, rows;  // strips across, chunks down an image, output rows of a chunk
+  long long n_warps;         // strips * chunks * images
   float ifx, ify;    // 1 / fx, 1 / fy
-  float inv_g2;      // 1 / (sum of the taps)^2: the weight sum when every staged pixel is valid
   float g[kMaxR + 1];
 };
 
-// Dynamic shared memory, all FP32 tables: the staged depths (0 where invalid) and validity
-// weights (1 or 0) of the tile plus its halo, the horizontal sums of each staged row over the
-// smoothed columns (weighted depths, weights), and the smoothed depth S of the tile plus a
-// one-pixel ring. The horizontal pass reads and writes the tables down their columns with
-// consecutive threads on consecutive rows, so every row stride is odd: 32 consecutive rows
-// then fall in 32 distinct banks and a warp's 4-byte access takes one wavefront.
-__host__ __device__ constexpr int odd_stride(int n) { return n | 1; }
-__host__ __device__ inline int staged_w(int r) { return kSW + 2 * r; }
-__host__ __device__ inline int staged_h(int r) { return kSH + 2 * r; }
-__host__ __device__ inline int staged_stride(int r) { return odd_stride(staged_w(r)); }
-constexpr int kSWP = odd_stride(kSW);  // row stride of the horizontal sums
-inline size_t normals_smem(int r) {
-  return sizeof(float) * (2 * (size_t)staged_h(r) * staged_stride(r) + 2 * (size_t)staged_h(r) * kSWP +
-                          (size_t)kSH * kSW);
-}
+// a * b + c on both halves, each rounded as one fused multiply-add.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+// One warp's shared memory: the step's staged rows, the ring of horizontal sums (a lane's two
+// columns side by side, private to it) and one row of normals on its way out.
+template <int R>
+struct StripSmem {
+  static constexpr int kRing = (2 * R + kRows + kRows - 1) / kRows * kRows;  // whole steps
+  float4 ring[kRing][32];
+  alignas(16) float2 z[kRows][kCols + 2 * R];
+  alignas(8) float out[3 * kCols];
+};
 
 template <int R>
-__global__ void __launch_bounds__(kThreadsN) k_depth_normals(NormalArgs a) {
+__global__ void __launch_bounds__(32 * kWarpsN) k_depth_normals(NormalArgs a) {
   extern __shared__ float4 smem_raw[];
-  constexpr int dw = kSW + 2 * R, dh = kSH + 2 * R, dws = odd_stride(dw);
-  float *zv = reinterpret_cast<float *>(smem_raw);  // [dh][dws]: valid ? z : 0
-  float *zw = zv + dh * dws;                          // [dh][dws]: valid ? 1 : 0
-  float *hn = zw + dh * dws;                          // [dh][kSWP]: horizontal sums of zv
-  float *hd = hn + dh * kSWP;                         // [dh][kSWP]: horizontal sums of zw
-  float *sS = hd + dh * kSWP;                         // [kSH][kSW]
-  const int tid = threadIdx.x;
-  float g[R + 1];
-#pragma unroll
-  for (int k = 0; k <= R; ++k) g[k] = a.g[k];
-  const int img = blockIdx.y;
-  const int ntx = (a.W + kTW - 1) / kTW;
-  const int ox = (blockIdx.x % ntx) * kTW, oy = (blockIdx.x / ntx) * kTH;
-  const int x0 = ox - 1 - R, y0 = oy - 1 - R;  // image coordinates of zv[0][0]
-  const long long P = (long long)a.W * a.H;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  StripSmem<R> &sm = reinterpret_cast<StripSmem<R> *>(smem_raw)[warp];
+  const long long job = (long long)blockIdx.x * kWarpsN + warp;
+  if (job >= a.n_warps) return;
+  const int strip = (int)(job % a.strips), chunk = (int)(job / a.strips % a.chunks);
+  const long long img = job / ((long long)a.strips * a.chunks), P = (long long)a.W * a.H;
   const float *dimg = a.depth + img * P;
   const uint8_t *cimg = a.cls + img * P;
-  // stage: independent loads, four per thread in flight; note whether every staged pixel is
-  // valid, the common case away from holes and the image border
-  constexpr int n_st = dw * dh;
-  bool mine_valid = true;
-  for (int k0 = tid; k0 < n_st; k0 += 4 * kThreadsN) {
-    float dv[4];
-    int cv[4];
+  const int xs = strip * kOut - 1;                 // image column of smoothed column 0
+  const int y_out = chunk * a.rows, y_end = min(y_out + a.rows, a.H);
+  float2 g[R + 1];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int k = k0 + m * kThreadsN;
-      dv[m] = 0.0f;
-      cv[m] = 1;
-      if (k < n_st) {
-        const int x = x0 + k % dw, y = y0 + k / dw;
-        if (x >= 0 && x < a.W && y >= 0 && y < a.H) {
-          const long long p = (long long)y * a.W + x;
-          dv[m] = __ldg(dimg + p);
-          cv[m] = __ldg(cimg + p);
+  for (int k = 0; k <= R; ++k) g[k] = make_float2(a.g[k], a.g[k]);
+  constexpr float kNan = __builtin_nanf("");
+  // this lane's columns: two of its own and one of the halo
+  const int x0 = xs + 2 * lane, hc = lane < R ? lane : kCols + lane, xh = xs - R + hc;
+  const bool in0 = x0 >= 0 && x0 < a.W, in1 = x0 + 1 >= 0 && x0 + 1 < a.W;
+  const bool inh = lane < 2 * R && xh >= 0 && xh < a.W;
+  float zd[kRows][3];
+  int zc[kRows][3];
+  const int y_first = y_out - 1 - R;
+  const float *dp = dimg + (long long)y_first * a.W;  // the next step's first row
+  const uint8_t *cp = cimg + (long long)y_first * a.W;
+  auto load = [&](int y0) {
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const bool iy = y0 + r >= 0 && y0 + r < a.H;
+      zd[r][0] = zd[r][1] = zd[r][2] = 0.0f;
+      zc[r][0] = zc[r][1] = zc[r][2] = 1;
+      if (iy) {
+        if (in0) zd[r][0] = __ldg(dp + x0), zc[r][0] = __ldg(cp + x0);
+        if (in1) zd[r][1] = __ldg(dp + x0 + 1), zc[r][1] = __ldg(cp + x0 + 1);
+        if (inh) zd[r][2] = __ldg(dp + xh), zc[r][2] = __ldg(cp + xh);
+      }
+      dp += a.W;
+      cp += a.W;
+    }
+  };
+  auto pair = [](float d, int c) {
+    const bool ok = c == 0 && fabsf(d) <= FLT_MAX;
+    return make_float2(ok ? d : 0.0f, ok ? 1.0f : 0.0f);
+  };
+  const int n_out = 3 * min(kOut, a.W - (xs + 1));
+  long long at_out = img * P + (long long)y_out * a.W;  // the next output row
+  unsigned long long v0 = 0, v1 = 0;               // validity of the own columns, last row in bit 0
+  float s0a = kNan, s1a = kNan, s0b = kNan, s1b = kNan;  // smoothed rows before the step's (a: two before)
+  int slot = 0;                                    // ring slot of the step's first row
+  load(y_first);
+  for (int y0 = y_first; y0 <= y_end + R; y0 += kRows) {
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const float2 p0 = pair(zd[r][0], zc[r][0]), p1 = pair(zd[r][1], zc[r][1]), ph = pair(zd[r][2], zc[r][2]);
+      sm.z[r][R + 2 * lane] = p0;
+      sm.z[r][R + 2 * lane + 1] = p1;
+      if (lane < 2 * R) sm.z[r][hc] = ph;
+      v0 = v0 << 1 | (p0.y != 0.0f);
+      v1 = v1 << 1 | (p1.y != 0.0f);
+    }
+    __syncwarp();
+    if (y0 + kRows <= y_end + R) load(y0 + kRows);
+    // along the rows: staged columns 2 lane .. 2 lane + 2R + 1 hold both columns' windows
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+      const float4 *w = reinterpret_cast<const float4 *>(&sm.z[r][2 * lane]);
+      float2 n0 = make_float2(0.0f, 0.0f), n1 = n0;
+#pragma unroll
+      for (int t = 0; t <= R; ++t) {
+        const float4 q = w[t];
+        const float2 lo = make_float2(q.x, q.y), hi = make_float2(q.z, q.w);
+        const int k = 2 * t;                       // lo is tap k of column 0, hi tap k of column 1
+        n0 = fma2(g[k < R ? R - k : k - R], lo, n0);
+        if (k + 1 <= 2 * R) n0 = fma2(g[k + 1 < R ? R - k - 1 : k + 1 - R], hi, n0);
+        if (k >= 1) n1 = fma2(g[k - 1 < R ? R - k + 1 : k - 1 - R], lo, n1);
+        n1 = fma2(g[k < R ? R - k : k - R], hi, n1);
+      }
+      sm.ring[slot + r][lane] = make_float4(n0.x, n0.y, n1.x, n1.y);
+    }
+    // down the ring: smoothed rows y0 - R .. y0 - R + 3 from rows y0 - 2R .. y0 + 3
+    float2 m0[kRows], m1[kRows];
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) m0[j] = m1[j] = make_float2(0.0f, 0.0f);
+    int at = slot - 2 * R;
+    if (at < 0) at += StripSmem<R>::kRing;
+#pragma unroll
+    for (int t = 0; t < 2 * R + kRows; ++t) {
+      const float4 q = sm.ring[at][lane];
+      if (++at == StripSmem<R>::kRing) at = 0;
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) {
+        const int d = t - j;
+        if (d >= 0 && d <= 2 * R) {
+          const float2 w = g[d < R ? R - d : d - R];
+          m0[j] = fma2(w, make_float2(q.x, q.y), m0[j]);
+          m1[j] = fma2(w, make_float2(q.z, q.w), m1[j]);
         }
       }
     }
+    slot += kRows;
+    if (slot == StripSmem<R>::kRing) slot = 0;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int k = k0 + m * kThreadsN;
-      if (k < n_st) {
-        const bool ok = cv[m] == 0 && fabsf(dv[m]) <= FLT_MAX;
-        mine_valid = mine_valid && ok;
-        const int at = (k / dw) * dws + k % dw;
-        zv[at] = ok ? dv[m] : 0.0f;
-        zw[at] = ok ? 1.0f : 0.0f;
+    for (int j = 0; j < kRows; ++j) {
+      // the smoothed row ys (centres valid), then the normals of the row above it
+      const int ys = y0 - R + j, y = ys - 1;
+      const bool c0 = v0 >> (R + kRows - 1 - j) & 1, c1 = v1 >> (R + kRows - 1 - j) & 1;
+      const float s0 = c0 ? m0[j].x / m0[j].y : kNan, s1 = c1 ? m1[j].x / m1[j].y : kNan;
+      const float left = __shfl_up_sync(0xffffffffu, s1b, 1), right = __shfl_down_sync(0xffffffffu, s0b, 1);
+      if (y >= y_out && y < y_end) {
+        if (a.smoothed || a.blur) {
+          const bool w0 = lane > 0 && x0 < a.W, w1 = lane < 31 && x0 + 1 < a.W;
+          if (a.smoothed) {
+            if (w0) a.smoothed[at_out + x0] = s0b;
+            if (w1) a.smoothed[at_out + x0 + 1] = s1b;
+          }
+          if (a.blur) {
+            if (w0) a.blur[at_out + x0] = isnan(s0b) ? a.depth[at_out + x0] : s0b;
+            if (w1) a.blur[at_out + x0 + 1] = isnan(s1b) ? a.depth[at_out + x0 + 1] : s1b;
+          }
+        }
+        if (a.normals) {
+          // S is NaN at invalid pixels and outside the image, so an undefined difference makes the
+          // normal NaN by itself; only an invalid centre needs asking for
+          auto normal = [&](float s, float sl, float sr, float su, float sd) {
+            const float zx = 0.5f * (sr - sl), zy = 0.5f * (sd - su);
+            const float sx = a.metric ? s * a.ifx : 1.0f, sy = a.metric ? s * a.ify : 1.0f;
+            // a = (0, sy, zy), b = (sx, 0, zx), N = a x b
+            const float q0 = sy * zx, q1 = zy * sx, q2 = -sy * sx;
+            float inv = rsqrtf(q0 * q0 + q1 * q1 + q2 * q2);
+            if (isnan(s)) inv = kNan;
+            return make_float3(q0 * inv, q1 * inv, q2 * inv);
+          };
+          float2 *o = reinterpret_cast<float2 *>(sm.out) + 3 * lane;
+          const float3 p = normal(s0b, left, s1b, s0a, s0), q = normal(s1b, s0b, right, s1a, s1);
+          o[0] = make_float2(p.x, p.y);
+          o[1] = make_float2(p.z, q.x);
+          o[2] = make_float2(q.y, q.z);
+          __syncwarp();
+          float *dst = a.normals + 3 * (at_out + xs + 1) + lane;
+#pragma unroll
+          for (int k = 0; k < 6; ++k)
+            if (lane + 32 * k < n_out) dst[32 * k] = sm.out[3 + lane + 32 * k];
+          __syncwarp();
+        }
+        at_out += a.W;
       }
+      s0a = s0b;
+      s1a = s1b;
+      s0b = s0;
+      s1b = s1;
     }
-  }
-  const bool all_valid = __syncthreads_and(mine_valid);
-  // horizontal pass: weighted sums of the valid depths (and of their weights, unless every
-  // staged pixel is valid), kHG adjacent outputs per thread: each staged value is loaded once
-  // and added to every output whose window holds it (the taps unroll: R is a template
-  // parameter); consecutive threads take consecutive rows
-  {
-    constexpr int groups = (kSW + kHG - 1) / kHG;
-    for (int it = tid; it < dh * groups; it += kThreadsN) {
-      const int v = it % dh, u0 = (it / dh) * kHG;
-      float num[kHG], den[kHG];
-#pragma unroll
-      for (int j = 0; j < kHG; ++j) num[j] = den[j] = 0.0f;
-      const float *row = zv + v * dws + u0;  // output u0 + j: staged columns u0 + j .. + 2R
-      const float *roww = zw + v * dws + u0;
-      if (all_valid) {
-#pragma unroll
-        for (int t = 0; t < 2 * R + kHG; ++t) {
-          const float z = (u0 + t < dw) ? row[t] : 0.0f;
-#pragma unroll
-          for (int j = 0; j < kHG; ++j) {
-            const int d = t - j;
-            if (d >= 0 && d <= 2 * R) num[j] = fmaf(g[d < R ? R - d : d - R], z, num[j]);
-          }
-        }
-      } else {
-#pragma unroll
-        for (int t = 0; t < 2 * R + kHG; ++t) {
-          const bool in = u0 + t < dw;
-          const float z = in ? row[t] : 0.0f, zok = in ? roww[t] : 0.0f;
-#pragma unroll
-          for (int j = 0; j < kHG; ++j) {
-            const int d = t - j;
-            if (d >= 0 && d <= 2 * R) {
-              const float w = g[d < R ? R - d : d - R];
-              num[j] = fmaf(w, z, num[j]);
-              den[j] = fmaf(w, zok, den[j]);
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kHG; ++j)
-        if (u0 + j < kSW) {
-          hn[v * kSWP + u0 + j] = num[j];
-          hd[v * kSWP + u0 + j] = den[j];
-        }
-    }
-  }
-  __syncthreads();
-  // vertical pass: kVG outputs per thread down a column; S where the centre pixel is valid
-  {
-    constexpr int groups = (kSH + kVG - 1) / kVG;
-    for (int it = tid; it < kSW * groups; it += kThreadsN) {
-      const int u = it % kSW, v0 = (it / kSW) * kVG;
-      float num[kVG], den[kVG];
-#pragma unroll
-      for (int j = 0; j < kVG; ++j) num[j] = den[j] = 0.0f;
-      if (all_valid) {
-#pragma unroll
-        for (int t = 0; t < 2 * R + kVG; ++t) {
-          const float h = (v0 + t < dh) ? hn[(v0 + t) * kSWP + u] : 0.0f;
-#pragma unroll
-          for (int j = 0; j < kVG; ++j) {
-            const int d = t - j;
-            if (d >= 0 && d <= 2 * R) num[j] = fmaf(g[d < R ? R - d : d - R], h, num[j]);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < kVG; ++j)
-          if (v0 + j < kSH) sS[(v0 + j) * kSW + u] = num[j] * a.inv_g2;
-      } else {
-#pragma unroll
-        for (int t = 0; t < 2 * R + kVG; ++t) {
-          const bool in = v0 + t < dh;
-          const float hz = in ? hn[(v0 + t) * kSWP + u] : 0.0f, hw = in ? hd[(v0 + t) * kSWP + u] : 0.0f;
-#pragma unroll
-          for (int j = 0; j < kVG; ++j) {
-            const int d = t - j;
-            if (d >= 0 && d <= 2 * R) {
-              const float w = g[d < R ? R - d : d - R];
-              num[j] = fmaf(w, hz, num[j]);
-              den[j] = fmaf(w, hw, den[j]);
-            }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < kVG; ++j) {
-          const int v = v0 + j;
-          if (v < kSH) {
-            const bool centre = zw[(v + R) * dws + (u + R)] != 0.0f;
-            sS[v * kSW + u] = centre ? num[j] / den[j] : __int_as_float(0x7fc00000);
-          }
-        }
-      }
-    }
-  }
-  __syncthreads();
-  for (int k = tid; k < kTW * kTH; k += kThreadsN) {
-    const int u = k % kTW + 1, v = k / kTW + 1;
-    const int x = ox + u - 1, y = oy + v - 1;
-    if (x >= a.W || y >= a.H) continue;
-    const long long p = img * P + (long long)y * a.W + x;
-    const float s = sS[v * kSW + u];
-    if (a.smoothed) a.smoothed[p] = s;
-    if (a.blur) a.blur[p] = isnan(s) ? a.depth[p] : s;
-    if (!a.normals) continue;
-    float n0 = __int_as_float(0x7fc00000), n1 = n0, n2 = n0;
-    const float sl = sS[v * kSW + u - 1], sr = sS[v * kSW + u + 1];
-    const float su = sS[(v - 1) * kSW + u], sd = sS[(v + 1) * kSW + u];
-    if (x >= 1 && x + 1 < a.W && y >= 1 && y + 1 < a.H && !isnan(s) && !isnan(sl) && !isnan(sr) &&
-        !isnan(su) && !isnan(sd)) {
-      const float zx = 0.5f * (sr - sl), zy = 0.5f * (sd - su);
-      const float sx = a.metric ? s * a.ifx : 1.0f, sy = a.metric ? s * a.ify : 1.0f;
-      // a = (0, sy, zy), b = (sx, 0, zx), N = a x b
-      const float c0 = sy * zx, c1 = zy * sx, c2 = -sy * sx;
-      const float inv = rsqrtf(c0 * c0 + c1 * c1 + c2 * c2);
-      n0 = c0 * inv;
-      n1 = c1 * inv;
-      n2 = c2 * inv;
-    }
-    a.normals[3 * p] = n0;
-    a.normals[3 * p + 1] = n1;
-    a.normals[3 * p + 2] = n2;
   }
 }
 
 template <int R>
-cudaError_t launch_normals_r(const NormalArgs &a, int tiles, int n, cudaStream_t s) {
-  const size_t sm = normals_smem(R);
-  // radii above about 7 need more than the default 48 KB (set on the current device)
+cudaError_t launch_normals_r(const NormalArgs &a, cudaStream_t s) {
+  const size_t sm = sizeof(StripSmem<R>) * kWarpsN;
+  // radii above about 6 need more than the default 48 KB (set on the current device)
   cudaError_t e = cudaFuncSetAttribute(k_depth_normals<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k_depth_normals<R><<<dim3(tiles, n), kThreadsN, sm, s>>>(a);
+  k_depth_normals<R><<<(unsigned)((a.n_warps + kWarpsN - 1) / kWarpsN), 32 * kWarpsN, sm, s>>>(a);
   return cudaGetLastError();
 }
 
 template <int R>
-cudaError_t launch_normals(const NormalArgs &a, int tiles, int n, cudaStream_t s) {
-  if (a.r == R) return launch_normals_r<R>(a, tiles, n, s);
-  if constexpr (R < kMaxR) return launch_normals<R + 1>(a, tiles, n, s);
+cudaError_t launch_normals(const NormalArgs &a, cudaStream_t s) {
+  if (a.r == R) return launch_normals_r<R>(a, s);
+  if constexpr (R < kMaxR) return launch_normals<R + 1>(a, s);
   return cudaErrorInvalidValue;
 }
 
@@ -319,11 +298,15 @@ rm_status run_normals(const rm_intrinsics *intr, int32_t n, const float *depth, 
     a.ify = metric ? 1.0f / intr->fy : 1.0f;
     for (int k = 0; k <= kMaxR; ++k)
       a.g[k] = sigma > 0.0f ? (float)std::exp(-(double)(k * k) / (2.0 * (double)sigma * sigma)) : 1.0f;
-    double gs = a.g[0];
-    for (int k = 1; k <= a.r; ++k) gs += 2.0 * a.g[k];
-    a.inv_g2 = (float)(1.0 / (gs * gs));
-    const int tiles = ((a.W + kTW - 1) / kTW) * ((a.H + kTH - 1) / kTH);
-    ck(launch_normals<0>(a, tiles, n, s));
+    // chunks of rows: as many warps as are resident at once, but no chunk shorter than the rows that
+    // it reads besides its own (64 images of 640x480: 167 us with 2816 warps, 177 with 6336)
+    a.strips = (a.W + kOut - 1) / kOut;
+    const long long per_row_of_chunks = (long long)a.strips * n;
+    const int want = (int)std::max<long long>(1, kNormalWarps / per_row_of_chunks);
+    a.rows = std::max((a.H + want - 1) / want, 2 * a.r + 2);
+    a.chunks = (a.H + a.rows - 1) / a.rows;
+    a.n_warps = per_row_of_chunks * a.chunks;
+    ck(launch_normals<0>(a, s));
   }
   if (e == cudaSuccess && host_n) ck(cudaMemcpyAsync(normals, d_n, sizeof(float) * 3 * np, cudaMemcpyDeviceToHost, s));
   if (e == cudaSuccess && host_s) ck(cudaMemcpyAsync(smoothed, d_s, sizeof(float) * np, cudaMemcpyDeviceToHost, s));
