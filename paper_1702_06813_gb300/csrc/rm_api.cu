@@ -1230,6 +1230,46 @@ rm_status write_pose(double *pose_out, const double *T) {
 
 }  // namespace
 
+namespace {
+
+// One pool a device, made on first use; pools are safe to use from several threads and streams.
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+
+cudaError_t scratch_pool(cudaMemPool_t *pool) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t made = nullptr;
+    if ((e = cudaMemPoolCreate(&made, &props)) != cudaSuccess) return e;
+    uint64_t kept = rmapi::kScratchKept;
+    if ((e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &kept)) != cudaSuccess) {
+      cudaMemPoolDestroy(made);
+      return e;
+    }
+    g_pool[dev] = made;
+  }
+  *pool = g_pool[dev];
+  return cudaSuccess;
+}
+
+// Gives the unused scratch of a device back to the system.
+void scratch_trim(int dev) {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (dev >= 0 && dev < kMaxDevices && g_pool[dev]) cudaMemPoolTrimTo(g_pool[dev], 0);
+}
+
+}  // namespace
+
 namespace rmapi {
 
 int map_device(const rm_map *m) { return m->device; }
@@ -1256,6 +1296,12 @@ void set_error(const std::string &msg) { g_err = msg; }
 rm_status check_intrinsics(const rm_intrinsics *in) { return check_intr(in); }
 
 bool is_device_pointer(const void *p) { return on_device(p); }
+
+cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s) {
+  cudaMemPool_t pool = nullptr;
+  const cudaError_t e = scratch_pool(&pool);
+  return e == cudaSuccess ? cudaMallocFromPoolAsync(p, bytes, pool, s) : e;
+}
 
 }  // namespace rmapi
 
@@ -1376,6 +1422,7 @@ void rm_map_destroy(rm_map *m) {
   cudaFree(m->d_cl_ids);
   cudaFree(m->arena);
   cudaFree(m->zbuf);
+  scratch_trim(m->device);
   if (m->aux_stream) cudaStreamDestroy(m->aux_stream);
   if (m->ev_fork) cudaEventDestroy(m->ev_fork);
   if (m->ev_join) cudaEventDestroy(m->ev_join);
@@ -1437,7 +1484,7 @@ rm_status rm_map_set_vertex_normals(rm_map *m, const float *normals, const doubl
   if (!m->d_vn) RM_CK(cudaMalloc((void **)&m->d_vn, sizeof(float4) * (size_t)V));
   float *buf = nullptr;
   const size_t nb = sizeof(float) * 3 * (size_t)V;
-  RM_CK(cudaMallocAsync((void **)&buf, nb + sizeof(R), s));
+  RM_CK(rmapi::scratch_alloc((void **)&buf, nb + sizeof(R), s));
   rm_status st = RM_OK;
   auto run = [&]() -> rm_status {
     RM_CK(cudaMemcpyAsync(buf, normals, nb, on_device(normals) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
@@ -1509,7 +1556,8 @@ rm_status rm_cost_grad_vertices(rm_map *m, const rm_scan *scan, const double *po
   RM_CK(cudaSetDevice(m->device));
   cudaStream_t s = (cudaStream_t)stream;
   const long long P = (long long)in->width * in->height;
-  const int chunk = (int)std::max<long long>(1, std::min<long long>(16, (1LL << 28) / std::max<long long>(P, 1)));
+  const int chunk = (int)std::max<long long>(
+      1, std::min<long long>(std::min<long long>(16, n), (1LL << 28) / std::max<long long>(P, 1)));
   const bool host_g = !on_device(grad_v), host_p = n > 0 && !on_device(poses);
   const bool host_sd = !on_device(scan->depth), host_sc = !on_device(scan->cls);
   const bool host_rays = in->model == RM_RAYTABLE && !on_device(in->rays);
@@ -1528,7 +1576,7 @@ rm_status rm_cost_grad_vertices(rm_map *m, const rm_scan *scan, const double *po
   const size_t o_id = take(sizeof(int) * P * chunk), o_d = take(sizeof(float) * P * chunk);
   const size_t o_b = take(sizeof(float) * 2 * P * chunk);
   unsigned char *buf = nullptr;
-  RM_CK(cudaMallocAsync((void **)&buf, off, s));
+  RM_CK(rmapi::scratch_alloc((void **)&buf, off, s));
   double *d_g = host_g ? reinterpret_cast<double *>(buf + o_g) : grad_v;
   double *d_p = reinterpret_cast<double *>(buf + o_p);
   const float *d_sd = host_sd ? reinterpret_cast<float *>(buf + o_sd) : scan->depth;
@@ -1593,7 +1641,7 @@ rm_status rm_cost_sweep(rm_map *m, const rm_scan *scan, const double *pose, int3
   RM_CK(cudaSetDevice(m->device));
   cudaStream_t s = (cudaStream_t)stream;
   double *buf = nullptr;
-  RM_CK(cudaMallocAsync((void **)&buf, sizeof(double) * (16 + 38 * (size_t)n), s));
+  RM_CK(rmapi::scratch_alloc((void **)&buf, sizeof(double) * (16 + 38 * (size_t)n), s));
   double *d_base = buf, *d_rep = buf + 16, *d_tw = d_rep + 16 * (size_t)n, *d_poses = d_tw + 6 * (size_t)n;
   auto body = [&]() -> rm_status {
     RM_CK(cudaMemcpyAsync(d_base, pose, sizeof(double) * 16,
@@ -1623,7 +1671,7 @@ rm_status rm_pose_retract(const double *poses, const double *twists, int32_t n, 
   }
   double *buf = nullptr;
   size_t per = 16 + 6 + 16 + 36;
-  RM_CK(cudaMallocAsync((void **)&buf, sizeof(double) * per * n, s));
+  RM_CK(rmapi::scratch_alloc((void **)&buf, sizeof(double) * per * n, s));
   double *bp = buf, *bt = buf + 16 * (size_t)n, *bo = bt + 6 * (size_t)n, *bj = bo + 16 * (size_t)n;
   rm_status st = RM_OK;
   auto run = [&]() -> rm_status {
@@ -1653,7 +1701,7 @@ rm_status rm_twist_grad(const double *twists, const double *grads, const double 
     return RM_OK;
   }
   double *buf = nullptr;
-  RM_CK(cudaMallocAsync((void **)&buf, sizeof(double) * 19 * (size_t)n, s));
+  RM_CK(rmapi::scratch_alloc((void **)&buf, sizeof(double) * 19 * (size_t)n, s));
   double *bt = buf, *bg = bt + 6 * (size_t)n, *bs = bg + 6 * (size_t)n, *bo = bs + (size_t)n;
   auto run = [&]() -> rm_status {
     RM_CK(cudaMemcpyAsync(bt, twists, sizeof(double) * 6 * n, dt ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));

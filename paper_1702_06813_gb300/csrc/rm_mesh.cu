@@ -1,18 +1,20 @@
 // rm_mesh.cu -- rm_meshify: the labelled interface mesh of one range image (Sec. IV.A, Fig. 5).
 //
-// Four kernels, all elementwise or per-block, in a fixed order so that the output is the same
-// run to run (row-major block order, no atomics):
-//   k_mesh_points  per grid pixel: class (return / no-return / dead), its FP32 camera-frame
-//                  point (returns at their depth, no-returns at the maximal range), and the
-//                  world vertex through the pose in FP64 (rounded once to FP32)
-//   k_mesh_quads   per 2x2 block of grid pixels: dropped when a pixel is dead, else FU when a
-//                  pixel is a no-return or a side or the diagonal is longer than the limit
-//                  (squared lengths in FP32), else FO; plus the kept count of each CTA
-//   k_mesh_scan    one CTA: exclusive scan of the per-CTA counts (the face offsets)
+// Two kernels (three for large images), in a fixed order so that the output is the same run to run
+// (row-major block order, no atomics):
+//   k_mesh_blocks  per grid pixel: the world vertex through the pose in FP64 (rounded once to
+//                  FP32); per 2x2 block of grid pixels: dropped when a pixel is dead, else FU when
+//                  a pixel is a no-return or a side or the diagonal is longer than the limit
+//                  (squared lengths in FP32), else FO; plus the kept count of each CTA. The
+//                  camera-frame points of a block's corners are computed again for each block
+//                  rather than kept: their inputs are in L1.
+//   k_mesh_scan    large images only (more than kScanCtas CTAs): exclusive scan of the counts
 //   k_mesh_emit    per block: two triangles (v00, v10, v11), (v00, v11, v01) at the block's
-//                  rank among the kept blocks
+//                  rank among the kept blocks; each CTA adds up the counts before its own
 // The arithmetic that decides a label uses explicitly rounded operations (no contraction), so
-// the decision is the same as any IEEE FP32 evaluation in the same order.
+// the decision is the same as any IEEE FP32 evaluation in the same order. One 640x480 image is
+// launches and latency: 352 -> 130 us a call, most of it the scratch that used to be allocated
+// and, at the call's synchronisation, given back to the system each time.
 #include <cfloat>
 #include <cmath>
 #include <string>
@@ -34,25 +36,23 @@ struct MeshArgs {
   const double *Tdev;   // or the pose in device memory (16 doubles)
   float max_range, lim;  // lim = max_edge^2 (FP32)
   float *vertices;
-  float4 *pc;           // camera-frame points
-  uint8_t *kind;        // 0 return, 1 no-return, 2 dead
   uint8_t *qcode;       // per block: 0 dropped, 1 FO, 2 FU
   int *cta_count;
-  long long *cta_off;   // exclusive offsets (in blocks), then the total
-  int n_cta;
+  long long *cta_off;   // exclusive offsets (in blocks), or null: k_mesh_emit adds up cta_count
+  int n_cta;            // CTAs that hold blocks
   int32_t *faces;
   uint8_t *labels;
   long long *n_faces;
 };
 
-__global__ void __launch_bounds__(256) k_mesh_points(MeshArgs a) {
-  const long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= (long long)a.Ws * a.Hs) return;
-  const int i = (int)(v % a.Ws), j = (int)(v / a.Ws);
+constexpr int kScanCtas = 2048;
+
+// Kind (0 return, 1 no-return, 2 dead) and camera-frame point of grid pixel (i, j).
+__device__ __forceinline__ int mesh_point(const MeshArgs &a, int i, int j, float3 &pc) {
   const int x = i * a.step, y = j * a.step;
   const long long p = (long long)y * a.W + x;
-  const float d = a.depth[p];
-  const int c = a.cls[p];
+  const float d = __ldg(a.depth + p);
+  const int c = __ldg(a.cls + p);
   const int k = (c > 1 || !(fabsf(d) <= FLT_MAX)) ? 2 : c;
   const float r = k == 0 ? d : (k == 1 ? a.max_range : 0.0f);
   float rx, ry, rz;
@@ -66,43 +66,44 @@ __global__ void __launch_bounds__(256) k_mesh_points(MeshArgs a) {
     ry = q[1];
     rz = q[2];
   }
-  const float px = __fmul_rn(r, rx), py = __fmul_rn(r, ry), pz = __fmul_rn(r, rz);
-  a.pc[v] = make_float4(px, py, pz, 0.0f);
-  a.kind[v] = (uint8_t)k;
-  for (int q = 0; q < 3; ++q) {
-    const double *m = (a.Tdev ? a.Tdev : a.T) + 4 * q;
-    double w = m[3];  // dead pixels stay at the sensor origin (unreferenced)
-    if (k != 2)
-      w = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(m[0], (double)px), __dmul_rn(m[1], (double)py)),
-                              __dmul_rn(m[2], (double)pz)),
-                    m[3]);
-    a.vertices[3 * v + q] = (float)w;
-  }
+  pc = make_float3(__fmul_rn(r, rx), __fmul_rn(r, ry), __fmul_rn(r, rz));
+  return k;
 }
 
-__device__ __forceinline__ float edge2(const float4 &a, const float4 &b) {
+__device__ __forceinline__ float edge2(const float3 &a, const float3 &b) {
   const float dx = __fsub_rn(a.x, b.x), dy = __fsub_rn(a.y, b.y), dz = __fsub_rn(a.z, b.z);
   return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-__global__ void __launch_bounds__(kQuadThreads) k_mesh_quads(MeshArgs a) {
-  const int qw = a.Ws - 1;
-  const long long nq = (long long)qw * (a.Hs - 1);
-  const long long q = (long long)blockIdx.x * kQuadThreads + threadIdx.x;
+// Thread v: grid pixel v, which is the first corner of a block unless it ends its row or column.
+__global__ void __launch_bounds__(kQuadThreads) k_mesh_blocks(MeshArgs a) {
+  const long long v = (long long)blockIdx.x * kQuadThreads + threadIdx.x;
+  const bool on = v < (long long)a.Ws * a.Hs;
+  const int i = on ? (int)(v % a.Ws) : 0, j = on ? (int)(v / a.Ws) : 0;
   int code = 0;
-  if (q < nq) {
-    const int i = (int)(q % qw), j = (int)(q / qw);
-    const long long v00 = (long long)j * a.Ws + i, v10 = v00 + 1, v01 = v00 + a.Ws, v11 = v01 + 1;
-    const int k00 = a.kind[v00], k10 = a.kind[v10], k01 = a.kind[v01], k11 = a.kind[v11];
-    if (k00 != 2 && k10 != 2 && k01 != 2 && k11 != 2) {
-      bool fu = k00 == 1 || k10 == 1 || k01 == 1 || k11 == 1;
-      const float4 A = a.pc[v00], B = a.pc[v10], C = a.pc[v11], D = a.pc[v01];
-      if (edge2(A, B) > a.lim || edge2(B, C) > a.lim || edge2(C, D) > a.lim || edge2(D, A) > a.lim ||
-          edge2(A, C) > a.lim)
-        fu = true;
-      code = fu ? 2 : 1;
+  if (on) {
+    float3 A;
+    const int k00 = mesh_point(a, i, j, A);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const double *m = (a.Tdev ? a.Tdev : a.T) + 4 * q;
+      double w = m[3];  // dead pixels stay at the sensor origin (unreferenced)
+      if (k00 != 2)
+        w = __dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(m[0], (double)A.x), __dmul_rn(m[1], (double)A.y)),
+                                __dmul_rn(m[2], (double)A.z)),
+                      m[3]);
+      a.vertices[3 * v + q] = (float)w;
     }
-    a.qcode[q] = (uint8_t)code;
+    if (i + 1 < a.Ws && j + 1 < a.Hs) {
+      float3 B, C, D;
+      const int k10 = mesh_point(a, i + 1, j, B), k11 = mesh_point(a, i + 1, j + 1, C), k01 = mesh_point(a, i, j + 1, D);
+      if (k00 != 2 && k10 != 2 && k01 != 2 && k11 != 2) {
+        const bool fu = k00 == 1 || k10 == 1 || k01 == 1 || k11 == 1 || edge2(A, B) > a.lim || edge2(B, C) > a.lim ||
+                        edge2(C, D) > a.lim || edge2(D, A) > a.lim || edge2(A, C) > a.lim;
+        code = fu ? 2 : 1;
+      }
+    }
+    a.qcode[v] = (uint8_t)code;
   }
   const int kept = __syncthreads_count(code != 0);
   if (threadIdx.x == 0) a.cta_count[blockIdx.x] = kept;
@@ -139,28 +140,39 @@ __global__ void __launch_bounds__(1024) k_mesh_scan(MeshArgs a) {
     if (threadIdx.x == 1023) carry = before + c;
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    a.cta_off[a.n_cta] = carry;
-    *a.n_faces = 2 * carry;
-  }
 }
 
 __global__ void __launch_bounds__(kQuadThreads) k_mesh_emit(MeshArgs a) {
   __shared__ int wcount[kQuadThreads / 32];
-  const int qw = a.Ws - 1;
-  const long long nq = (long long)qw * (a.Hs - 1);
-  const long long q = (long long)blockIdx.x * kQuadThreads + threadIdx.x;
-  const int code = q < nq ? a.qcode[q] : 0;
+  __shared__ long long wbefore[kQuadThreads / 32];
+  const long long v = (long long)blockIdx.x * kQuadThreads + threadIdx.x;
+  const bool on = v < (long long)a.Ws * a.Hs;
+  const int code = on ? a.qcode[v] : 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned m = __ballot_sync(0xffffffffu, code != 0);
-  if (lane == 0) wcount[warp] = __popc(m);
+  long long before = 0;  // kept blocks of the CTAs before this one
+  if (!a.cta_off) {
+    for (int k = threadIdx.x; k < (int)blockIdx.x; k += kQuadThreads) before += a.cta_count[k];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) before += __shfl_xor_sync(0xffffffffu, before, off);
+  }
+  if (lane == 0) {
+    wcount[warp] = __popc(m);
+    wbefore[warp] = before;
+  }
   __syncthreads();
   int rank = __popc(m & ((1u << lane) - 1));
   for (int w = 0; w < warp; ++w) rank += wcount[w];
+  if (a.cta_off) {
+    before = a.cta_off[blockIdx.x];
+  } else {
+    before = 0;
+    for (int w = 0; w < kQuadThreads / 32; ++w) before += wbefore[w];
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kQuadThreads - 1) *a.n_faces = 2 * (before + rank + (code != 0));
   if (code == 0) return;
-  const int i = (int)(q % qw), j = (int)(q / qw);
-  const int v00 = j * a.Ws + i, v10 = v00 + 1, v01 = v00 + a.Ws, v11 = v01 + 1;
-  const long long f = 2 * (a.cta_off[blockIdx.x] + rank);
+  const int v00 = (int)v, v10 = v00 + 1, v01 = v00 + a.Ws, v11 = v01 + 1;
+  const long long f = 2 * (before + rank);
   int32_t *o = a.faces + 3 * f;
   o[0] = v00;
   o[1] = v10;
@@ -210,7 +222,7 @@ extern "C" rm_status rm_meshify(const rm_scan *scan, const double *pose,
   const bool host_f = NQ > 0 && !rmapi::is_device_pointer(faces);
   const bool host_l = NQ > 0 && !rmapi::is_device_pointer(labels);
   const bool host_n = !rmapi::is_device_pointer(n_faces);
-  const int n_cta = (int)std::max<long long>(1, (NQ + kQuadThreads - 1) / kQuadThreads);
+  const int n_cta = (int)((NV + kQuadThreads - 1) / kQuadThreads);
   // one stream-ordered scratch block: staged inputs and outputs, then the work arrays
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -223,11 +235,11 @@ extern "C" rm_status rm_meshify(const rm_scan *scan, const double *pose,
   const size_t o_v = host_v ? take(sizeof(float) * 3 * NV) : 0;
   const size_t o_f = host_f ? take(sizeof(int32_t) * 6 * NQ) : 0;
   const size_t o_l = host_l ? take(2 * NQ) : 0;
-  const size_t o_pc = take(sizeof(float4) * NV), o_k = take(NV), o_q = take(std::max<long long>(NQ, 1));
-  const size_t o_cc = take(sizeof(int) * n_cta), o_co = take(sizeof(long long) * (n_cta + 1));
+  const size_t o_q = take(NV), o_cc = take(sizeof(int) * n_cta);
+  const size_t o_co = n_cta > kScanCtas ? take(sizeof(long long) * n_cta) : 0;
   const size_t o_n = take(sizeof(long long));
   unsigned char *buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void **)&buf, off, s);
+  cudaError_t e = rmapi::scratch_alloc((void **)&buf, off, s);
   if (e != cudaSuccess) return mf_fail(RM_ENOMEM, std::string("rm_meshify: ") + cudaGetErrorString(e));
   auto ck = [&](cudaError_t x) {
     if (e == cudaSuccess) e = x;
@@ -251,11 +263,9 @@ extern "C" rm_status rm_meshify(const rm_scan *scan, const double *pose,
   a.max_range = prm->max_range;
   a.lim = prm->max_edge * prm->max_edge;
   a.vertices = host_v ? reinterpret_cast<float *>(buf + o_v) : vertices;
-  a.pc = reinterpret_cast<float4 *>(buf + o_pc);
-  a.kind = buf + o_k;
   a.qcode = buf + o_q;
   a.cta_count = reinterpret_cast<int *>(buf + o_cc);
-  a.cta_off = reinterpret_cast<long long *>(buf + o_co);
+  a.cta_off = n_cta > kScanCtas ? reinterpret_cast<long long *>(buf + o_co) : nullptr;
   a.n_cta = n_cta;
   a.faces = host_f ? reinterpret_cast<int32_t *>(buf + o_f) : faces;
   a.labels = host_l ? buf + o_l : labels;
@@ -264,18 +274,14 @@ extern "C" rm_status rm_meshify(const rm_scan *scan, const double *pose,
   if (host_c) ck(cudaMemcpyAsync((void *)a.cls, scan->cls, P, cudaMemcpyHostToDevice, s));
   if (host_r) ck(cudaMemcpyAsync((void *)a.rays, in.rays, sizeof(float) * 3 * P, cudaMemcpyHostToDevice, s));
   if (e == cudaSuccess) {
-    k_mesh_points<<<(unsigned)((NV + 255) / 256), 256, 0, s>>>(a);
+    k_mesh_blocks<<<n_cta, kQuadThreads, 0, s>>>(a);
     ck(cudaGetLastError());
   }
-  if (e == cudaSuccess) {
-    k_mesh_quads<<<n_cta, kQuadThreads, 0, s>>>(a);
-    ck(cudaGetLastError());
-  }
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && a.cta_off) {
     k_mesh_scan<<<1, 1024, 0, s>>>(a);
     ck(cudaGetLastError());
   }
-  if (e == cudaSuccess && NQ > 0) {
+  if (e == cudaSuccess) {
     k_mesh_emit<<<n_cta, kQuadThreads, 0, s>>>(a);
     ck(cudaGetLastError());
   }

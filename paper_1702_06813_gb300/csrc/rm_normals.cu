@@ -276,11 +276,11 @@ rm_status run_normals(const rm_intrinsics *intr, int32_t n, const float *depth, 
   auto ck = [&](cudaError_t x) {
     if (e == cudaSuccess) e = x;
   };
-  if (host_d) ck(cudaMallocAsync((void **)&d_d, sizeof(float) * np, s));
-  if (host_c) ck(cudaMallocAsync((void **)&d_c, np, s));
-  if (host_n) ck(cudaMallocAsync((void **)&d_n, sizeof(float) * 3 * np, s));
-  if (host_s) ck(cudaMallocAsync((void **)&d_s, sizeof(float) * np, s));
-  if (host_b) ck(cudaMallocAsync((void **)&d_b, sizeof(float) * np, s));
+  if (host_d) ck(rmapi::scratch_alloc((void **)&d_d, sizeof(float) * np, s));
+  if (host_c) ck(rmapi::scratch_alloc((void **)&d_c, np, s));
+  if (host_n) ck(rmapi::scratch_alloc((void **)&d_n, sizeof(float) * 3 * np, s));
+  if (host_s) ck(rmapi::scratch_alloc((void **)&d_s, sizeof(float) * np, s));
+  if (host_b) ck(rmapi::scratch_alloc((void **)&d_b, sizeof(float) * np, s));
   if (e == cudaSuccess && host_d) ck(cudaMemcpyAsync(d_d, depth, sizeof(float) * np, cudaMemcpyHostToDevice, s));
   if (e == cudaSuccess && host_c) ck(cudaMemcpyAsync(d_c, cls, np, cudaMemcpyHostToDevice, s));
   if (e == cudaSuccess) {

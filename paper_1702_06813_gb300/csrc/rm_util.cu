@@ -92,7 +92,7 @@ extern "C" rm_status rm_scan_from_range(const float *range, int64_t n, float ran
   const size_t nb = (size_t)n;
   const size_t bytes = (hr ? 4 * nb : 0) + (hd ? 4 * nb : 0) + (hc ? nb : 0);
   cudaError_t e = cudaSuccess;
-  if (bytes) e = cudaMallocAsync((void **)&buf, bytes, s);
+  if (bytes) e = rmapi::scratch_alloc((void **)&buf, bytes, s);
   if (e != cudaSuccess) return ut_fail(RM_ENOMEM, std::string("rm_scan_from_range: ") + cudaGetErrorString(e));
   unsigned char *p = buf;
   const float *d_r = range;
@@ -125,7 +125,7 @@ extern "C" rm_status rm_pose_from_x(const double *X, int32_t n, double *poses, v
   const bool hx = !rmapi::is_device_pointer(X), ht = !rmapi::is_device_pointer(poses);
   double *buf = nullptr;
   cudaError_t e = cudaSuccess;
-  if (hx || ht) e = cudaMallocAsync((void **)&buf, sizeof(double) * 22 * (size_t)n, s);
+  if (hx || ht) e = rmapi::scratch_alloc((void **)&buf, sizeof(double) * 22 * (size_t)n, s);
   if (e != cudaSuccess) return ut_fail(RM_ENOMEM, std::string("rm_pose_from_x: ") + cudaGetErrorString(e));
   const double *d_x = hx ? buf : X;
   double *d_t = ht ? buf + 6 * (size_t)n : poses;
