@@ -88,9 +88,10 @@ struct rm_map {
   float4 *d_cl_pos = nullptr;
   uchar4 *d_cl_tris = nullptr;
   int *d_cl_ids = nullptr;
+  char *scratch = nullptr;  // one allocation: the z-buffers, then the arena
   char *arena = nullptr;
   size_t arena_bytes = 0;
-  unsigned long long *zbuf = nullptr;  // z-buffer keys of a call's waves, see ensure_zbuf
+  unsigned long long *zbuf = nullptr;  // z-buffer keys of a call's waves, see ensure_scratch
   size_t zbuf_keys = 0;
   bool zbuf_empty = false;
   unsigned *status = nullptr;  // status word, pinned host memory
@@ -160,7 +161,7 @@ uint64_t curve_key(uint32_t X[3]) {
 // cannot be started leaves its share to the caller.
 template <class F>
 void in_parts(int64_t n, F f) {
-  const int64_t parts = n < (1 << 17) ? 1 : std::min<int64_t>(8, std::max(1u, std::thread::hardware_concurrency()));
+  const int64_t parts = n < (1 << 13) ? 1 : std::min<int64_t>(8, std::max(1u, std::thread::hardware_concurrency()));
   std::vector<std::thread> pool;
   pool.reserve((size_t)parts);
   int64_t done = 0;
@@ -306,21 +307,34 @@ void build_clusters(const std::vector<float4> &hv, const int32_t *faces, int64_t
   flush();
 }
 
-rm_status ensure_arena(rm_map *m, size_t bytes, cudaStream_t s) {
-  if (bytes <= m->arena_bytes) return RM_OK;
-  RM_CK(cudaStreamSynchronize(s));
-  if (m->batch_exec) {  // the captured batch graph points into the old arena
-    cudaGraphExecDestroy(m->batch_exec);
-    m->batch_exec = nullptr;
-    m->batch_sig.clear();
+// The arena (`bytes`, carved by each call) and the z-buffers of a call's waves (`keys` of them, every
+// one kKeyEmpty), in one allocation that grows with either. The z-buffers are kept between calls:
+// the raster leaves every key it reads empty, so a call pays only for the tiles it touches.
+rm_status ensure_scratch(rm_map *m, size_t bytes, size_t keys, cudaStream_t s) {
+  if (bytes > m->arena_bytes || keys > m->zbuf_keys) {
+    RM_CK(cudaStreamSynchronize(s));
+    if (m->batch_exec) {  // the captured batch graph points into the old arena
+      cudaGraphExecDestroy(m->batch_exec);
+      m->batch_exec = nullptr;
+      m->batch_sig.clear();
+    }
+    m->batch_inputs_valid = false;
+    const size_t want = bytes > m->arena_bytes ? align_up(bytes + bytes / 8, 1 << 20) : m->arena_bytes;
+    const size_t want_keys = std::max(keys, m->zbuf_keys), zbytes = align_up(sizeof(unsigned long long) * want_keys, 256);
+    if (m->scratch) RM_CK(cudaFree(m->scratch));
+    m->scratch = m->arena = nullptr;
+    m->zbuf = nullptr;
+    m->arena_bytes = m->zbuf_keys = 0;
+    RM_CK(cudaMalloc(&m->scratch, zbytes + want));
+    m->zbuf = reinterpret_cast<unsigned long long *>(m->scratch);
+    m->zbuf_keys = want_keys;
+    m->zbuf_empty = false;
+    m->arena = m->scratch + zbytes;
+    m->arena_bytes = want;
   }
-  m->batch_inputs_valid = false;
-  if (m->arena) RM_CK(cudaFree(m->arena));
-  m->arena = nullptr;
-  m->arena_bytes = 0;
-  size_t want = align_up(bytes + bytes / 8, 1 << 20);
-  RM_CK(cudaMalloc(&m->arena, want));
-  m->arena_bytes = want;
+  if (!m->zbuf_empty)  // every byte of kKeyEmpty is 0xff
+    RM_CK(cudaMemsetAsync(m->zbuf, 0xff, sizeof(unsigned long long) * m->zbuf_keys, s));
+  m->zbuf_empty = true;
   return RM_OK;
 }
 
@@ -329,24 +343,6 @@ rm_status ensure_aux(rm_map *m) {
   if (!m->aux_stream) RM_CK(cudaStreamCreateWithFlags(&m->aux_stream, cudaStreamNonBlocking));
   if (!m->ev_fork) RM_CK(cudaEventCreateWithFlags(&m->ev_fork, cudaEventDisableTiming));
   if (!m->ev_join) RM_CK(cudaEventCreateWithFlags(&m->ev_join, cudaEventDisableTiming));
-  return RM_OK;
-}
-
-// The z-buffers of a call's waves (`keys` of them, every one kKeyEmpty): kept between calls, because
-// the raster leaves every key it reads empty, so a call pays only for the tiles it touches.
-rm_status ensure_zbuf(rm_map *m, size_t keys, cudaStream_t s) {
-  if (keys > m->zbuf_keys) {
-    RM_CK(cudaStreamSynchronize(s));
-    if (m->zbuf) RM_CK(cudaFree(m->zbuf));
-    m->zbuf = nullptr;
-    m->zbuf_keys = 0;
-    RM_CK(cudaMalloc(&m->zbuf, sizeof(unsigned long long) * keys));
-    m->zbuf_keys = keys;
-    m->zbuf_empty = false;
-  }
-  if (!m->zbuf_empty)  // every byte of kKeyEmpty is 0xff
-    RM_CK(cudaMemsetAsync(m->zbuf, 0xff, sizeof(unsigned long long) * m->zbuf_keys, s));
-  m->zbuf_empty = true;
   return RM_OK;
 }
 
@@ -584,8 +580,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
     plan.take<unsigned char>((size_t)tg.ntiles * tg.cap * nw * tg.rec_bytes * nbuf);
     plan.take<double>((size_t)tg.ntiles * rmk::kNumVals * nw * nbuf);
     plan.take<int>(2);
-    RM_TRY(ensure_arena(m, plan.off, s));
-    RM_TRY(ensure_zbuf(m, (size_t)P * nw * nbuf, s));
+    RM_TRY(ensure_scratch(m, plan.off, (size_t)P * nw * nbuf, s));
     m->batch_inputs_valid = false;
     // ---- carve it
     Carver cv{m->arena};
@@ -851,8 +846,7 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
     };
     Carver plan{nullptr};
     layout(plan);
-    RM_TRY(ensure_arena(m, plan.off, s));
-    RM_TRY(ensure_zbuf(m, px_total, s));
+    RM_TRY(ensure_scratch(m, plan.off, px_total, s));
     Carver cv{m->arena};
     layout(cv);
     // ---- inputs
@@ -936,7 +930,7 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       b_off += align_up((size_t)tg[p].ntiles * tg[p].cap * tg[p].rec_bytes, 256);
     }
     // the argument blocks are re-sent only when they changed since the last batch call on this arena
-    // (batch_inputs_valid is read here, after ensure_arena: a reallocated arena holds nothing)
+    // (batch_inputs_valid is read here, after ensure_scratch: a reallocated arena holds nothing)
     const bool same_args = m->batch_inputs_valid && m->batch_args.size() == args.size() &&
                            std::memcmp(m->batch_args.data(), args.data(), sizeof(WaveArgs) * n) == 0;
     m->batch_inputs_valid = false;
@@ -1420,8 +1414,7 @@ void rm_map_destroy(rm_map *m) {
   cudaFree(m->d_cl_pos);
   cudaFree(m->d_cl_tris);
   cudaFree(m->d_cl_ids);
-  cudaFree(m->arena);
-  cudaFree(m->zbuf);
+  cudaFree(m->scratch);
   scratch_trim(m->device);
   if (m->aux_stream) cudaStreamDestroy(m->aux_stream);
   if (m->ev_fork) cudaEventDestroy(m->ev_fork);
@@ -1820,8 +1813,7 @@ rm_status rm_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     double *d_els, *d_grad, *d_jtj;
     Carver plan{nullptr};
     arrays(plan, &d_st, &d_counts, &d_etable, &d_els, &d_grad, &d_jtj);
-    RM_TRY(ensure_arena(m, plan.off, s));
-    RM_TRY(ensure_zbuf(m, (size_t)in->width * in->height, s));
+    RM_TRY(ensure_scratch(m, plan.off, (size_t)in->width * in->height, s));
     m->batch_inputs_valid = false;
     Carver cv{m->arena};
     arrays(cv, &d_st, &d_counts, &d_etable, &d_els, &d_grad, &d_jtj);
@@ -1900,8 +1892,7 @@ rm_status rm_dfo_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     double *d_els;
     Carver plan{nullptr};
     arrays(plan, &d_st, &d_counts, &d_et, &d_els);
-    RM_TRY(ensure_arena(m, plan.off, s));
-    RM_TRY(ensure_zbuf(m, (size_t)in->width * in->height * S, s));
+    RM_TRY(ensure_scratch(m, plan.off, (size_t)in->width * in->height * S, s));
     m->batch_inputs_valid = false;
     Carver cv{m->arena};
     arrays(cv, &d_st, &d_counts, &d_et, &d_els);
@@ -2004,8 +1995,7 @@ rm_status rm_icp_align(rm_map *m, const rm_scan *scan, const double *init_pose,
     double *d_l1, *d_e2, *d_g, *d_H;
     Carver plan{nullptr};
     arrays(plan, &d_st, &d_n, &d_l1, &d_e2, &d_g, &d_H);
-    RM_TRY(ensure_arena(m, plan.off, s));
-    RM_TRY(ensure_zbuf(m, (size_t)in->width * in->height, s));
+    RM_TRY(ensure_scratch(m, plan.off, (size_t)in->width * in->height, s));
     m->batch_inputs_valid = false;
     Carver cv{m->arena};
     arrays(cv, &d_st, &d_n, &d_l1, &d_e2, &d_g, &d_H);

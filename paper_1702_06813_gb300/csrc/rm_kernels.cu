@@ -1,20 +1,23 @@
 // rm_kernels.cu -- the pose-cost hot path on sm_103a.
 //
 // Per pose (one wave of poses at a time, blockIdx.y = pose within the wave):
-//   k_pose_to_m   camera-to-world FP64 pose -> world-to-camera FP32 3x4 (Eq. 1's T(X) -> Y)
+//   k_begin       camera-to-world FP64 pose -> world-to-camera FP32 3x4 (Eq. 1's T(X) -> Y), and
+//                 the call's counters to zero
 //   k_cull        per cluster of <= 64 triangles: bounding sphere against the view volume
-//   k_setup       per visible cluster: camera-space vertices and their 1/256-px snapped
-//                 projections, then per triangle: near-plane cut, cull, depth plane, append
-//                 to the screen-tile bins
-//   k_raster      one CTA per (pose, tile): bins staged into shared memory with bulk (TMA)
-//                 copies, integer edge functions with the top-left rule, 64-bit
+//   k_setup_pin, k_setup_ray
+//                 per visible cluster: camera-space vertices and their 1/256-px snapped
+//                 projections (or ray-table columns and rows), then per triangle that can hold a
+//                 sample: near-plane cut, depth plane, and either its samples' keys straight into
+//                 the z-buffer or a record in the screen-tile bins
+//   k_raster      one CTA per (pose, tile): the tile's z-buffer keys, bins staged into shared memory
+//                 with bulk (TMA) copies, integer edge functions with the top-left rule, 64-bit
 //                 depth|id z-test by shared-memory atomicMin (the z-buffer R(Y) of Sec. IV);
 //                 then the fused epilogue: Table I per pixel (Sec. IV.B), the truncated
 //                 least-squares residual, its pose Jacobian, and a fixed-order reduction;
 //                 in ICP mode instead the projective association of each pixel's map
 //                 surface with its scan return and the point-to-plane terms (Sec. V)
 //   k_reduce      per pose: fixed-order sum of the per-tile partials
-// k_lm_* and k_icp_* take the Levenberg-Marquardt and ICP steps between evaluations.
+// k_step_one and k_dfo_step end an evaluation of a search (LM, ICP, derivative-free) with its step.
 // The k_*_batch kernels run the same phases for problems of different cameras and scans.
 #include <cfloat>
 #include <cmath>
@@ -185,7 +188,7 @@ __device__ __forceinline__ bool cluster_visible(const DevCam &cam, const float *
   return true;
 }
 
-// Reads of data that another CTA of the same (persistent) kernel may have written bypass L1.
+// Reads of data that an earlier kernel wrote and this one does not bypass L1.
 __device__ __forceinline__ int ld_cg(const int *p) { return __ldcg(p); }
 __device__ __forceinline__ bool skipped(const WaveArgs &a) { return a.skip && __ldcg(a.skip) != 0; }
 
