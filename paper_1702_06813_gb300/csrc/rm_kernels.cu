@@ -1996,8 +1996,8 @@ static cudaError_t launch_raster(const WaveArgs &a, int mode, cudaStream_t s) {
 
 // Setup CTAs (four warps) per pose: 32 in a large wave, so that each warp sets up several clusters
 // and the next wave's setup (on the other stream) takes few enough SMs to run beside this wave's
-// raster; waves of few poses (single-pose alignment) get up to seven CTAs per SM in total and as
-// little as one cluster to a warp: the chain of a cluster's loads is what they wait for.
+// raster; waves of few poses get up to kSetupCtasPerGpu in total and as little as one cluster to a
+// warp: the chain of a cluster's loads is what a single pose waits for.
 static int setup_blocks(int n_clusters, int n_poses) {
   const int per_pose = max(32, (kSetupCtasPerGpu + n_poses - 1) / n_poses);
   return min((n_clusters + 3) / 4, per_pose);

@@ -208,7 +208,10 @@ struct BatchArgs {
   int *progress;           // one problem's loop: host memory for (evaluations done, ended), or null
 };
 
-constexpr int kSetupCtasPerGpu = 1064;  // setup CTAs a small wave may spread over (152 SMs x 7)
+// Setup CTAs a wave of few poses spreads over: several times what is resident (152 SMs x 7), so that
+// the SMs even out clusters of unequal work. 64 Lidar poses 1.92 ms with 1064, 1.69 with 1824, 1.62
+// with 3648, 1.61 with 5472; 24 mixed agents 3.46, 3.23, 3.30, 3.52.
+constexpr int kSetupCtasPerGpu = 3648;
 
 cudaError_t launch_lm_init_batch(LMState *st, const double *T0, int n, const LMArgs &a,
                                  float *Ms, int *skip, cudaStream_t s);
