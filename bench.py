@@ -599,7 +599,7 @@ def run_icp(a):
     mbytes = 5 * P_img + 12 * P_img + 13 * nfaces
     mesh_line = {"image": [cam.width, cam.height], "faces": nfaces, "us_per_call": ms_m / 20 * 1e3,
                  "algorithmic_bytes": mbytes, "achieved_gbs": mbytes * 20 / (ms_m * 1e-3) / 1e9,
-                 "kernels_per_call": 4}
+                 "kernels_per_call": 2}
 
     # derivative-free alignment on the Table I cost (Sec. IV.C), room scan from 3 cm / 1.5 deg
     rng2 = np.random.Generator(np.random.PCG64(a.seed + 9))

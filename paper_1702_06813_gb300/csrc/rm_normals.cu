@@ -10,8 +10,8 @@
 // shuffle. Rows are not convolved twice and only 12 of 74 columns (radius 5) and the chunk's first
 // and last rows are halo. One instantiation per radius, so the taps unroll with their weights in
 // registers. Each depth and class byte is read about once from HBM and each normal written once
-// (17 bytes per pixel). Bound by the shared-memory pipe (0.88 of its peak: about 60 wavefronts a row
-// of 64 columns, two fifths of them the row windows) beside instruction issue (0.65). 64 images of
+// (17 bytes per pixel). Bound by the shared-memory pipe (0.76 of its peak: about 60 wavefronts a row
+// of 64 columns, two fifths of them the row windows) beside instruction issue (0.66). 64 images of
 // 640x480 at radius 5: 146 us; the form before it, one CTA per 64x16 tile with its halo staged
 // and convolved again by its neighbours, 229 us and 1.9 times the instructions.
 #include <cfloat>
