@@ -781,7 +781,13 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
   // problems that share a host array share one staged copy; device arrays are read in place
   using Key = std::tuple<const void *, int, int>;
   std::map<Key, size_t> staged;    // offset in the staging area
-  std::map<const void *, int> tables;  // ray tables, numbered
+  // tables' deviations from their layouts, numbered: one for everything that k_ray_dev reads, as
+  // problems may look at one array with different layouts or at its first rows only
+  using Table = std::tuple<const void *, int, int, float, float, float, float>;
+  std::map<Table, int> tables;
+  auto table_of = [](const rm_intrinsics &in) {
+    return Table(in.rays, in.width, in.height, in.az0, in.az_step, in.el0, in.el_step);
+  };
   size_t stage_bytes = 0;
   auto stage = [&](const void *h, size_t bytes, int W, int H) {
     if (!on_device(h) && staged.emplace(Key(h, W, H), stage_bytes).second) stage_bytes += align_up(bytes, 256);
@@ -793,7 +799,7 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
     stage(sc.cls, P, sc.intr.width, sc.intr.height);
     if (sc.intr.model == RM_RAYTABLE) {
       stage(sc.intr.rays, sizeof(float) * 3 * P, sc.intr.width, sc.intr.height);
-      tables.emplace(sc.intr.rays, (int)tables.size());
+      tables.emplace(table_of(sc.intr), (int)tables.size());
     }
   }
   for (int attempt = 0;; ++attempt) {
@@ -902,7 +908,7 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       a.touched = d.counters + n + tiles_total + t_off;
       a.zbuf = m->zbuf + px_off;
       if (rays) {
-        const int t = tables[in->rays];
+        const int t = tables[table_of(*in)];
         a.ray_dev = d.dev + 2 * t;
         if (!measured[t]) RM_CK(rmk::launch_ray_dev(a.cam, d.dev + 2 * t, s));
         measured[t] = 1;
