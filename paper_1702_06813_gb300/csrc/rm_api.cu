@@ -778,9 +778,10 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       if ((probs[p].scan.intr.model == RM_RAYTABLE) == (md == 1)) order.push_back(p);
   int n_pin = 0;
   for (int p = 0; p < n; ++p) n_pin += probs[p].scan.intr.model != RM_RAYTABLE;
-  // problems that share a host array share one staged copy; device arrays are read in place
-  using Key = std::tuple<const void *, int, int>;
-  std::map<Key, size_t> staged;    // offset in the staging area
+  // problems that share a host array share one staged copy; device arrays are read in place. Arrays
+  // of different lengths are staged apart, also where they start at one address.
+  using Key = std::pair<const void *, size_t>;  // array, bytes
+  std::map<Key, size_t> staged;                 // offset in the staging area
   // tables' deviations from their layouts, numbered: one for everything that k_ray_dev reads, as
   // problems may look at one array with different layouts or at its first rows only
   using Table = std::tuple<const void *, int, int, float, float, float, float>;
@@ -789,16 +790,16 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
     return Table(in.rays, in.width, in.height, in.az0, in.az_step, in.el0, in.el_step);
   };
   size_t stage_bytes = 0;
-  auto stage = [&](const void *h, size_t bytes, int W, int H) {
-    if (!on_device(h) && staged.emplace(Key(h, W, H), stage_bytes).second) stage_bytes += align_up(bytes, 256);
+  auto stage = [&](const void *h, size_t bytes) {
+    if (!on_device(h) && staged.emplace(Key(h, bytes), stage_bytes).second) stage_bytes += align_up(bytes, 256);
   };
   for (int p = 0; p < n; ++p) {
     const rm_scan &sc = probs[p].scan;
     const size_t P = (size_t)sc.intr.width * sc.intr.height;
-    stage(sc.depth, sizeof(float) * P, sc.intr.width, sc.intr.height);
-    stage(sc.cls, P, sc.intr.width, sc.intr.height);
+    stage(sc.depth, sizeof(float) * P);
+    stage(sc.cls, P);
     if (sc.intr.model == RM_RAYTABLE) {
-      stage(sc.intr.rays, sizeof(float) * 3 * P, sc.intr.width, sc.intr.height);
+      stage(sc.intr.rays, sizeof(float) * 3 * P);
       tables.emplace(table_of(sc.intr), (int)tables.size());
     }
   }
@@ -865,8 +866,8 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
                               on_device(probs[p].pose) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     }
     std::vector<char> sent(staged.size(), 0), measured(tables.size(), 0);
-    auto device_array = [&](const void *h, size_t bytes, int W, int H, const void **dv) -> rm_status {
-      const auto it = staged.find(Key(h, W, H));
+    auto device_array = [&](const void *h, size_t bytes, const void **dv) -> rm_status {
+      const auto it = staged.find(Key(h, bytes));
       if (it == staged.end()) {
         *dv = h;
         return RM_OK;
@@ -885,9 +886,9 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       const rm_intrinsics *in = &sc.intr;
       const size_t P = (size_t)in->width * in->height;
       const void *sd, *cls, *rays = nullptr;
-      RM_TRY(device_array(sc.depth, sizeof(float) * P, in->width, in->height, &sd));
-      RM_TRY(device_array(sc.cls, P, in->width, in->height, &cls));
-      if (in->model == RM_RAYTABLE) RM_TRY(device_array(in->rays, sizeof(float) * 3 * P, in->width, in->height, &rays));
+      RM_TRY(device_array(sc.depth, sizeof(float) * P, &sd));
+      RM_TRY(device_array(sc.cls, P, &cls));
+      if (in->model == RM_RAYTABLE) RM_TRY(device_array(in->rays, sizeof(float) * 3 * P, &rays));
       WaveArgs &a = args[k];
       std::memset(&a, 0, sizeof(WaveArgs));  // padding too: the argument block is compared bytewise
       a.cam = make_cam(in, static_cast<const float *>(rays));
