@@ -781,7 +781,11 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
   // problems that share a host array share one staged copy; device arrays are read in place. Arrays
   // of different lengths are staged apart, also where they start at one address.
   using Key = std::pair<const void *, size_t>;  // array, bytes
-  std::map<Key, size_t> staged;                 // offset in the staging area
+  struct Staged {
+    size_t at;         // offset in the staging area
+    int sent_for = -1;  // the attempt that it was last copied for
+  };
+  std::map<Key, Staged> staged;
   // tables' deviations from their layouts, numbered: one for everything that k_ray_dev reads, as
   // problems may look at one array with different layouts or at its first rows only
   using Table = std::tuple<const void *, int, int, float, float, float, float>;
@@ -791,7 +795,7 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
   };
   size_t stage_bytes = 0;
   auto stage = [&](const void *h, size_t bytes) {
-    if (!on_device(h) && staged.emplace(Key(h, bytes), stage_bytes).second) stage_bytes += align_up(bytes, 256);
+    if (!on_device(h) && staged.emplace(Key(h, bytes), Staged{stage_bytes}).second) stage_bytes += align_up(bytes, 256);
   };
   for (int p = 0; p < n; ++p) {
     const rm_scan &sc = probs[p].scan;
@@ -865,17 +869,17 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
         RM_CK(cudaMemcpyAsync(d.poses + 16 * (size_t)p, probs[p].pose, sizeof(double) * 16,
                               on_device(probs[p].pose) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
     }
-    std::vector<char> sent(staged.size(), 0), measured(tables.size(), 0);
+    std::vector<char> measured(tables.size(), 0);
     auto device_array = [&](const void *h, size_t bytes, const void **dv) -> rm_status {
       const auto it = staged.find(Key(h, bytes));
       if (it == staged.end()) {
         *dv = h;
         return RM_OK;
       }
-      *dv = d.staged + it->second;
-      char &done = sent[(size_t)std::distance(staged.begin(), it)];
-      if (!done) RM_CK(cudaMemcpyAsync(d.staged + it->second, h, bytes, cudaMemcpyHostToDevice, s));
-      done = 1;
+      Staged &st = it->second;
+      *dv = d.staged + st.at;
+      if (st.sent_for != attempt) RM_CK(cudaMemcpyAsync(d.staged + st.at, h, bytes, cudaMemcpyHostToDevice, s));
+      st.sent_for = attempt;
       return RM_OK;
     };
     std::vector<WaveArgs> args(n);

@@ -3,6 +3,8 @@ of several sizes, and a class array that starts at the address of another scan's
 problem equals rm_cost_grad on the device bit for bit."""
 from __future__ import annotations
 
+import time
+
 import numpy as np
 import pytest
 
@@ -64,3 +66,24 @@ def test_shared_host_arrays_of_several_sizes(scene):
     scans.append(rm.Scan(scans[2].intr, scans[2].depth * 1.01, scans[2].cls))  # its table and classes, another depth
     order = [2, 0, 1, 0, 3, 4, 2, 1, 3]
     _same_as_calls(gm, [(scans[k], synth.perturb_fixed(c["gt"], r, 0.03, 1.0)) for k in order])
+
+
+def test_many_host_scans_take_time_in_proportion(scene):
+    """Eight times the scans, each with its own host arrays, take about eight times as long (a search
+    of the list of arrays for each of them: 31 times)."""
+    c, gm = scene
+    intr = rm.Intrinsics.from_camera(cases.small_pinhole(16, 16, 14.0))
+    scans = [rm.Scan(intr, torch.full((16, 16), 2.0 + 1e-3 * k), torch.zeros((16, 16), dtype=torch.uint8))
+             for k in range(4096)]
+    poses = torch.as_tensor(c["gt"]).cuda().expand(4096, 4, 4).contiguous()
+
+    def best(n):
+        rm.cost_grad_batch(gm, scans=scans[:n], poses=poses[:n])
+        took = []
+        for _ in range(5):
+            t = time.perf_counter()
+            rm.cost_grad_batch(gm, scans=scans[:n], poses=poses[:n])
+            took.append(time.perf_counter() - t)
+        return min(took)
+
+    assert best(4096) < 16 * best(512)
