@@ -38,8 +38,10 @@
  * status word that the call reads back. rm_last_error() gives a message for the calling
  * thread's last failure.
  *
- * Threading: calls on one map are serialised by the map (they share its scratch memory).
- * Different maps may be used from different threads concurrently.
+ * Threading: calls on one map are serialised by the map (they share its scratch memory), on the
+ * device too when they are given different streams and do not wait (async_status). The launches
+ * of a graph that captured such calls are the caller's to order: they must not overlap each other
+ * or other calls on the map. Different maps may be used from different threads concurrently.
  */
 #ifndef RENDERMAP_H
 #define RENDERMAP_H

@@ -113,6 +113,10 @@ struct rm_map {
   // culling and setup overlap the previous wave's raster
   cudaStream_t aux_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // the end of the last call that returned before the device was done (async_status): the next call
+  // on the map waits for it on the device, as the scratch is one for all streams
+  cudaEvent_t ev_queued = nullptr;
+  bool queued = false;
   cudaGraphExec_t batch_exec = nullptr;
   std::string batch_sig;
   // host copy of the batch's per-problem arguments last uploaded into the arena; valid until
@@ -307,10 +311,22 @@ void build_clusters(const std::vector<float4> &hv, const int32_t *faces, int64_t
   flush();
 }
 
+// Whether s is being captured into a graph: nothing that a call enqueues then runs before the graph does.
+rm_status capturing(cudaStream_t s, bool *yes) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  RM_CK(cudaStreamIsCapturing(s, &st));
+  *yes = st != cudaStreamCaptureStatusNone;
+  return RM_OK;
+}
+
 // The arena (`bytes`, carved by each call) and the z-buffers of a call's waves (`keys` of them, every
 // one kKeyEmpty), in one allocation that grows with either. The z-buffers are kept between calls:
-// the raster leaves every key it reads empty, so a call pays only for the tiles it touches.
+// the raster leaves every key it reads empty, so a call pays only for the tiles it touches. Orders
+// the call after one that is still queued; a graph's launches are the caller's to order.
 rm_status ensure_scratch(rm_map *m, size_t bytes, size_t keys, cudaStream_t s) {
+  bool captured = false;
+  if (m->queued || m->tuning.async_status) RM_TRY(capturing(s, &captured));
+  if (m->queued && !captured) RM_CK(cudaStreamWaitEvent(s, m->ev_queued, 0));
   if (bytes > m->arena_bytes || keys > m->zbuf_keys) {
     RM_CK(cudaStreamSynchronize(s));
     if (m->batch_exec) {  // the captured batch graph points into the old arena
@@ -334,7 +350,7 @@ rm_status ensure_scratch(rm_map *m, size_t bytes, size_t keys, cudaStream_t s) {
   }
   if (!m->zbuf_empty)  // every byte of kKeyEmpty is 0xff
     RM_CK(cudaMemsetAsync(m->zbuf, 0xff, sizeof(unsigned long long) * m->zbuf_keys, s));
-  m->zbuf_empty = true;
+  m->zbuf_empty = m->zbuf_empty || !captured;  // a captured fill is the graph's, not the next call's
   return RM_OK;
 }
 
@@ -479,11 +495,26 @@ rm_status grow_bins(rm_map *m, unsigned st, int attempt) {
   return RM_OK;
 }
 
+// The end of a call that does not wait for the device.
+rm_status leave_queued(rm_map *m, cudaStream_t s) {
+  bool captured;
+  RM_TRY(capturing(s, &captured));
+  if (captured) return RM_OK;
+  if (!m->ev_queued) RM_CK(cudaEventCreateWithFlags(&m->ev_queued, cudaEventDisableTiming));
+  RM_CK(cudaEventRecord(m->ev_queued, s));
+  m->queued = true;
+  return RM_OK;
+}
+
 // Waits for the stream, then reads and clears the status word: it is in pinned host memory, which the
 // kernels write only when something went wrong (a copy back and a memset on every call cost a
 // single-pose evaluation 12 us of 96).
 rm_status read_status(rm_map *m, cudaStream_t s, unsigned *out) {
   RM_CK(cudaStreamSynchronize(s));
+  if (m->queued) {  // still queued only if on another stream than s, with no call on the map since
+    m->queued = cudaEventQuery(m->ev_queued) == cudaErrorNotReady;
+    cudaGetLastError();
+  }
   volatile unsigned *h = m->status;
   *out = *h;
   *h = 0;
@@ -673,6 +704,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       RM_CK(cudaEventRecord(m->ev_fork, s));
       RM_CK(cudaStreamWaitEvent(m->aux_stream, m->ev_fork, 0));
     }
+    const bool was_empty = m->zbuf_empty;  // not after a fill that was only captured
     m->zbuf_empty = false;  // until every wave's raster is on its way
     for (int w0 = 0, k = 0; w0 < r.n; w0 += nw, ++k) {
       const int b = k % nbuf;  // buffer set and stream of this wave
@@ -687,7 +719,7 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       a.touched = d_touched + (size_t)w0 * tg.ntiles;
       RM_TRY(wave(m, a, r.mode, b == 0 ? s : m->aux_stream));
     }
-    m->zbuf_empty = true;
+    m->zbuf_empty = was_empty;
     if (nbuf == 2) {
       RM_CK(cudaEventRecord(m->ev_join, m->aux_stream));
       RM_CK(cudaStreamWaitEvent(s, m->ev_join, 0));
@@ -714,7 +746,9 @@ rm_status run_eval(rm_map *m, const EvalReq &r, cudaStream_t s) {
       }
     }
     if (m->tuning.async_status && !r.batch) {
-      if (host_out) RM_CK(cudaStreamSynchronize(s));
+      if (!host_out) return leave_queued(m, s);
+      RM_CK(cudaStreamSynchronize(s));
+      m->queued = false;
       return RM_OK;
     }
     unsigned st = 0;
@@ -1430,6 +1464,7 @@ void rm_map_destroy(rm_map *m) {
   if (m->aux_stream) cudaStreamDestroy(m->aux_stream);
   if (m->ev_fork) cudaEventDestroy(m->ev_fork);
   if (m->ev_join) cudaEventDestroy(m->ev_join);
+  if (m->ev_queued) cudaEventDestroy(m->ev_queued);
   if (m->status) cudaFreeHost(m->status);
   if (m->h_progress) cudaFreeHost(m->h_progress);
   for (auto &ev : m->ev_pending)
