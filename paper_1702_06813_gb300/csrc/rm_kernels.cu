@@ -925,9 +925,11 @@ struct QuickRect {
     half_turn = 3.1f / cam.az_step;
     last = (unsigned)(cam.W - 1) | (unsigned)(cam.H - 1) << 16;
     // never for a margin that can cross the seam, nor for a table that neither covers one turn
-    // nor stays within (-pi, pi], where the general way places columns past the seam differently
+    // nor stays within (-pi, pi], where the general way places columns past the seam differently;
+    // nor for a layout many turns from zero, whose columns FP32 rounds by more than kAngleErr (up to
+    // 32 radians by at most 0.66 of the margin, from about 1400 on by more than all of it)
     const float span = cam.W * cam.az_step;
-    const bool turn = fabsf(span - 6.28318531f) < 0.05f * cam.az_step;
+    const bool turn = fabsf(span - 6.28318531f) < 0.05f * cam.az_step && fabsf(cam.az0) <= 32.0f;
     if (!(a0 < -0.05f && (turn || (cam.az0 >= -3.14160f && cam.az0 + span <= 3.14160f)))) half_turn = -1.0f;
   }
   // b1: the row margin - 1/2 for edges of squared angular length up to L2.
