@@ -1054,9 +1054,10 @@ rm_status run_batch(rm_map *m, const rm_problem *probs, int n, const rm_cost_par
       m->batch_sig = key;
     }
     m->zbuf_empty = false;  // until every evaluation's raster is on its way
+    auto slices = [](int k) { return (k + rmk::kMaxGridRows - 1) / rmk::kMaxGridRows; };
     for (int it = 0; it <= K; it += E) {
       RM_CK(cudaGraphLaunch(m->batch_exec, s));
-      m->launches += (size_t)E * ((n_pin > 0) + (n_pin < n)) * (nc > 0 ? 4 : 2);
+      m->launches += (size_t)E * (slices(n_pin) + slices(n - n_pin)) * (nc > 0 ? 4 : 2);
     }
     m->zbuf_empty = true;
     bool host_out = false;

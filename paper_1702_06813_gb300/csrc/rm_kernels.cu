@@ -2821,25 +2821,30 @@ cudaError_t launch_step_one(const WaveArgs &a, const BatchArgs &b, cudaStream_t 
 
 cudaError_t launch_batch_eval(const WaveArgs *probs, int n, int model, int mode, bool vnormals, int n_clusters,
                               int max_tiles, const BatchArgs &b, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  if (n_clusters > 0) {
-    k_cull_batch<<<dim3((n_clusters + 255) / 256, n), 256, 0, s>>>(probs);
-    const int blocks = setup_blocks(n_clusters, n);
-    if (model == 0) k_setup_pin_batch<<<dim3(blocks, n), kPinSetupThreads, 0, s>>>(probs);
-    else k_setup_ray_batch<<<dim3(blocks, n), kRaySetupThreads, 0, s>>>(probs);
+  for (int first = 0; first < n; first += kMaxGridRows) {
+    const WaveArgs *p = probs + first;
+    const int rows = min(n - first, kMaxGridRows);
+    if (n_clusters > 0) {
+      k_cull_batch<<<dim3((n_clusters + 255) / 256, rows), 256, 0, s>>>(p);
+      const dim3 gs(setup_blocks(n_clusters, n), rows);
+      if (model == 0) k_setup_pin_batch<<<gs, kPinSetupThreads, 0, s>>>(p);
+      else k_setup_ray_batch<<<gs, kRaySetupThreads, 0, s>>>(p);
+    }
+    const dim3 grid(max_tiles, rows);
+    if (model == 0) {
+      if (mode == kCostGrad) k_raster_batch<kCostGrad, 0><<<grid, kThreads, 0, s>>>(p);
+      else if (vnormals) k_raster_batch<kIcpVn, 0><<<grid, kThreads, 0, s>>>(p);
+      else k_raster_batch<kIcp, 0><<<grid, kThreads, 0, s>>>(p);
+    } else {
+      if (mode == kCostGrad) k_raster_batch<kCostGrad, 1><<<grid, kThreads, 0, s>>>(p);
+      else if (vnormals) k_raster_batch<kIcpVn, 1><<<grid, kThreads, 0, s>>>(p);
+      else k_raster_batch<kIcp, 1><<<grid, kThreads, 0, s>>>(p);
+    }
+    k_step_batch<<<rows, 256, 0, s>>>(p, b);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
   }
-  const dim3 grid(max_tiles, n);
-  if (model == 0) {
-    if (mode == kCostGrad) k_raster_batch<kCostGrad, 0><<<grid, kThreads, 0, s>>>(probs);
-    else if (vnormals) k_raster_batch<kIcpVn, 0><<<grid, kThreads, 0, s>>>(probs);
-    else k_raster_batch<kIcp, 0><<<grid, kThreads, 0, s>>>(probs);
-  } else {
-    if (mode == kCostGrad) k_raster_batch<kCostGrad, 1><<<grid, kThreads, 0, s>>>(probs);
-    else if (vnormals) k_raster_batch<kIcpVn, 1><<<grid, kThreads, 0, s>>>(probs);
-    else k_raster_batch<kIcp, 1><<<grid, kThreads, 0, s>>>(probs);
-  }
-  k_step_batch<<<n, 256, 0, s>>>(probs, b);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace rmk

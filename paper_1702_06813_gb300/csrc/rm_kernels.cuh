@@ -217,8 +217,10 @@ cudaError_t launch_lm_init_batch(LMState *st, const double *T0, int n, const LMA
                                  float *Ms, int *skip, cudaStream_t s);
 // The end of an evaluation of the one problem a (launch_wave without its reduction).
 cudaError_t launch_step_one(const WaveArgs &a, const BatchArgs &b, cudaStream_t s);
-// One evaluation (and LM or ICP step) of the n problems probs[0..n) of one camera model: cull,
-// setup, raster, step. max_tiles: the most screen tiles of one problem; vnormals: the map carries
+// Problems that one launch of a batch takes: they are the grid's rows, of which there are at most 65535.
+constexpr int kMaxGridRows = 65535;
+// One evaluation (and LM or ICP step) of the n problems probs[0..n) of one camera model, in slices of
+// kMaxGridRows: cull, setup, raster, step. max_tiles: the most screen tiles of one problem; vnormals: the map carries
 // vertex normals (ICP).
 cudaError_t launch_batch_eval(const WaveArgs *probs, int n, int model, int mode, bool vnormals, int n_clusters,
                               int max_tiles, const BatchArgs &b, cudaStream_t s);
