@@ -829,6 +829,9 @@ constexpr int kDirectRay = RM_DIRECT_RAY;
 static_assert(kDirectRay <= kFragmentMax, "fragment index decode");
 constexpr float kFarColumn = 1e30f;  // column of a vertex the quick rectangle cannot hold
 constexpr float kAngleErr = 6e-6f;   // error bound of the vertices' approximate angles, radians
+// From here on FP32 rounds a layout's columns by too much for QuickRect: up to 32 radians by at most
+// 0.66 of its margin, from about 1400 on by more than all of it.
+constexpr float kFarAzimuth = 32.0f;
 constexpr float kRoundMagic = 12582912.0f;  // 1.5 2^23: x + this holds rint(x) in its low bits
 
 struct RaySetupSmem {
@@ -925,11 +928,9 @@ struct QuickRect {
     half_turn = 3.1f / cam.az_step;
     last = (unsigned)(cam.W - 1) | (unsigned)(cam.H - 1) << 16;
     // never for a margin that can cross the seam, nor for a table that neither covers one turn
-    // nor stays within (-pi, pi], where the general way places columns past the seam differently;
-    // nor for a layout many turns from zero, whose columns FP32 rounds by more than kAngleErr (up to
-    // 32 radians by at most 0.66 of the margin, from about 1400 on by more than all of it)
+    // nor stays within (-pi, pi], where the general way places columns past the seam differently
     const float span = cam.W * cam.az_step;
-    const bool turn = fabsf(span - 6.28318531f) < 0.05f * cam.az_step && fabsf(cam.az0) <= 32.0f;
+    const bool turn = fabsf(span - 6.28318531f) < 0.05f * cam.az_step;
     if (!(a0 < -0.05f && (turn || (cam.az0 >= -3.14160f && cam.az0 + span <= 3.14160f)))) half_turn = -1.0f;
   }
   // b1: the row margin - 1/2 for edges of squared angular length up to L2.
@@ -982,8 +983,12 @@ __device__ __forceinline__ void setup_ray_table(const WaveArgs &a, int q, RaySet
   float2 *uv = sm.uv[warp];
   float4 *ring = sm.ring[warp];
   if (threadIdx.x == 0) sm.nvis = ld_cg(&a.vis_count[q]);
+  // a layout many turns from zero: a pixel, which QuickRect refuses (here, and not as a test of its
+  // own, which costs k_setup_ray four registers that it does not have: 64 poses 1.56 -> 1.59 ms)
   if (threadIdx.x < 2)
-    sm.dev[threadIdx.x] = a.ray_dev ? fminf(kRayMarginPx, __int_as_float(__ldg(a.ray_dev + threadIdx.x))) : kRayMarginPx;
+    sm.dev[threadIdx.x] = fabsf(a.cam.az0) > kFarAzimuth ? 1.0f
+                          : a.ray_dev ? fminf(kRayMarginPx, __int_as_float(__ldg(a.ray_dev + threadIdx.x)))
+                                      : kRayMarginPx;
   load_m_block(a, q, sm.M);
   const DevCam &cam = a.cam;
   const int nvis = sm.nvis, stride = gridDim.x * (kRaySetupThreads / 32);
