@@ -1,23 +1,20 @@
 // rm_normals.cu -- rm_depth_normals: surface normals of depth images (Eq. 2, Sec. V).
 //
-// One warp per (62-column strip, chunk of rows, image), fused and without block barriers: it walks
-// down its strip four rows at a time. Each row's depths are staged in shared memory as (depth,
-// weight) pairs, zero where invalid, with a halo of the Gaussian's radius; a lane smooths two
-// adjacent columns along the row, sums and weight sums together in packed FP32 pairs (a
-// normalised convolution), and keeps the result in its own ring of the last rows; four smoothed
-// rows then come from one pass down the ring, and the normals N = a x b with a = (0, s_y, dz/dy),
-// b = (s_x, 0, dz/dx) from the smoothed rows in registers, the columns beside a lane's own by
-// shuffle. Rows are not convolved twice and only 12 of 74 columns (radius 5) and the chunk's first
-// and last rows are halo. One instantiation per radius, so the taps unroll with their weights in
-// registers. Each depth and class byte is read about once from HBM and each normal written once
-// (17 bytes per pixel). Bound by the shared-memory pipe (0.76 of its peak: about 60 wavefronts a row
-// of 64 columns, two fifths of them the row windows) beside instruction issue (0.66). 64 images of
-// 640x480 at radius 5: 146 us; the form before it, one CTA per 64x16 tile with its halo staged
-// and convolved again by its neighbours, 229 us and 1.9 times the instructions.
+// Gaussian smoothing as a normalised convolution (weighted sums of the valid depths and of their
+// weights, along the rows, then down the columns) and the normals N = a x b with a = (0, s_y, dz/dy),
+// b = (s_x, 0, dz/dx) by central differences of the smoothed depth S, fused. Each depth and class byte
+// is read about once from HBM and each normal written once (17 bytes per pixel). One instantiation per
+// radius, so the taps unroll with their weights in registers. Two kernels that add and divide in the
+// same order and agree bit for bit:
+//   k_depth_normals       many pixels: one warp per (62-column strip, chunk of rows, image) walks down
+//                         its strip without block barriers
+//   k_depth_normals_tile  few pixels: one CTA per (64x16 output tile, image)
 #include <cfloat>
 #include <algorithm>
 #include <cmath>
+#include <cstdlib>
 #include <string>
+#include <type_traits>
 
 #include "rendermap.h"
 #include "rm_kernels.cuh"
@@ -41,8 +38,40 @@ struct NormalArgs {
   int strips, chunks, rows;  // strips across, chunks down an image, output rows of a chunk
   long long n_warps;         // strips * chunks * images
   float ifx, ify;    // 1 / fx, 1 / fy
+  float den_all;     // the weight sum where every pixel of the window is valid, summed as the kernels do
   float g[kMaxR + 1];
 };
+
+// A staged pixel as (depth, weight), zero where invalid.
+__device__ __forceinline__ float2 depth_pair(float d, int c) {
+  const bool ok = c == 0 && fabsf(d) <= FLT_MAX;
+  return make_float2(ok ? d : 0.0f, ok ? 1.0f : 0.0f);
+}
+
+// The normal at smoothed depth s between its neighbours left, right, up and down. S is NaN at invalid
+// pixels and outside the image, so an undefined difference makes the normal NaN by itself; only an
+// invalid centre needs asking for.
+__device__ __forceinline__ float3 eq2_normal(const NormalArgs &a, float s, float sl, float sr, float su, float sd) {
+  const float zx = 0.5f * (sr - sl), zy = 0.5f * (sd - su);
+  const float sx = a.metric ? s * a.ifx : 1.0f, sy = a.metric ? s * a.ify : 1.0f;
+  // a = (0, sy, zy), b = (sx, 0, zx), N = a x b
+  const float q0 = sy * zx, q1 = zy * sx, q2 = -sy * sx;
+  float inv = rsqrtf(q0 * q0 + q1 * q1 + q2 * q2);
+  if (isnan(s)) inv = __builtin_nanf("");
+  return make_float3(q0 * inv, q1 * inv, q2 * inv);
+}
+
+// ------------------------------------------------------------------ strips (many pixels)
+//
+// A warp walks down its strip four rows at a time. Each row's depths are staged in shared memory as
+// (depth, weight) pairs with a halo of the Gaussian's radius; a lane smooths two adjacent columns
+// along the row, sums and weight sums together in packed FP32 pairs, and keeps the result in its own
+// ring of the last rows; four smoothed rows then come from one pass down the ring, and the normals
+// from the smoothed rows in registers, the columns beside a lane's own by shuffle. Rows are not
+// convolved twice and only 12 of 74 columns (radius 5) and the chunk's first and last rows are halo.
+// Bound by the shared-memory pipe (0.76 of its peak: about 60 wavefronts a row of 64 columns, two
+// fifths of them the row windows) beside instruction issue (0.66). 64 images of 640x480 at radius 5:
+// 146 us, where the tiles below take 229 and 1.9 times the instructions.
 
 // a * b + c on both halves, each rounded as one fused multiply-add.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
@@ -98,10 +127,6 @@ __global__ void __launch_bounds__(32 * kWarpsN) k_depth_normals(NormalArgs a) {
       cp += a.W;
     }
   };
-  auto pair = [](float d, int c) {
-    const bool ok = c == 0 && fabsf(d) <= FLT_MAX;
-    return make_float2(ok ? d : 0.0f, ok ? 1.0f : 0.0f);
-  };
   const int n_out = 3 * min(kOut, a.W - (xs + 1));
   long long at_out = img * P + (long long)y_out * a.W;  // the next output row
   unsigned long long v0 = 0, v1 = 0;               // validity of the own columns, last row in bit 0
@@ -112,7 +137,8 @@ __global__ void __launch_bounds__(32 * kWarpsN) k_depth_normals(NormalArgs a) {
     __syncwarp();
 #pragma unroll
     for (int r = 0; r < kRows; ++r) {
-      const float2 p0 = pair(zd[r][0], zc[r][0]), p1 = pair(zd[r][1], zc[r][1]), ph = pair(zd[r][2], zc[r][2]);
+      const float2 p0 = depth_pair(zd[r][0], zc[r][0]), p1 = depth_pair(zd[r][1], zc[r][1]),
+                   ph = depth_pair(zd[r][2], zc[r][2]);
       sm.z[r][R + 2 * lane] = p0;
       sm.z[r][R + 2 * lane + 1] = p1;
       if (lane < 2 * R) sm.z[r][hc] = ph;
@@ -180,19 +206,8 @@ __global__ void __launch_bounds__(32 * kWarpsN) k_depth_normals(NormalArgs a) {
           }
         }
         if (a.normals) {
-          // S is NaN at invalid pixels and outside the image, so an undefined difference makes the
-          // normal NaN by itself; only an invalid centre needs asking for
-          auto normal = [&](float s, float sl, float sr, float su, float sd) {
-            const float zx = 0.5f * (sr - sl), zy = 0.5f * (sd - su);
-            const float sx = a.metric ? s * a.ifx : 1.0f, sy = a.metric ? s * a.ify : 1.0f;
-            // a = (0, sy, zy), b = (sx, 0, zx), N = a x b
-            const float q0 = sy * zx, q1 = zy * sx, q2 = -sy * sx;
-            float inv = rsqrtf(q0 * q0 + q1 * q1 + q2 * q2);
-            if (isnan(s)) inv = kNan;
-            return make_float3(q0 * inv, q1 * inv, q2 * inv);
-          };
           float2 *o = reinterpret_cast<float2 *>(sm.out) + 3 * lane;
-          const float3 p = normal(s0b, left, s1b, s0a, s0), q = normal(s1b, s0b, right, s1a, s1);
+          const float3 p = eq2_normal(a, s0b, left, s1b, s0a, s0), q = eq2_normal(a, s1b, s0b, right, s1a, s1);
           o[0] = make_float2(p.x, p.y);
           o[1] = make_float2(p.z, q.x);
           o[2] = make_float2(q.y, q.z);
@@ -213,10 +228,182 @@ __global__ void __launch_bounds__(32 * kWarpsN) k_depth_normals(NormalArgs a) {
   }
 }
 
+// ------------------------------------------------------------------ tiles (few pixels)
+//
+// A strip's warp is a long chain: its chunk is no shorter than the halo that it reads besides, and
+// with few pixels there are too few warps to hide it. Here one CTA stages a tile's depths and weights
+// with a halo of radius + 1, smooths along the rows (four outputs a thread) and down the columns
+// (six), and takes the differences of the smoothed tile. Bound by latency: a load, two passes and two
+// barriers. One image of 640x480 with strips and with tiles: radius 2 8.4 and 4.6 us, 5 14.1 and 5.7,
+// 8 21.6 and 7.3, 15 43.2 and 10.5.
+
+constexpr int kTW = 64, kTH = 16;      // output tile
+constexpr int kSW = kTW + 2;           // smoothed region (tile plus a one-pixel ring)
+constexpr int kSH = kTH + 2;
+constexpr int kTileThreads = 256;
+constexpr int kHG = 4;                 // along the rows: outputs per thread
+constexpr int kVG = 6;                 // down the columns: outputs per thread
+// Below this many pixels in all the tiles are faster, at any radius but 0: at 1.2 M pixels strips take
+// 1.25 to 1.6 times as long (4 images of 640x480; 64 of 160x120, 0.95 to 1.2), at 2.1 M to 2.5 M 0.7 to
+// 1.3 (widths and radii either way), at 4.9 M 0.7 to 1.1. At radius 0 strips take 0.75 to 1.15 times
+// as long from one small image on.
+constexpr long long kTilePixels = 1ll << 21;
+
+// The tables' row strides are odd: the pass along the rows goes down their columns with consecutive
+// threads on consecutive rows, and 32 consecutive rows then fall in 32 distinct banks.
+__host__ __device__ constexpr int odd_stride(int n) { return n | 1; }
 template <int R>
-cudaError_t launch_normals_r(const NormalArgs &a, cudaStream_t s) {
+struct TileShape {
+  static constexpr int kW = kSW + 2 * R, kH = kSH + 2 * R, kStride = odd_stride(kW);  // staged pixels
+  static constexpr int kSumStride = odd_stride(kSW);
+  static constexpr size_t kBytes = sizeof(float) * (2 * kH * kStride + 2 * kH * kSumStride + kSH * kSW);
+};
+
+template <int R>
+__global__ void __launch_bounds__(kTileThreads) k_depth_normals_tile(NormalArgs a) {
+  extern __shared__ float4 smem_raw[];
+  using Shape = TileShape<R>;
+  constexpr int dw = Shape::kW, dh = Shape::kH, dws = Shape::kStride, hs = Shape::kSumStride;
+  float *zv = reinterpret_cast<float *>(smem_raw);  // [dh][dws]: valid ? z : 0
+  float *zw = zv + dh * dws;                        // [dh][dws]: valid ? 1 : 0
+  float *hn = zw + dh * dws;                        // [dh][hs]: sums of zv along the rows
+  float *hd = hn + dh * hs;                         // [dh][hs]: sums of zw
+  float *sS = hd + dh * hs;                         // [kSH][kSW]: smoothed depth
+  const int tid = threadIdx.x;
+  float g[R + 1];
+#pragma unroll
+  for (int k = 0; k <= R; ++k) g[k] = a.g[k];
+  const int ntx = (a.W + kTW - 1) / kTW;
+  const int ox = (blockIdx.x % ntx) * kTW, oy = (blockIdx.x / ntx) * kTH;
+  const int x0 = ox - 1 - R, y0 = oy - 1 - R;  // image coordinates of zv[0]
+  const long long P = (long long)a.W * a.H, img = blockIdx.y;
+  const float *dimg = a.depth + img * P;
+  const uint8_t *cimg = a.cls + img * P;
+  // stage, four loads in flight a thread; whether every staged pixel is valid is the common case away
+  // from holes and the image border
+  constexpr int n_st = dw * dh;
+  bool mine_valid = true;
+  for (int k0 = tid; k0 < n_st; k0 += 4 * kTileThreads) {
+    float dv[4];
+    int cv[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int k = k0 + m * kTileThreads, x = x0 + k % dw, y = y0 + k / dw;
+      dv[m] = 0.0f;
+      cv[m] = 1;
+      if (k < n_st && x >= 0 && x < a.W && y >= 0 && y < a.H) {
+        const long long p = (long long)y * a.W + x;
+        dv[m] = __ldg(dimg + p);
+        cv[m] = __ldg(cimg + p);
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int k = k0 + m * kTileThreads;
+      if (k < n_st) {
+        const float2 z = depth_pair(dv[m], cv[m]);
+        const int at = (k / dw) * dws + k % dw;
+        mine_valid = mine_valid && z.y != 0.0f;
+        zv[at] = z.x;
+        zw[at] = z.y;
+      }
+    }
+  }
+  const bool all_valid = __syncthreads_and(mine_valid);
+  // along the rows, then down the columns: a value is loaded once and added to every output whose
+  // window holds it; the weight sums only where a staged pixel is invalid
+  auto smooth = [&](auto all) {
+    constexpr bool kAll = decltype(all)::value;
+    constexpr int h_groups = (kSW + kHG - 1) / kHG, v_groups = (kSH + kVG - 1) / kVG;
+    for (int it = tid; it < dh * h_groups; it += kTileThreads) {
+      const int v = it % dh, u0 = (it / dh) * kHG;
+      float num[kHG], den[kHG];
+#pragma unroll
+      for (int j = 0; j < kHG; ++j) num[j] = den[j] = 0.0f;
+      const float *row = zv + v * dws + u0, *roww = zw + v * dws + u0;
+#pragma unroll
+      for (int t = 0; t < 2 * R + kHG; ++t) {
+        const bool in = u0 + t < dw;
+        const float z = in ? row[t] : 0.0f, zok = !kAll && in ? roww[t] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < kHG; ++j) {
+          const int d = t - j;
+          if (d >= 0 && d <= 2 * R) {
+            const float w = g[d < R ? R - d : d - R];
+            num[j] = fmaf(w, z, num[j]);
+            if (!kAll) den[j] = fmaf(w, zok, den[j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kHG; ++j)
+        if (u0 + j < kSW) {
+          hn[v * hs + u0 + j] = num[j];
+          if (!kAll) hd[v * hs + u0 + j] = den[j];
+        }
+    }
+    __syncthreads();
+    for (int it = tid; it < kSW * v_groups; it += kTileThreads) {
+      const int u = it % kSW, v0 = (it / kSW) * kVG;
+      float num[kVG], den[kVG];
+#pragma unroll
+      for (int j = 0; j < kVG; ++j) num[j] = den[j] = 0.0f;
+#pragma unroll
+      for (int t = 0; t < 2 * R + kVG; ++t) {
+        const bool in = v0 + t < dh;
+        const float hz = in ? hn[(v0 + t) * hs + u] : 0.0f, hw = !kAll && in ? hd[(v0 + t) * hs + u] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < kVG; ++j) {
+          const int d = t - j;
+          if (d >= 0 && d <= 2 * R) {
+            const float w = g[d < R ? R - d : d - R];
+            num[j] = fmaf(w, hz, num[j]);
+            if (!kAll) den[j] = fmaf(w, hw, den[j]);
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kVG; ++j) {
+        const int v = v0 + j;
+        if (v < kSH) {
+          const bool centre = kAll || zw[(v + R) * dws + (u + R)] != 0.0f;
+          sS[v * kSW + u] = centre ? num[j] / (kAll ? a.den_all : den[j]) : __builtin_nanf("");
+        }
+      }
+    }
+  };
+  if (all_valid) smooth(std::true_type{});
+  else smooth(std::false_type{});
+  __syncthreads();
+  for (int k = tid; k < kTW * kTH; k += kTileThreads) {
+    const int u = k % kTW + 1, v = k / kTW + 1, x = ox + u - 1, y = oy + v - 1;
+    if (x >= a.W || y >= a.H) continue;
+    const long long p = img * P + (long long)y * a.W + x;
+    const float *c = sS + v * kSW + u;
+    if (a.smoothed) a.smoothed[p] = *c;
+    if (a.blur) a.blur[p] = isnan(*c) ? a.depth[p] : *c;
+    if (!a.normals) continue;
+    const float3 n = eq2_normal(a, c[0], c[-1], c[1], c[-kSW], c[kSW]);
+    a.normals[3 * p] = n.x;
+    a.normals[3 * p + 1] = n.y;
+    a.normals[3 * p + 2] = n.z;
+  }
+}
+
+template <int R>
+cudaError_t launch_normals_r(const NormalArgs &a, int n, cudaStream_t s) {
+  // the larger radii need more than the default 48 KB (set on the current device)
+  if constexpr (R > 0) {
+    if ((long long)a.W * a.H * n < kTilePixels) {
+      const size_t sm = TileShape<R>::kBytes;
+      cudaError_t e = cudaFuncSetAttribute(k_depth_normals_tile<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e != cudaSuccess) return e;
+      const int tiles = ((a.W + kTW - 1) / kTW) * ((a.H + kTH - 1) / kTH);
+      k_depth_normals_tile<R><<<dim3(tiles, n), kTileThreads, sm, s>>>(a);
+      return cudaGetLastError();
+    }
+  }
   const size_t sm = sizeof(StripSmem<R>) * kWarpsN;
-  // radii above about 6 need more than the default 48 KB (set on the current device)
   cudaError_t e = cudaFuncSetAttribute(k_depth_normals<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   k_depth_normals<R><<<(unsigned)((a.n_warps + kWarpsN - 1) / kWarpsN), 32 * kWarpsN, sm, s>>>(a);
@@ -224,9 +411,9 @@ cudaError_t launch_normals_r(const NormalArgs &a, cudaStream_t s) {
 }
 
 template <int R>
-cudaError_t launch_normals(const NormalArgs &a, cudaStream_t s) {
-  if (a.r == R) return launch_normals_r<R>(a, s);
-  if constexpr (R < kMaxR) return launch_normals<R + 1>(a, s);
+cudaError_t launch_normals(const NormalArgs &a, int n, cudaStream_t s) {
+  if (a.r == R) return launch_normals_r<R>(a, n, s);
+  if constexpr (R < kMaxR) return launch_normals<R + 1>(a, n, s);
   return cudaErrorInvalidValue;
 }
 
@@ -298,6 +485,9 @@ rm_status run_normals(const rm_intrinsics *intr, int32_t n, const float *depth, 
     a.ify = metric ? 1.0f / intr->fy : 1.0f;
     for (int k = 0; k <= kMaxR; ++k)
       a.g[k] = sigma > 0.0f ? (float)std::exp(-(double)(k * k) / (2.0 * (double)sigma * sigma)) : 1.0f;
+    float row = 0.0f;
+    for (int d = 0; d <= 2 * a.r; ++d) row = std::fmaf(a.g[std::abs(d - a.r)], 1.0f, row);
+    for (int d = 0; d <= 2 * a.r; ++d) a.den_all = std::fmaf(a.g[std::abs(d - a.r)], row, a.den_all);
     // chunks of rows: as many warps as are resident at once, but no chunk shorter than the rows that
     // it reads besides its own (64 images of 640x480: 167 us with 2816 warps, 177 with 6336)
     a.strips = (a.W + kOut - 1) / kOut;
@@ -306,7 +496,7 @@ rm_status run_normals(const rm_intrinsics *intr, int32_t n, const float *depth, 
     a.rows = std::max((a.H + want - 1) / want, 2 * a.r + 2);
     a.chunks = (a.H + a.rows - 1) / a.rows;
     a.n_warps = per_row_of_chunks * a.chunks;
-    ck(launch_normals<0>(a, s));
+    ck(launch_normals<0>(a, n, s));
   }
   if (e == cudaSuccess && host_n) ck(cudaMemcpyAsync(normals, d_n, sizeof(float) * 3 * np, cudaMemcpyDeviceToHost, s));
   if (e == cudaSuccess && host_s) ck(cudaMemcpyAsync(smoothed, d_s, sizeof(float) * np, cudaMemcpyDeviceToHost, s));
