@@ -33,6 +33,11 @@
  *  - Pointers marked "host or device" may point to either; the library finds out with
  *    cudaPointerGetAttributes. Host outputs make the call wait for the stream.
  *
+ * Memory: a map keeps its scratch (one allocation, as large as its largest call needed: bins,
+ * per-pose arrays and, for each pose or problem evaluated at once, 8 bytes a pixel of z-buffer)
+ * until it is destroyed. Calls that stage host arrays or take scratch outside a map keep up to
+ * 256 MB a device between calls, given back when a map on it is destroyed.
+ *
  * Errors: every entry point returns an rm_status. Nothing crosses the ABI as an exception and
  * no kernel traps: device-side problems (a full bin, a wait that ran out) are recorded in a
  * status word that the call reads back. rm_last_error() gives a message for the calling

@@ -512,7 +512,7 @@ rm_status leave_queued(rm_map *m, cudaStream_t s) {
 rm_status read_status(rm_map *m, cudaStream_t s, unsigned *out) {
   RM_CK(cudaStreamSynchronize(s));
   if (m->queued) {  // still queued only if on another stream than s, with no call on the map since
-    m->queued = cudaEventQuery(m->ev_queued) == cudaErrorNotReady;
+    m->queued = cudaEventQuery(m->ev_queued) != cudaSuccess;
     cudaGetLastError();
   }
   volatile unsigned *h = m->status;

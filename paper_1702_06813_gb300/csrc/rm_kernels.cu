@@ -1076,7 +1076,7 @@ __device__ __forceinline__ void setup_ray_table(const WaveArgs &a, int q, RaySet
       const int k = k0 + lane;
       bool live = k < info.w, slow = false;
       uchar4 t = make_uchar4(0, 0, 0, 0);
-      unsigned hi = 0, lo = 0;  // the triangle's rectangle, as QuickRect::bounds
+      unsigned hi = 0, lo = 0;  // the triangle's rectangle, as QuickRect::hi and lo
       if (live) {
         t = a.cl_tris[info.y + k];
         const float2 p0 = uv[t.x], p1 = uv[t.y], p2 = uv[t.z];

@@ -243,7 +243,7 @@ bool is_device_pointer(const void *p);
 // the library's own: a call that waits for its stream would otherwise hand the default pool's
 // memory back to the system and pay for it again (300 us for a few megabytes). The pool keeps at
 // most kScratchKept bytes a device between calls (the vertex gradient of 16 poses of 640x480 takes
-// 157 MB) and gives them back when a map is destroyed.
+// 79 MB) and gives them back when a map is destroyed.
 cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t s);
 constexpr uint64_t kScratchKept = 256ull << 20;
 // The device the map's arrays live on (the device current at rm_map_create).
