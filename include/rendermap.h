@@ -496,8 +496,9 @@ rm_status rm_cost_grad_noalloc(const rm_map *map, const rm_scan *scan, const dou
                                const rm_cost_params *params, const rm_cost_out *out,
                                void *stream);
 
-/* Reads and clears the map's device status word after work queued with async_status = 1;
- * returns RM_OK, RM_EOVERFLOW or RM_ETIMEOUT. */
+/* Reads and clears the map's device status word after work queued with async_status = 1; waits for
+ * `stream` and for the map's last queued call, whatever its stream (not for a graph's launches on
+ * other streams). Returns RM_OK, RM_EOVERFLOW or RM_ETIMEOUT. */
 rm_status rm_status_sync(rm_map *map, void *stream);
 
 /* Message for the calling thread's last non-RM_OK status ("" if none). */

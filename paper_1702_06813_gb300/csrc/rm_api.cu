@@ -506,15 +506,13 @@ rm_status leave_queued(rm_map *m, cudaStream_t s) {
   return RM_OK;
 }
 
-// Waits for the stream, then reads and clears the status word: it is in pinned host memory, which the
+// Waits for the stream and for a queued call, then reads and clears the status word: it is in pinned host memory, which the
 // kernels write only when something went wrong (a copy back and a memset on every call cost a
 // single-pose evaluation 12 us of 96).
 rm_status read_status(rm_map *m, cudaStream_t s, unsigned *out) {
   RM_CK(cudaStreamSynchronize(s));
-  if (m->queued) {  // still queued only if on another stream than s, with no call on the map since
-    m->queued = cudaEventQuery(m->ev_queued) != cudaSuccess;
-    cudaGetLastError();
-  }
+  if (m->queued) RM_CK(cudaEventSynchronize(m->ev_queued));  // on another stream than s, if it still runs
+  m->queued = false;
   volatile unsigned *h = m->status;
   *out = *h;
   *h = 0;

@@ -84,3 +84,19 @@ def test_captured_call_between_others(scene):
         _same(got, want, sel)
     _finish(gm)
     gm.close()
+
+
+def test_status_waits_for_a_call_on_another_stream(scene):
+    mesh, scan, poses, want = scene
+    gm = rm.Map(mesh.vertices, mesh.faces, mesh.labels)
+    rm.cost_grad(gm, scan, poses)  # sizes the scratch
+    gm.set_tuning(async_status=True)
+    s = torch.cuda.Stream()
+    for turn in range(3):
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(20_000_000)  # about 10 ms
+            got = rm.cost_grad(gm, scan, poses)
+        _finish(gm)
+        assert s.query()
+        _same(got, want, slice(None))
+    gm.close()
