@@ -1503,6 +1503,7 @@ rm_status rm_map_set_vertex_normals(rm_map *m, const float *normals, const doubl
   std::lock_guard<std::mutex> lk(m->mu);
   RM_CK(cudaSetDevice(m->device));
   cudaStream_t s = (cudaStream_t)stream;
+  if (m->queued) RM_CK(cudaStreamWaitEvent(s, m->ev_queued, 0));  // it may read the normals that this call replaces
   if (!normals) {
     if (m->d_vn) {
       RM_CK(cudaStreamSynchronize(s));

@@ -100,3 +100,25 @@ def test_status_waits_for_a_call_on_another_stream(scene):
         assert s.query()
         _same(got, want, slice(None))
     gm.close()
+
+
+def test_normals_replaced_while_a_call_is_queued(scene):
+    mesh, scan, poses, _ = scene
+    n = np.random.Generator(np.random.PCG64(3)).normal(size=(2, len(mesh.vertices), 3)).astype(np.float32)
+    normals = torch.as_tensor(n).cuda()
+    gm = rm.Map(mesh.vertices, mesh.faces, mesh.labels)
+    want = []
+    for k in range(2):
+        gm.set_vertex_normals(normals[k])
+        want.append(rm.icp_terms(gm, scan, poses, tol=0.1))
+    gm.set_tuning(async_status=True)
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for turn in range(3):  # the map's normals are those of turn - 1 (1 at first)
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(4_000_000)
+            got = rm.icp_terms(gm, scan, poses, tol=0.1)
+        gm.set_vertex_normals(normals[turn % 2])
+        _finish(gm)
+        _same(got, want[(turn + 1) % 2], slice(None))
+    gm.close()
